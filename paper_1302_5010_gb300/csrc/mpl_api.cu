@@ -81,6 +81,7 @@ struct mpl_ctx {
     float* pm1 = nullptr;   // Adam moments
     float* pm2 = nullptr;
     float* pgrad = nullptr; // gradient accumulator
+    float* ppart = nullptr; // partial gradients of a training pass (TRAIN_MAX_ROWS rows)
     float* pacc = nullptr;  // [0] loss sum, [1] (int) live examples
     float* rn = nullptr;    // ||A^T a_j|| estimates (m)
     bool prop_ready = false, rn_ready = false;
@@ -459,7 +460,7 @@ void mpl_destroy(mpl_handle_t h) {
     cudaFree(h->Bst);
     cudaFree(h->lamst);
     cudaFree(h->Xst);
-    for (float* q : {h->pw, h->pwb, h->pm1, h->pm2, h->pgrad, h->pacc, h->rn}) cudaFree(q);
+    for (float* q : {h->pw, h->pwb, h->pm1, h->pm2, h->pgrad, h->ppart, h->pacc, h->rn}) cudaFree(q);
     if (h->cnt_h) cudaFreeHost(h->cnt_h);
     if (h->fin_h) cudaFreeHost(h->fin_h);
     clear_graphs(h);
@@ -1142,6 +1143,8 @@ static cudaError_t prop_alloc(mpl_ctx* h) {
     }
     cudaError_t e = cudaMalloc(&h->pacc, 4 * sizeof(float));
     if (e != cudaSuccess) return e;
+    e = cudaMalloc(&h->ppart, (size_t)TRAIN_MAX_ROWS * PROP_NPARAM * sizeof(float));
+    if (e != cudaSuccess) return e;
     return cudaMalloc(&h->rn, (size_t)h->m * sizeof(float));
 }
 
@@ -1296,33 +1299,58 @@ mpl_status_t mpl_proposal_train(mpl_handle_t h, const float* B, int p, const flo
     CK(cudaMemcpy(h->pw, w.data(), PROP_NPARAM * sizeof(float), cudaMemcpyHostToDevice));
     CK(cudaMemset(h->pm1, 0, PROP_NPARAM * sizeof(float)));
     CK(cudaMemset(h->pm2, 0, PROP_NPARAM * sizeof(float)));
-    CK(cudaMemset(h->pgrad, 0, PROP_NPARAM * sizeof(float)));
-    int* perm = nullptr;
-    CK(cudaMalloc(&perm, live.size() * sizeof(int)));
+    const int nlive = (int)live.size();
+    // the epochs run back to back: while one trains, the host shuffles the next one's order
+    // (two orders in turn, each rewritten only after its copy), and the losses come back at
+    // the end
+    struct Scratch {
+        int* perm[2] = {nullptr, nullptr};
+        float* acc = nullptr;
+        cudaEvent_t copied[2] = {nullptr, nullptr};
+        ~Scratch() {
+            for (int* q : perm) cudaFree(q);
+            cudaFree(acc);
+            for (cudaEvent_t q : copied)
+                if (q) cudaEventDestroy(q);
+        }
+    } t;
+    for (int q = 0; q < 2; ++q) {
+        CK(cudaMalloc(&t.perm[q], live.size() * sizeof(int)));
+        CK(cudaEventCreateWithFlags(&t.copied[q], cudaEventDisableTiming));
+    }
+    std::vector<float> acc(2 * (size_t)std::max(epochs, 1), 0.f);  // loss sum, live examples per epoch
+    CK(cudaMalloc(&t.acc, acc.size() * sizeof(float)));
+    CK(cudaMemsetAsync(t.acc, 0, acc.size() * sizeof(float), st));
+    std::vector<int> order[2] = {live, {}};
     int64_t nl = 0;
     int step = 0;
-    const int nlive = (int)live.size();
-    for (int ep = 0; ep < epochs; ++ep) {
-        std::shuffle(live.begin(), live.end(), rng);
-        CK(cudaMemcpyAsync(perm, live.data(), live.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-        CK(cudaMemsetAsync(h->pacc, 0, 4 * sizeof(float), st));
-        for (int off = 0; off < nlive; off += batch) {
+    mpl_status_t rc = MPL_OK;
+    for (int ep = 0; ep < epochs && rc == MPL_OK; ++ep) {
+        const int q = ep & 1;
+        cudaError_t e = ep > 1 ? cudaEventSynchronize(t.copied[q]) : cudaSuccess;
+        if (ep > 0) order[q] = order[q ^ 1];
+        std::shuffle(order[q].begin(), order[q].end(), rng);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(t.perm[q], order[q].data(), live.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaEventRecord(t.copied[q], st);
+        for (int off = 0; off < nlive && e == cudaSuccess; off += batch) {
             const int cnt = std::min(batch, nlive - off);
-            CK(launch_train_step(h->pw, exd, perm, off, cnt, 1.f / (float)cnt, h->pgrad, h->pacc,
-                                 reinterpret_cast<int*>(h->pacc + 1), st, &nl));
-            CK(launch_adam(h->pw, h->pgrad, h->pm1, h->pm2, (float)lr, ++step, st, &nl));
+            e = launch_train_step(h->pw, exd, t.perm[q], off, cnt, 1.f / (float)cnt, h->ppart, h->pm1, h->pm2,
+                                  (float)lr, ++step, t.acc + 2 * ep, reinterpret_cast<int*>(t.acc + 2 * ep + 1), st, &nl);
         }
-        float acc[2];
-        CK(cudaMemcpyAsync(acc, h->pacc, 2 * sizeof(float), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        int cntl;
-        std::memcpy(&cntl, &acc[1], sizeof(int));
-        if (loss_out) loss_out[ep] = cntl > 0 ? acc[0] / (float)cntl : 0.f;
+        rc = from_cuda(e);
     }
-    CK(launch_round_bf16(h->pw, h->pwb, st, &nl));
-    CK(cudaStreamSynchronize(st));
-    cudaFree(perm);
+    if (rc == MPL_OK) rc = from_cuda(launch_round_bf16(h->pw, h->pwb, st, &nl));
+    const cudaError_t es = cudaStreamSynchronize(st);  // (the orders and the scratch outlive the copies)
     cudaFree(exd);
+    if (rc != MPL_OK) return rc;
+    CK(es);
+    CK(cudaMemcpy(acc.data(), t.acc, acc.size() * sizeof(float), cudaMemcpyDeviceToHost));
+    for (int ep = 0; ep < epochs && loss_out; ++ep) {
+        int cntl;
+        std::memcpy(&cntl, &acc[2 * (size_t)ep + 1], sizeof(int));
+        loss_out[ep] = cntl > 0 ? acc[2 * (size_t)ep] / (float)cntl : 0.f;
+    }
     h->prop_ready = true;
     clear_graphs(h);
     return MPL_OK;
@@ -1348,7 +1376,7 @@ mpl_status_t mpl_proposal_loss_grad(mpl_handle_t h, const float* B, int p, const
     CK(cudaMemsetAsync(h->pacc, 0, 4 * sizeof(float), st));
     int64_t nl = 0;
     const int nlive = (int)live.size();
-    CK(launch_train_step(h->pw, exd, perm, 0, nlive, nlive > 0 ? 1.f / (float)nlive : 0.f, h->pgrad, h->pacc,
+    CK(launch_train_grad(h->pw, exd, perm, nlive, nlive > 0 ? 1.f / (float)nlive : 0.f, h->ppart, h->pgrad, h->pacc,
                          reinterpret_cast<int*>(h->pacc + 1), st, &nl));
     float acc[2];
     CK(cudaMemcpyAsync(acc, h->pacc, 2 * sizeof(float), cudaMemcpyDeviceToHost, st));

@@ -265,9 +265,15 @@ cudaError_t launch_max_reduce(const float* v, int len, float* out, cudaStream_t 
 // Proposal network support (proposal.cu).
 cudaError_t launch_sketch_rownorm(const float* A32, int n, int m, int T, float* Z, cudaStream_t s, int64_t* nl);
 cudaError_t launch_rownorm(const float* C, int m, int T, float* rn, cudaStream_t s, int64_t* nl);
-cudaError_t launch_train_step(const float* w, const float* ex, const int* perm, int off, int count, float inv_batch,
-                              float* grad, float* loss_acc, int* n_acc, cudaStream_t s, int64_t* nl);
-cudaError_t launch_adam(float* w, float* grad, float* m1, float* m2, float lr, int step, cudaStream_t s, int64_t* nl);
+// One pass of the training over `count` examples writes its partial gradients to part
+// (TRAIN_MAX_ROWS x PROP_NPARAM floats); loss_acc and n_acc take the loss sum and the live
+// examples.  _grad adds the summed gradient to grad, _step takes an Adam step (1-based) on w.
+constexpr int TRAIN_MAX_ROWS = 304;  // two CTAs per SM of 152
+cudaError_t launch_train_grad(const float* w, const float* ex, const int* perm, int count, float inv_batch,
+                              float* part, float* grad, float* loss_acc, int* n_acc, cudaStream_t s, int64_t* nl);
+cudaError_t launch_train_step(float* w, const float* ex, const int* perm, int off, int count, float inv_batch,
+                              float* part, float* m1, float* m2, float lr, int step, float* loss_acc, int* n_acc,
+                              cudaStream_t s, int64_t* nl);
 cudaError_t launch_round_bf16(const float* w, float* wb, cudaStream_t s, int64_t* nl);
 
 // One-time kernel attribute set-up (call before any stream capture).

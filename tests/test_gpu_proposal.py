@@ -114,3 +114,30 @@ def test_warm_start_plain_and_mixed_identical():
     np.testing.assert_array_equal(out[0][1], out[1][1])
     s0.close()
     s1.close()
+
+
+@pytest.mark.parametrize("p,candidates", [(1, 1), (3, 5), (2, 8), (3, 17), (7, 16), (80, 64)])
+def test_gradient_is_the_mean_over_signals(p, candidates):
+    """The training pass works on groups of 16 examples, at most 304 groups at a time: ragged and
+    full groups, and more examples (5120) than one sweep of the groups takes.  The loss and the
+    gradient are means over the examples, so those of a batch are the mean of its signals' (each
+    has the same number of candidates).  Tolerance: a sum of the pass has at most 16 * 2 terms in
+    a chain, then 304 / 8 + 8 in the reduction, so it is off by less than 80 * 2^-24 = 4.8e-6 of
+    the sum of its terms' magnitudes, and the chain through both layers (64 terms each) by
+    about as much again; every norm below is at least the gradient's."""
+    torch = _torch()
+    P = synth.small_problem(256, 2048, 80, 8, 24, rho=6, seed=33)
+    s, _ = _trained(P, epochs=1, candidates=candidates)
+    Xref = _reference(P)
+    B, lam = torch.from_numpy(P.B).cuda(), torch.from_numpy(P.lam).cuda()
+    loss, g = mpl.mpl_proposal_loss_grad(s.h, B[:p], p, lam[:p], Xref[:p])
+    losses, grads, norms = [], [], []
+    for i in range(p):
+        li, gi = mpl.mpl_proposal_loss_grad(s.h, B[i:i + 1], 1, lam[i:i + 1], Xref[i:i + 1])
+        losses.append(li)
+        grads.append(gi.astype(np.float64))
+        norms.append(np.linalg.norm(gi))
+    s.close()
+    assert abs(loss - np.mean(losses)) <= 2e-5 * np.mean(losses)
+    assert np.linalg.norm(g - np.mean(grads, axis=0)) <= 2e-5 * np.mean(norms)
+    assert np.any(g[6:] != 0) and np.all(g[:6] == 0)
