@@ -249,7 +249,7 @@ cudaError_t build_gram_q(const float* A32, int n, int m, float* Q, int* act, Cou
     d.Cs = Q;
     d.act[0] = act;
     d.cnt = cnt;
-    return launch_corr_f32(d, 0, m, s, nl);
+    return launch_corr_chain(d, 0, m, s, nl);
 }
 
 }  // namespace mpl

@@ -1,0 +1,454 @@
+// Worst-case analysis of Algorithm 1 in FP32 on the 5th-generation tensor cores: C = A^T R with
+// every FP32 operand split into two TF32 parts.
+//
+//   x = hi + lo,  hi = x rounded to TF32's 11 significant bits, lo = x - hi rounded to them too:
+//   |x - hi - lo| <= 2^-23 |x|.  a r is taken as a_hi r_lo + a_lo r_hi + a_hi r_hi (the
+//   dropped a_lo r_lo is at most 2^-22 |a r|, of either sign).
+//
+// The sums of 32 products along n are accumulated in TMEM (the small products first, then the
+// large ones) and added to FP32 registers with round-to-nearest, so that the tensor core's
+// truncating accumulation acts over 32 products only and the sequential FP32 chain is n / 32
+// long instead of n.
+//
+// A persistent CTA walks output tiles of 128 atoms x w signals.  Roles (five warpgroups):
+//   warps 0-7   loaders: rows of atoms and of the active signals' residuals (gathered through the
+//               active list) are copied asynchronously, as FP32, to where their hi part goes in
+//               one of two stages (128-byte-swizzled tiles); each lane then splits the 16 bytes it
+//               copied, so that no thread waits for another's copies.
+//   warp 8      allocates TMEM; one thread issues the 12 tcgen05.mma of a stage (kind::tf32,
+//               M = 128, N = w, K = 8) into the stage's accumulator and commits.
+//   warps 12-19 accumulate: tcgen05.ld of the finished stage's accumulator, added to registers
+//               (each warp its 32 atoms and half of the tile's signals); scores stored at the end.
+// setmaxnreg moves registers from the loaders to the accumulating warps.
+//
+// What bounds it: the loaders' instructions.  A stage of a 128 x 256 tile takes 3500 cycles, of
+// which the tensor core works 2100 and shared memory (three reads of every operand by
+// the MMAs, the copies and the split: 340 KB) at least 2650.  2044 x 32771 x 500: 480 us
+// (140 TFLOP/s), 4096 x 65536 x 1024: 3.13 ms, 1024 x 8192 x 256: 51 us; the FP32 chain on the SIMT
+// cores takes 1596 us, 12.2 ms and 162 us.  Loads staged in registers (592 us), six loader warps
+// (507 us) and more, shorter stages with the copies issued ahead (557 to 650 us) were slower.
+// Error against FP64 (2-norm, Gaussian data): 1.3e-7 at n = 128, 2.4e-7 at n = 4096, the chain's
+// 2.0e-7 and 1.15e-6.
+//
+// Inputs at or near overflow (infinities, NaN, |x| >= 2^128 (1 - 2^-12)) have no split: their rows
+// are flagged and the affected scores recomputed with one FP32 FMA chain over n, so that a
+// score is infinite or NaN where the FP32 product is.
+//
+// Every wait is bounded; on expiry the CTA records DERR_TIMEOUT, the MMA thread waits (bounded) for
+// the MMAs it issued, and the CTA frees its TMEM and returns.
+#include "mpl_internal.cuh"
+#include "tc_ptx.cuh"
+
+namespace mpl {
+
+namespace {
+
+constexpr int TF_BM = 128;           // atoms per tile
+constexpr int TF_BN = 256;           // most signals per tile
+constexpr int TF_BK = 32;            // columns of n per stage: one 128-byte swizzle row
+constexpr int TF_STAGES = 2;         // stages, each with its TMEM accumulator
+constexpr int TF_THREADS = 640;
+constexpr int TF_LOADERS = 8;        // loader warps
+constexpr int TF_MMA_WARP = 8;
+constexpr int TF_ITEMS = 12;         // most 4-row items per loader warp and stage: (128 + 256) / 4 / 8
+constexpr int TF_STEP = 4 * TF_LOADERS;  // rows from one item of a warp to its next (a multiple of 8)
+constexpr int TF_ACC_WARPS = 8;
+constexpr int TF_REGS_ACC = 152, TF_REGS_LOAD = 56;  // per thread after setmaxnreg
+constexpr int TF_SLOTS = 8;          // flag slots by tile (the loaders run at most 4 tiles ahead)
+constexpr int TF_ROWS = TF_BM + TF_BN;
+
+constexpr int TF_A_BYTES = TF_BM * 128;
+constexpr int TF_HALF_BYTES = TF_ROWS * 128;          // the hi (or lo) tiles: atoms, then signals
+constexpr int TF_STAGE_BYTES = 2 * TF_HALF_BYTES;
+
+struct TfShared {
+    uint64_t full[TF_STAGES];    // the loaders have filled the stage
+    uint64_t done[TF_STAGES];    // its MMAs are complete: stage free, accumulator ready
+    uint64_t tempty[TF_STAGES];  // its accumulator has been read
+    uint64_t drain;
+    uint32_t tmem;
+    int abort_flag;
+    const float* row[TF_ROWS];                   // the tile's rows (atoms, signals), null past the end
+    unsigned char inf[TF_SLOTS][TF_ROWS];        // the row holds a value without a split
+    unsigned char nan[TF_SLOTS][TF_ROWS];        // ... a NaN
+    unsigned char any[TF_SLOTS][8];              // any such row, by loader warp
+};
+constexpr size_t TF_SMEM = (size_t)TF_STAGES * TF_STAGE_BYTES + 1024 + sizeof(TfShared);
+static_assert(TF_SMEM <= 227 * 1024, "two stages and the barriers fit one CTA's shared memory");
+static_assert(TF_ITEMS * TF_STEP == TF_ROWS && TF_STEP % 8 == 0, "every row has one loader");
+
+// Instruction descriptor, kind::tf32: D f32, A/B tf32, both K-major, M x N.
+__device__ __forceinline__ uint32_t idesc_tf32(int M, int N) {
+    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc));
+}
+
+// Asynchronous copies of four consecutive entries to shared memory, zero past the first `left`.
+__device__ __forceinline__ void copy4_16(uint32_t dst, const float* src, int left) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(left > 0 ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void copy4_4(uint32_t dst, const float* src, int left) {  // rows of any alignment
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 4 * e), "l"(left > e ? src + e : src),
+                     "r"(left > e ? 4 : 0)
+                     : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+__device__ __forceinline__ float4 ld_shared4(uint32_t src) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(src) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_shared4(uint32_t dst, const uint32_t (&v)[4]) {
+    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3])
+                 : "memory");
+}
+
+// Signals per tile (a multiple of 16, at most TF_BN): the count of active signals shrinks from one
+// outer iteration to the next, and a narrower tile costs less.  A stage takes about 576 + w units
+// (2700 cycles measured at w = 64, 3000 at 128, 3500 at 256), and ceil(tiles / grid) tiles run
+// in turn on a CTA.
+__device__ __forceinline__ int pick_width(int act_n, int tiles_m, int grid) {
+    const int t0 = (act_n + TF_BN - 1) / TF_BN;
+    int best = TF_BN;
+    float cost = 3e38f;
+    for (int t = t0; t < t0 + 8; ++t) {
+        const int w = (((act_n + t - 1) / t) + 15) / 16 * 16;
+        const float tiles = (float)tiles_m * (float)((act_n + w - 1) / w);
+        const float c = ceilf(tiles / (float)grid) * (float)(576 + w);
+        if (c < cost) { cost = c; best = w; }
+    }
+    return best;
+}
+
+constexpr uint32_t TF_NOSPLIT = 0x7f7ff000u;  // |x| bits from here on: rounding x to TF32 is not finite
+
+__device__ __forceinline__ uint32_t tf32_hi(uint32_t x) { return (x + 0x1000u) & 0xffffe000u; }
+
+// Four entries of which some may have no split: those keep their upper bits (a NaN stays one) and
+// flag the row.
+__device__ __noinline__ void store_nosplit(float4 v, uint32_t dst, unsigned char* inf, unsigned char* nan) {
+    const float f[4] = {v.x, v.y, v.z, v.w};
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const uint32_t x = __float_as_uint(f[e]);
+        const uint32_t a = x & 0x7fffffffu;
+        hi[e] = tf32_hi(x);
+        lo[e] = __float_as_uint(__uint_as_float(x) - __uint_as_float(hi[e])) + 0x1000u;
+        if (a >= TF_NOSPLIT) { hi[e] = x & 0xffffe000u; lo[e] = 0u; *inf = 1; }
+        if (a > 0x7f800000u) { hi[e] = 0x7fc00000u; *nan = 1; }
+    }
+    st_shared4(dst, hi);
+    st_shared4(dst + TF_HALF_BYTES, lo);
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
+    pdl_enter();
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    TfShared& sh = *reinterpret_cast<TfShared*>(base + TF_STAGES * TF_STAGE_BYTES);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int act_n = d.cnt->act_n[cur];
+    const int m = d.m, n = d.n;
+    const int tiles_m = (m + TF_BM - 1) / TF_BM;
+    if (act_n <= 0) return;
+    const int w = pick_width(act_n, tiles_m, (int)gridDim.x);
+    const int tiles_n = (act_n + w - 1) / w;
+    const long long ntiles = (long long)tiles_m * tiles_n;
+    if ((long long)blockIdx.x >= ntiles) return;  // (the whole CTA, before it holds anything)
+    const int nk = (n + TF_BK - 1) / TF_BK;
+    volatile int* abort_flag = &sh.abort_flag;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < TF_STAGES; ++s) {
+            mbar_init(&sh.full[s], TF_LOADERS);
+            mbar_init(&sh.done[s], 1);
+            mbar_init(&sh.tempty[s], TF_ACC_WARPS);
+        }
+        mbar_init(&sh.drain, 1);
+        sh.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == TF_MMA_WARP) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem)),
+                     "r"(TF_STAGES * TF_BN));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = sh.tmem;
+
+    auto give_up = [&]() {
+        *abort_flag = 1;
+        atomicCAS(&d.cnt->err, 0, (int)DERR_TIMEOUT);
+    };
+
+    if (warp < 12) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TF_REGS_LOAD));
+        if (warp < TF_LOADERS) {
+            // item i of this warp: rows 4 warp + TF_STEP i .. + 3 of [atoms | signals], eight lanes
+            // (16 bytes each) per row; in groups of four items, of which a narrow tile takes fewer
+            const int r0 = warp * 4 + (lane >> 3), kc = (lane & 7) * 4;
+            const int rows = TF_BM + w;
+            const uint32_t dst0 = smem_u32(base) + (uint32_t)(r0 * 128 + (((lane & 7) ^ (r0 & 7)) << 4));
+            int stage = 0;
+            uint32_t ph = 0;
+            unsigned tcount = 0;
+            bool ok = true;
+            for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tcount) {
+                const int tm = (int)(t / tiles_n), tn = (int)(t - (long long)tm * tiles_n);
+                const int slot = tcount & (TF_SLOTS - 1);
+                __syncwarp();
+                if ((lane & 7) == 0) {
+#pragma unroll 1
+                    for (int r = r0; r < TF_ROWS; r += TF_STEP) {
+                        const int j = tm * TF_BM + r, k = tn * w + r - TF_BM;
+                        const float* row = nullptr;
+                        if (r < TF_BM) {
+                            if (j < m) row = d.A32 + (size_t)j * n;
+                        } else if (r < rows && k < act_n) {
+                            row = d.R32 + (size_t)d.act[cur][k] * n;
+                        }
+                        sh.row[r] = row;
+                        sh.inf[slot][r] = 0;
+                        sh.nan[slot][r] = 0;
+                    }
+                }
+                if (lane == 0) sh.any[slot][warp] = 0;
+                __syncwarp();
+                for (int kb = 0; kb < nk; ++kb) {
+                    ok = mbar_wait(&sh.done[stage], ph ^ 1u, abort_flag);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) { if (lane == 0) give_up(); break; }
+                    // copied as FP32 to where hi goes: each lane splits the 16 bytes it copied, so
+                    // its own copies are all it waits for
+                    const uint32_t dst = dst0 + (uint32_t)(stage * TF_STAGE_BYTES);
+                    const int k = kb * TF_BK + kc;
+#pragma unroll
+                    for (int g = 0; g < TF_ITEMS / 4; ++g) {
+                        if (4 * warp + 4 * g * TF_STEP < rows) {  // (the same in all lanes)
+                            const float* row[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) row[i] = sh.row[r0 + (4 * g + i) * TF_STEP];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const uint32_t q = dst + (uint32_t)((4 * g + i) * TF_STEP * 128);
+                                // (zeros past the end: a row repeated there instead would be one
+                                // hot line for every CTA)
+                                const bool in = row[i] != nullptr && k < n;
+                                if (VEC) copy4_16(q, in ? row[i] + k : d.A32, in ? n - k : 0);
+                                else copy4_4(q, in ? row[i] + k : d.A32, in ? n - k : 0);
+                            }
+                        }
+                        copy_commit();
+                    }
+#pragma unroll
+                    for (int g = 0; g < TF_ITEMS / 4; ++g) {
+                        if (g == 0) copy_wait<2>();
+                        else if (g == 1) copy_wait<1>();
+                        else copy_wait<0>();
+                        if (4 * warp + 4 * g * TF_STEP >= rows) continue;
+                        float4 v[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) v[i] = ld_shared4(dst + (uint32_t)((4 * g + i) * TF_STEP * 128));
+                        float chk = 0.f;  // NaN once some lo is not finite
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float x[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+                            uint32_t hi[4], lo[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                hi[e] = tf32_hi(__float_as_uint(x[e]));
+                                const float l = x[e] - __uint_as_float(hi[e]);
+                                chk = fmaf(l, 0.f, chk);
+                                lo[e] = __float_as_uint(l) + 0x1000u;  // (the tensor core reads the upper bits)
+                            }
+                            st_shared4(dst + (uint32_t)((4 * g + i) * TF_STEP * 128), hi);
+                            st_shared4(dst + (uint32_t)((4 * g + i) * TF_STEP * 128 + TF_HALF_BYTES), lo);
+                        }
+                        if (chk != chk) {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const int r = r0 + (4 * g + i) * TF_STEP;
+                                store_nosplit(v[i], dst + (uint32_t)((4 * g + i) * TF_STEP * 128), &sh.inf[slot][r],
+                                              &sh.nan[slot][r]);
+                            }
+                            sh.any[slot][warp] = 1;
+                        }
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&sh.full[stage]);
+                    if (++stage == TF_STAGES) { stage = 0; ph ^= 1u; }
+                }
+            }
+        } else if (warp == TF_MMA_WARP && lane == 0) {
+            const uint32_t idesc = idesc_tf32(TF_BM, w);
+            int stage = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+                for (int kb = 0; kb < nk; ++kb) {
+                    if (!mbar_wait(&sh.tempty[stage], ph ^ 1u, abort_flag) ||
+                        !mbar_wait(&sh.full[stage], ph, abort_flag)) {
+                        give_up();
+                        ok = false;
+                        break;
+                    }
+                    // the loaders' writes, ordered before this by the barrier, become visible to the
+                    // tensor core here
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    fence_after();
+                    const uint8_t* sb = base + stage * TF_STAGE_BYTES;
+                    const uint64_t ah = sdesc_sw128(sb), bh = sdesc_sw128(sb + TF_A_BYTES);
+                    const uint64_t al = sdesc_sw128(sb + TF_HALF_BYTES);
+                    const uint64_t bl = sdesc_sw128(sb + TF_HALF_BYTES + TF_A_BYTES);
+                    const uint32_t dt = tmem + (uint32_t)(stage * TF_BN);
+#pragma unroll
+                    for (int k = 0; k < TF_BK / 8; ++k) {  // 8 columns of n: 32 bytes along the swizzle row
+                        const uint64_t off = (uint64_t)((k * 32) >> 4);
+                        mma_tf32(dt, ah + off, bl + off, idesc, k ? 1u : 0u);
+                        mma_tf32(dt, al + off, bh + off, idesc, 1u);
+                    }
+#pragma unroll
+                    for (int k = 0; k < TF_BK / 8; ++k) {
+                        const uint64_t off = (uint64_t)((k * 32) >> 4);
+                        mma_tf32(dt, ah + off, bh + off, idesc, 1u);
+                    }
+                    mma_commit(&sh.done[stage]);
+                    if (++stage == TF_STAGES) { stage = 0; ph ^= 1u; }
+                }
+            }
+            if (*abort_flag) {
+                // every MMA this thread issued completes before the accumulators are freed
+                mma_commit(&sh.drain);
+                mbar_wait_drain(&sh.drain, 0);
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(TF_REGS_ACC));
+        // lane quarter q of TMEM = 32 atoms of the tile; the two warpgroups take the tile's
+        // 16-signal blocks in turn
+        const int q = warp & 3, grp = (warp - 12) >> 2;
+        const int nblk = w / 16;
+        int stage = 0;
+        uint32_t ph = 0;
+        unsigned tcount = 0;
+        bool ok = true;
+        for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tcount) {
+            const int tm = (int)(t / tiles_n), tn = (int)(t - (long long)tm * tiles_n);
+            float acc[TF_BN / 32][16];
+#pragma unroll
+            for (int i = 0; i < TF_BN / 32; ++i)
+#pragma unroll
+                for (int e = 0; e < 16; ++e) acc[i][e] = 0.f;
+            for (int kb = 0; kb < nk; ++kb) {
+                ok = true;
+                if (lane == 0) ok = mbar_wait(&sh.done[stage], ph, abort_flag);
+                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                if (!ok) { if (lane == 0) give_up(); break; }
+                fence_after();
+                const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(stage * TF_BN);
+#pragma unroll
+                for (int i = 0; i < TF_BN / 32; ++i) {
+                    if (2 * i + grp < nblk) {
+                        float v[16];
+                        tmem_ld16(tb + (uint32_t)((2 * i + grp) * 16), v);
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) acc[i][e] += v[e];
+                    }
+                }
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sh.tempty[stage]);
+                if (++stage == TF_STAGES) { stage = 0; ph ^= 1u; }
+            }
+            if (!ok) break;
+            const int slot = tcount & (TF_SLOTS - 1);
+            const int ar = q * 32 + lane;
+            const int atom = tm * TF_BM + ar;
+            bool flagged = false;
+#pragma unroll
+            for (int l = 0; l < TF_LOADERS; ++l) flagged |= sh.any[slot][l] != 0;
+#pragma unroll
+            for (int i = 0; i < TF_BN / 32; ++i) {
+                if (2 * i + grp < nblk) {
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        const int col = (2 * i + grp) * 16 + e;
+                        const int k = tn * w + col;
+                        if (k < act_n && atom < m) d.Cs[(size_t)k * m + atom] = acc[i][e];
+                    }
+                }
+            }
+            if (flagged && atom < m) {
+                // scores with a value that has no split (and no NaN, whose products are NaN):
+                // one FP32 FMA chain over n
+#pragma unroll 1
+                for (int col = 0; col < w; ++col) {
+                    if (((col >> 4) & 1) != grp) continue;
+                    const int k = tn * w + col;
+                    if (k >= act_n || sh.nan[slot][ar] || sh.nan[slot][TF_BM + col]) continue;
+                    if (!sh.inf[slot][ar] && !sh.inf[slot][TF_BM + col]) continue;
+                    const float* a = d.A32 + (size_t)atom * n;
+                    const float* r = d.R32 + (size_t)d.act[cur][k] * n;
+                    float s = 0.f;
+#pragma unroll 1
+                    for (int x = 0; x < n; ++x) s = fmaf(__ldg(a + x), __ldg(r + x), s);
+                    d.Cs[(size_t)k * m + atom] = s;
+                }
+            }
+        }
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (warp == TF_MMA_WARP) {
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TF_STAGES * TF_BN));
+    }
+}
+
+// The registers that setmaxnreg hands out come from the launch's own: 5 x 128 threads at numRegs.
+bool regs_cover(const cudaFuncAttributes& a) { return 5 * a.numRegs >= 2 * TF_REGS_ACC + 3 * TF_REGS_LOAD; }
+
+template <bool VEC>
+cudaError_t launch_t(const Dev& d, int cur, int act_n_ub, cudaStream_t s) {
+    // (per launch: the attribute belongs to the current context; about a microsecond of host time)
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, k_corr_tf32<VEC>);
+    if (e != cudaSuccess) return e;
+    if (!regs_cover(fa)) return cudaErrorNotSupported;
+    e = cudaFuncSetAttribute(k_corr_tf32<VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TF_SMEM);
+    if (e != cudaSuccess) return e;
+    int dev = 0, sms = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    // one CTA per SM; tiles of 16 signals are the narrowest
+    const long long tiles = (long long)((d.m + TF_BM - 1) / TF_BM) * ((act_n_ub + 15) / 16);
+    const int grid = (int)(tiles < sms ? tiles : sms);
+    return launch_chain(k_corr_tf32<VEC>, dim3(grid), dim3(TF_THREADS), TF_SMEM, s, d, cur);
+}
+
+}  // namespace
+
+cudaError_t launch_corr_tf32(const Dev& d, int cur, int act_n_ub, cudaStream_t s, int64_t* nl) {
+    const cudaError_t e = (d.n & 3) == 0 ? launch_t<true>(d, cur, act_n_ub, s) : launch_t<false>(d, cur, act_n_ub, s);
+    if (e != cudaSuccess) return e;
+    ++*nl;
+    return cudaSuccess;
+}
+
+}  // namespace mpl

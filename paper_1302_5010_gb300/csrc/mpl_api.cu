@@ -296,21 +296,28 @@ void set_bounds(mpl_ctx* h, Dev& d) {
     const double gam = nu / (1.0 - nu);
     const double c32 = 2.0 * (gam + u);  // sequential FP32 dot vs exact, incl. rounding of r
     d.bound_c32 = (float)(c32 * 1.01);
-    d.bound_f32 = (float)(c32 * 1.01);
+    // the split TF32 correlation (corr_tf32.cu): the operands' splits (2^-23 each) and the dropped
+    // product of their low parts (2^-22), the tensor core's accumulation of 32 x 3 products
+    // (assumed to lose at most 2^-22 of the running magnitude per product, as for BF16), and
+    // the FP32 sum of the n / 32 groups; the wider of the two FP32 forms covers both kernels
+    const double tf = 1.25 * (98.0 * std::ldexp(1.0, -22) + ((double)h->n / 32.0 + 2.0) * u);
+    const double cf = std::max(c32, tf);
+    d.bound_f32 = (float)(cf * 1.01);
     // identity route: FP32 beta and Q entries (gamma_n each, relative to colmax ||b|| and
     // colmax^2 ||x||_1), the FP32 sum over at most smax terms, and the FP32 residual the
     // re-score reads (gamma_smax each)
     const int smax = h->smax > 0 ? h->smax : default_smax(h);
     const double su = (double)(smax + 1) * u;
     const double gs = su / (1.0 - su);
-    d.bound_q = (float)((gam + 2.0 * gs * (1.0 + gam) + u) * 1.01);
+    const double gb = std::max(gam, tf);  // beta comes from either FP32 kernel
+    d.bound_q = (float)((gb + 2.0 * gs * (1.0 + gb) + u) * 1.01);
     if (h->precision == 1) {
         // BF16 operands (relative 2^-8 each) with an FP32 accumulator assumed to
         // keep at least 22 bits per addition; plus the FP32 terms above.
         const double cb = 1.25 * (std::ldexp(1.0, -7) + std::ldexp(1.0, -16) + (double)h->n * std::ldexp(1.0, -22));
         d.bound_c = (float)(cb + c32);
     } else {
-        d.bound_c = (float)(c32 * 1.01);
+        d.bound_c = (float)(cf * 1.01);
     }
     // the measured form of the same bound: a^T r - bf(a)^T bf(r) = (a - bf(a))^T r +
     // bf(a)^T (r - bf(r)) exactly, each term bounded by Cauchy-Schwarz, plus the
