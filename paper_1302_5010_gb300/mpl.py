@@ -127,7 +127,7 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
     lib.mpl_set_option.restype = i32
     lib.mpl_get_option.argtypes = [vp, i32, ctypes.POINTER(f64)]
     lib.mpl_get_option.restype = i32
-    lib.mpl_get_stats.argtypes = [vp, i32, ctypes.POINTER(SignalStats)]
+    lib.mpl_get_stats.argtypes = [vp, i32, vp]
     lib.mpl_get_stats.restype = i32
     lib.mpl_get_solution_f64.argtypes = [vp, i32, vp]
     lib.mpl_get_solution_f64.restype = i32
@@ -259,12 +259,23 @@ def mpl_proposal_loss_grad(h, B, p: int, lam, Xref):
     return loss.value, g
 
 
+# the statistics record as numpy sees it (the layout of SignalStats)
+_STATS_DTYPE = np.dtype([(f, np.int32 if t is ctypes.c_int32 else np.float64) for f, t in SignalStats._fields_],
+                        align=True)
+assert _STATS_DTYPE.itemsize == ctypes.sizeof(SignalStats)
+_STATS_COLUMNS = [(f, np.int64 if t is ctypes.c_int32 else np.float64) for f, t in SignalStats._fields_]
+
+
 def mpl_get_stats(h, p: int) -> dict:
-    arr = (SignalStats * max(p, 1))()
-    rc = load().mpl_get_stats(h, int(p), arr)
+    # one copy into a record array, then a column per field (a Python object per signal and
+    # field took 0.3 ms for 256 signals and 2.1 ms for 2048, a quarter of a small solve)
+    arr = np.empty(max(p, 1), dtype=_STATS_DTYPE)
+    rc = load().mpl_get_stats(h, int(p), arr.ctypes.data)
     if rc != MPL_OK:
         raise MplError(rc, "mpl_get_stats")
-    return {f: np.array([getattr(arr[i], f) for i in range(p)]) for f, _ in SignalStats._fields_}
+    if p <= 0:
+        return {f: np.array([]) for f in _STATS_DTYPE.names}
+    return {f: arr[f].astype(t) for f, t in _STATS_COLUMNS}
 
 
 def mpl_get_solution_f64(h, p: int, X64) -> None:
