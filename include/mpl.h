@@ -60,7 +60,10 @@ typedef enum {
     MPL_OPT_INNER_MAX = 5,  /* s_max, PG iterations per master problem.  default 400 */
     MPL_OPT_WARM_START = 6, /* 0: x^0 = 0 (Alg. 1);
                                2: proposal network seeds the active sets.  default 0 */
-    MPL_OPT_SYNC_EVERY = 7, /* outer iterations launched per host/device handshake. default 2 */
+    MPL_OPT_SYNC_EVERY = 7, /* outer iterations launched per host/device handshake, 1..64.  Accepted
+                               and kept, without effect: every iteration's selection writes the
+                               work-list lengths to mapped host memory, and the host reads them
+                               while the iteration still runs.  default 2 */
     MPL_OPT_PROFILE = 8,    /* 1: record per-phase device times (mpl_get_phase_times) with
                                timing events, inside the captured graphs too. default 0 */
     MPL_OPT_GRAPH = 9,      /* 1: each outer iteration is replayed from a captured CUDA graph

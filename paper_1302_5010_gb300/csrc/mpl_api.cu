@@ -8,11 +8,12 @@
 //   finish       FP64 exact finish / certificate  (k_finish, signals w/o violators)
 //   master       accelerated PG on the Gram block (k_apg, persistent work queue)
 //   residual     R = B - A_S X_S                  (k_residual)
-// followed by one 40-byte device-to-host read of the work counters.
+// The host learns the lengths of the work lists from mapped memory that the selection writes.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <numeric>
 #include <random>
@@ -57,13 +58,12 @@ struct mpl_ctx {
     cudaStream_t side2 = nullptr; // master problems with blocks outside shared memory, beside the others
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     cudaEvent_t ev_fork2 = nullptr, ev_join2 = nullptr;
-    cudaEvent_t ev_sel = nullptr;                 // the selection of the current iteration is done
-    cudaEvent_t ev_fcnt = nullptr;                // ... and its finish count copied to fin_h
-    int* fin_h = nullptr;                         // pinned
+    HostView* view = nullptr;                     // mapped pinned memory, written by the compaction
+    bool in_solve = false;                        // a solve began and did not end (it returned an error)
     cudaEvent_t ev_fin[FIN_SLOTS] = {};           // the exact finish of the last iteration of each slot
     int use_graph = 1;
     struct GraphEntry {
-        int p, tk, par, nog, prof, route, part;
+        int p, tk, slot, nog, prof, route;
         double tol;
         int64_t kernels;  // kernel launches captured in the graph
         cudaGraphExec_t exec;
@@ -443,7 +443,7 @@ mpl_status_t mpl_create(const float* A, int n, int m, mpl_handle_t* out) {
     if (cudaMalloc(&h->colnorm, (size_t)m * sizeof(float)) != cudaSuccess) return fail(MPL_ERR_OOM);
     if (cudaMalloc(&h->scal, 16 * sizeof(float)) != cudaSuccess) return fail(MPL_ERR_OOM);
     if (cudaMallocHost(&h->cnt_h, sizeof(Counters)) != cudaSuccess) return fail(MPL_ERR_OOM);
-    if (cudaMallocHost(&h->fin_h, sizeof(int)) != cudaSuccess) return fail(MPL_ERR_OOM);
+    if (cudaHostAlloc(&h->view, sizeof(HostView), cudaHostAllocMapped) != cudaSuccess) return fail(MPL_ERR_OOM);
     if (cudaMemcpy(h->A32, A, bytes, cudaMemcpyDefault) != cudaSuccess) return fail(MPL_ERR_CUDA);
     int64_t nl = 0;
     if (launch_colnorm(h->A32, n, m, h->colnorm, nullptr, 0, &nl) != cudaSuccess) return fail(MPL_ERR_CUDA);
@@ -469,7 +469,7 @@ void mpl_destroy(mpl_handle_t h) {
     cudaFree(h->Xst);
     for (float* q : {h->pw, h->pwb, h->pm1, h->pm2, h->pgrad, h->ppart, h->pacc, h->rn}) cudaFree(q);
     if (h->cnt_h) cudaFreeHost(h->cnt_h);
-    if (h->fin_h) cudaFreeHost(h->fin_h);
+    if (h->view) cudaFreeHost(h->view);
     clear_graphs(h);
     for (cudaStream_t q : h->fin_st)
         if (q) cudaStreamDestroy(q);
@@ -479,8 +479,6 @@ void mpl_destroy(mpl_handle_t h) {
     if (h->ev_join2) cudaEventDestroy(h->ev_join2);
     if (h->ev_in) cudaEventDestroy(h->ev_in);
     if (h->ev_out) cudaEventDestroy(h->ev_out);
-    for (cudaEvent_t e : {h->ev_sel, h->ev_fcnt})
-        if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : h->ev_fin)
         if (e) cudaEventDestroy(e);
     for (auto e : h->evpool) cudaEventDestroy(e);
@@ -665,23 +663,20 @@ static int iteration_route(const mpl_ctx* h, const Dev& d, int t) {
     return sb <= h->qroute ? ROUTE_Q : ROUTE_GEMM;
 }
 
-// One outer iteration of Algorithm 1 for every active signal, in two parts (kernels only):
-//   part 0  re-entry of the signals whose exact finish of an earlier iteration is done (the
-//           slots the host put in the device counter mslots), the worst-case analysis
-//           (correlation) and the selection, which ends by building the work lists;
-//   part 1  Gram growth, master problems and residual update of the signals that took atoms.
-// Between the parts the host launches the exact finish of the signals without violators
-// (list_fin[t % FIN_SLOTS]) on its own stream, where it overlaps part 1 and the next
-// iterations.
+// One outer iteration of Algorithm 1 for every active signal (kernels only): the worst-case
+// analysis (correlation) and the selection, which ends by building the work lists and telling the
+// host their lengths (HostView); then Gram growth, master problems and residual update of the
+// signals that took atoms.  While these run, the host launches the exact finish of the
+// signals without violators (list_fin[t % FIN_SLOTS]) on its own stream, where it overlaps
+// them and the next iterations, and queues the next iteration.
 // pt == nullptr: no timing events (graph capture).
-static cudaError_t launch_part(mpl_ctx* h, const Dev& d, int t, int part, int act_ub, cudaStream_t run,
-                               PhaseTimer* pt, int64_t* nl) {
-    const int cur = t & 1;
+static cudaError_t launch_iteration(mpl_ctx* h, const Dev& d, int t, int act_ub, cudaStream_t run, PhaseTimer* pt,
+                                    int64_t* nl) {
+    const int cur = t & 1, slot = t % FIN_SLOTS;
     cudaError_t e;
-    if (part == 0) {
+    {
         const int no_grow = t >= h->max_outer;
         const int route = iteration_route(h, d, t);
-        if (t >= 1 && (e = launch_merge(d, cur, act_ub, run, nl)) != cudaSuccess) return e;
         const int ph_corr = route == ROUTE_Q ? PH_QROUTE : 1;
         cudaEvent_t e0 = pt ? pt->begin_if(ph_corr, run) : nullptr;
         if (route == ROUTE_Q) {
@@ -711,7 +706,7 @@ static cudaError_t launch_part(mpl_ctx* h, const Dev& d, int t, int part, int ac
             pa.w = h->pwb;
             pa.rn = h->rn;
         }
-        if ((e = launch_select(d, cur, no_grow, act_ub, run, nl, propose ? &pa : nullptr, route, fuse, 1)) !=
+        if ((e = launch_select(d, cur, no_grow, act_ub, run, nl, propose ? &pa : nullptr, route, fuse, 1, slot)) !=
             cudaSuccess)
             return e;
         if (d.ovf_list) {
@@ -726,9 +721,8 @@ static cudaError_t launch_part(mpl_ctx* h, const Dev& d, int t, int part, int ac
                 cudaSuccess)
                 return e;
         }
-        if (!fuse && (e = launch_compact(d, cur, run, nl)) != cudaSuccess) return e;
+        if (!fuse && (e = launch_compact(d, cur, slot, run, nl)) != cudaSuccess) return e;
         if (pt) pt->end(2, e0, run);
-        return cudaSuccess;
     }
     // bound on |S| after this iteration's growth: omega*rho explored atoms on top of rho per
     // earlier iteration (Algorithm 2 prunes back to rho), plus what a warm start admits
@@ -762,23 +756,17 @@ static cudaError_t launch_part(mpl_ctx* h, const Dev& d, int t, int part, int ac
     return cudaSuccess;
 }
 
-// Bound on |S| of the signals an iteration sends to the exact finish.
-static int finish_scap(const mpl_ctx* h, const Dev& d, int t) {
-    return std::min(d.smax, t * d.rho + d.omega * d.rho + warm_additions(h, d));
-}
-
-// Captured part of iteration (p, t): iterations past the point where the active-set bound
-// saturates share one graph per parity and part.
-static cudaError_t iteration_graph(mpl_ctx* h, const Dev& d, int t, int part, int p, double tol, cudaStream_t run,
-                                   size_t* out, int64_t* nl) {
+// Captured iteration (p, t): iterations past the point where the active-set bound saturates
+// share one graph per finish list slot.
+static cudaError_t iteration_graph(mpl_ctx* h, const Dev& d, int t, int p, double tol, cudaStream_t run, size_t* out) {
     const int tsat = (d.smax + d.rho - 1) / d.rho;  // beyond this the active-set bound is smax
     const int tk = std::min(t, tsat + 2);
-    const int par = t & 1, nog = t >= h->max_outer ? 1 : 0, prof = h->profile ? 1 : 0;
+    const int slot = t % FIN_SLOTS, nog = t >= h->max_outer ? 1 : 0, prof = h->profile ? 1 : 0;
     const int route = iteration_route(h, d, t) + 4 * (t == 0 && h->qroute > 0 ? 1 : 0);
     for (size_t gi = 0; gi < h->graphs.size(); ++gi) {
         const auto& g = h->graphs[gi];
-        if (g.p == p && g.tk == tk && g.par == par && g.nog == nog && g.prof == prof && g.route == route &&
-            g.part == part && g.tol == tol) {
+        if (g.p == p && g.tk == tk && g.slot == slot && g.nog == nog && g.prof == prof && g.route == route &&
+            g.tol == tol) {
             *out = gi;
             return cudaSuccess;
         }
@@ -788,7 +776,7 @@ static cudaError_t iteration_graph(mpl_ctx* h, const Dev& d, int t, int part, in
     int64_t cnt = 0;
     PhaseTimer gpt{h, run, {}, 0, true};
     gpt.only_a = -1;  // every phase (the profiling pass is timed apart from the reported one)
-    cudaError_t el = launch_part(h, d, t, part, p, run, prof ? &gpt : nullptr, &cnt);
+    cudaError_t el = launch_iteration(h, d, t, p, run, prof ? &gpt : nullptr, &cnt);
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(run, &graph);
     if (el != cudaSuccess) {
@@ -800,9 +788,8 @@ static cudaError_t iteration_graph(mpl_ctx* h, const Dev& d, int t, int part, in
     e = cudaGraphInstantiate(&exec, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return e;
-    h->graphs.push_back({p, tk, par, nog, prof, route, part, tol, cnt, exec, gpt.marks});
+    h->graphs.push_back({p, tk, slot, nog, prof, route, tol, cnt, exec, gpt.marks});
     *out = h->graphs.size() - 1;
-    (void)nl;
     return cudaSuccess;
 }
 
@@ -815,10 +802,29 @@ static mpl_status_t ensure_streams(mpl_ctx* h) {
     CK(cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi));
     for (cudaStream_t& q : h->fin_st) CK(cudaStreamCreateWithPriority(&q, cudaStreamNonBlocking, prio_lo));
     CK(cudaStreamCreateWithPriority(&h->side2, cudaStreamNonBlocking, prio_hi));
-    cudaEvent_t* evs[] = {&h->ev_fork2, &h->ev_join2, &h->ev_in, &h->ev_out, &h->ev_sel, &h->ev_fcnt};
+    cudaEvent_t* evs[] = {&h->ev_fork2, &h->ev_join2, &h->ev_in, &h->ev_out};
     for (cudaEvent_t* e : evs) CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
     for (cudaEvent_t& e : h->ev_fin) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     CK(cudaStreamCreateWithPriority(&h->main, cudaStreamNonBlocking, prio_hi));
+    return MPL_OK;
+}
+
+// Until the compaction of the solve's `want`-th selection has written the view.  The stream is
+// asked now and then whether it failed, or ran dry without writing it (every kernel of the
+// chain is bounded, so one or the other happens).
+static mpl_status_t wait_view(mpl_ctx* h, cudaStream_t st, unsigned want) {
+    const volatile unsigned* seq = &h->view->seq;
+    for (unsigned spin = 1; *seq != want; ++spin) {
+        if ((spin & 0xffffu) != 0u) continue;
+        const cudaError_t q = cudaStreamQuery(st);
+        if (q == cudaErrorNotReady) {
+            (void)cudaGetLastError();  // (not an error: still running)
+            continue;
+        }
+        CK(q);
+        if (*seq != want) return MPL_ERR_CUDA;
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
     return MPL_OK;
 }
 
@@ -876,6 +882,12 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
     d.A16 = h->A16;
     d.B = h->Bint;
     d.lam = h->lamint;
+    d.view = h->view;
+    // no kernel of an earlier solve may write the view after this: one that ended has waited for
+    // them, one that returned an error has not
+    if (h->in_solve) CK(cudaDeviceSynchronize());
+    h->in_solve = true;
+    std::memset(h->view, 0, sizeof(HostView));
     set_bounds(h, d);
     // a second, FP32 selection pass for bands that overflow the candidate buffer: only
     // for the wide bands (BF16 GEMM, identity route) of dictionaries above the row cache
@@ -910,11 +922,10 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
     bool pend[FIN_SLOTS] = {};  // finish launched, its signals not merged yet
     int pend_n[FIN_SLOTS] = {};  // and how many signals it took
     int pend_t[FIN_SLOTS] = {};  // and the iteration it was launched in
-    std::vector<size_t> window;  // graphs launched since the last handshake (phase timing)
     double graph_phase[16] = {0};
     int t = 0;
 #ifdef MPL_TIMELINE
-    // diagnostic build: device timestamps of every iteration's parts and finish
+    // diagnostic build: device timestamps of every iteration and finish
     struct Mark { int t, kind; cudaEvent_t e; };
     std::vector<Mark> marks;
     auto mark = [&](int kind, cudaStream_t s_) {
@@ -925,17 +936,18 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
     };
     mark(-1, st);
 #endif
+    const bool early = h->stop_rinf >= 0.0 || h->stop_r2 >= 0.0 || h->stop_eps >= 0.0;
+    bool drain = false;  // only finishes are left: the next iteration waits for all of them
     for (; live > 0 && t < hard_cap; ++t) {
-        const int par = t & 1;
         const int fs = t % FIN_SLOTS;
         cudaStream_t fin_st = h->fin_st[fs];
         // re-entry: the finishes that are done by now, and the one whose slot this iteration's
         // selection fills (launched FIN_SLOTS iterations ago), waited for; with
         // MPL_OPT_REENTRY = 1 exactly the finish of two iterations back, waited for
-        int mask = 0;
+        int mask = 0, back = 0;
         for (int q = 0; q < FIN_SLOTS; ++q) {
             if (!pend[q]) continue;
-            bool ready = q == fs || (h->reentry == 1 && pend_t[q] + 2 <= t);
+            bool ready = q == fs || drain || (h->reentry == 1 && pend_t[q] + 2 <= t);
             if (!ready && h->reentry == 0) {
                 const cudaError_t eq = cudaEventQuery(h->ev_fin[q]);
                 if (eq == cudaSuccess) {
@@ -950,100 +962,86 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
             if (ready) {
                 CK(cudaStreamWaitEvent(st, h->ev_fin[q], 0));
                 mask |= 1 << q;
+                back += pend_n[q];
                 pend[q] = false;
             }
         }
-        // (the slot itself advances on the device, in the merge at the start of part 0)
-        if (mask) CK(launch_set_merge(d, mask, st, &nl));
+        drain = false;
+        if (mask) CK(launch_merge(d, t & 1, mask, back, st, &nl));
 #ifdef MPL_TIMELINE
         mark(0, st);
 #endif
-        for (int part = 0; part < 2; ++part) {
-            if (graph) {
-                size_t gi = 0;
-                CK(iteration_graph(h, d, t, part, p, tol, st, &gi, &nl));
-                CK(cudaGraphLaunch(h->graphs[gi].exec, st));
-                nl += h->graphs[gi].kernels;
-                window.push_back(gi);
-            } else {
-                CK(launch_part(h, d, t, part, live, st, &pt, &nl));
+        if (graph) {
+            size_t gi = 0;
+            CK(iteration_graph(h, d, t, p, tol, st, &gi));
+            CK(cudaGraphLaunch(h->graphs[gi].exec, st));
+            nl += h->graphs[gi].kernels;
+            if (h->profile) {  // (the next launch of this graph would overwrite its events)
+                CK(cudaStreamSynchronize(st));
+                for (auto& mk : h->graphs[gi].marks) {
+                    float ms = 0.f;
+                    cudaEventElapsedTime(&ms, mk.second.first, mk.second.second);
+                    graph_phase[mk.first] += ms;
+                }
             }
-            if (part == 0) {
-                // the selection is done: its count of signals without violators comes back
-                // while part 1 runs
-                CK(cudaEventRecord(h->ev_sel, st));
-                CK(cudaMemcpyAsync(h->fin_h, &d.cnt->fin_par[fs], sizeof(int), cudaMemcpyDeviceToHost, st));
-                CK(cudaEventRecord(h->ev_fcnt, st));
-#ifdef MPL_TIMELINE
-                mark(1, st);
-#endif
-            }
-        }
-        {
-            // the exact finish of the signals without violators, beside part 1 and the next
-            // iterations, its grid and cluster size from their count
-            CK(cudaEventSynchronize(h->ev_fcnt));
-            const int nf = *h->fin_h;
-            CK(cudaStreamWaitEvent(fin_st, h->ev_sel, 0));
-            cudaEvent_t f0 = pt.begin(fin_st);
-#ifdef MPL_TIMELINE
-            mark(3, fin_st);
-#endif
-            if (nf > 0) CK(launch_finish(d, fs, nf, nf, finish_scap(h, d, t), fin_st, &nl, h->sms));
-            pt.end(4, f0, fin_st);
-            CK(cudaEventRecord(h->ev_fin[fs], fin_st));
-            pend[fs] = nf > 0;
-            pend_n[fs] = nf;
-            pend_t[fs] = t;
-#ifdef MPL_TIMELINE
-            mark(4, fin_st);
-#endif
+        } else {
+            CK(launch_iteration(h, d, t, live, st, &pt, &nl));
         }
 #ifdef MPL_TIMELINE
         mark(2, st);
 #endif
-        const bool last = t + 1 >= hard_cap;
-        if ((t + 1) % h->sync_every == 0 || last) {
-            CK(cudaMemcpyAsync(h->cnt_h, d.cnt, sizeof(Counters), cudaMemcpyDeviceToHost, st));
-            CK(cudaStreamSynchronize(st));
+        // the lists of this iteration, known as soon as its selection is done: the host launches
+        // the finish and queues the next iteration while the rest of this one runs
+        const mpl_status_t vs = wait_view(h, st, (unsigned)t + 1u);
+        if (vs != MPL_OK) return vs;
+        const HostView v = *h->view;
 #ifdef MPL_BOUNDS
-            if (h->cnt_h->err != 0)
-                fprintf(stderr, "mpl: device error %d at iteration %d, bounds site %d\n", h->cnt_h->err, t,
-                        h->cnt_h->bounds_site);
+        if (v.err != 0) fprintf(stderr, "mpl: device error %d at iteration %d\n", v.err, t);
 #endif
-            if (h->cnt_h->err != 0) return h->cnt_h->err == DERR_TIMEOUT ? MPL_ERR_TIMEOUT : MPL_ERR_CUDA;
-            // active next iteration, plus the signals of the finishes not merged yet
-            const int act_next = h->cnt_h->act_n[par ^ 1];
-            int in_fin = 0;
-            for (int q = 0; q < FIN_SLOTS; ++q) in_fin += pend[q] ? pend_n[q] : 0;
-            live = act_next + in_fin;
-            if (act_next == 0 && in_fin > 0) {
-                // nothing left to iterate on but finishes in flight: wait for them, and go on
-                // only for the signals they send back
-                for (int q = 0; q < FIN_SLOTS; ++q)
-                    if (pend[q]) CK(cudaEventSynchronize(h->ev_fin[q]));
-                CK(cudaMemcpyAsync(h->cnt_h, d.cnt, sizeof(Counters), cudaMemcpyDeviceToHost, st));
-                CK(cudaStreamSynchronize(st));
-                if (h->cnt_h->err != 0) return h->cnt_h->err == DERR_TIMEOUT ? MPL_ERR_TIMEOUT : MPL_ERR_CUDA;
-                int back = 0;
-                for (int q = 0; q < FIN_SLOTS; ++q) back += pend[q] ? h->cnt_h->reent_n[q] : 0;
-                if (back == 0)
-                    for (bool& q : pend) q = false;
-                live = back;
-            }
-
+        if (v.err != 0) return v.err == DERR_TIMEOUT ? MPL_ERR_TIMEOUT : MPL_ERR_CUDA;
+        {
+            // the exact finish of the signals without violators, its grid, cluster size and
+            // shared memory from their count and their largest active set (its launch follows
+            // the selection through the view)
+            cudaEvent_t f0 = pt.begin(fin_st);
 #ifdef MPL_TIMELINE
-            fprintf(stderr, "TC %d %d %d %d\n", t, act_next, h->cnt_h->fin_par[fs], h->cnt_h->grow_n);
+            mark(3, fin_st);
 #endif
-            if (graph && h->profile) {
-                for (size_t gi : window)
-                    for (auto& mk : h->graphs[gi].marks) {
-                        float ms = 0.f;
-                        cudaEventElapsedTime(&ms, mk.second.first, mk.second.second);
-                        graph_phase[mk.first] += ms;
-                    }
+            h->view->reent[fs] = 0;
+            if (v.fin_n > 0) {
+                CK(launch_finish(d, fs, v.fin_n, v.fin_n, std::max(v.fin_smax, 1), fin_st, &nl, h->sms));
+                CK(cudaEventRecord(h->ev_fin[fs], fin_st));
             }
-            window.clear();
+            pt.end(4, f0, fin_st);
+            pend[fs] = v.fin_n > 0;
+            pend_n[fs] = v.fin_n;
+            pend_t[fs] = t;
+#ifdef MPL_TIMELINE
+            mark(4, fin_st);
+            fprintf(stderr, "TC %d %d %d %d\n", t, v.act_next, v.fin_n, v.grow_n);
+#endif
+        }
+        // active next iteration, plus the signals of the finishes not merged yet
+        int in_fin = 0;
+        for (int q = 0; q < FIN_SLOTS; ++q) in_fin += pend[q] ? pend_n[q] : 0;
+        live = v.act_next + in_fin;
+        if (v.act_next == 0 && in_fin > 0) {
+            // nothing left to iterate on but finishes in flight.  Their signals come back for the
+            // worst-case analysis, so the next iteration is queued behind them; under an
+            // early-stopping rule they may all have ended, so the host waits and looks
+            drain = h->reentry == 0;
+            if (early) {
+                bool any = false;
+                for (int q = 0; q < FIN_SLOTS; ++q)
+                    if (pend[q]) {
+                        CK(cudaEventSynchronize(h->ev_fin[q]));
+                        any = any || *const_cast<volatile int*>(&h->view->reent[q]) != 0;
+                    }
+                if (!any) {
+                    for (bool& q : pend) q = false;
+                    live = 0;
+                }
+            }
         }
     }
     // the last finishes, then the results
@@ -1067,6 +1065,7 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
     CK(cudaEventRecord(h->ev_out, st));
     CK(cudaStreamWaitEvent(caller, h->ev_out, 0));
     CK(cudaStreamSynchronize(st));
+    h->in_solve = false;
     if (h->cnt_h->err != 0) return h->cnt_h->err == DERR_TIMEOUT ? MPL_ERR_TIMEOUT : MPL_ERR_CUDA;
     pt.collect();
 #ifdef MPL_TIMELINE

@@ -60,9 +60,8 @@ struct Counters {
     int fin_par[FIN_SLOTS];  // ... by list slot (a finish runs while the next iterations do)
     int reent_n[FIN_SLOTS];  // finished signals waiting to re-enter the active list, by the
                              // slot of the finish they left
-    int fslot;       // the slot this iteration's selection fills (t % FIN_SLOTS, kept by the merge)
-    int mslots;      // bit s: the finish of slot s is done, merge its signals this iteration
-                     // (set by the host through k_set_merge, cleared by the merge)
+    int merge_done;  // merge CTAs finished (the last one updates the lengths)
+    unsigned iters;  // selections completed by this solve
     int apg_n;       // signals in the master-problem list (grow + failed finishes)
     int apg_head;    // work-queue head of the persistent master-problem kernel
     int apg_head2;   // head of its second queue (blocks streamed from global memory)
@@ -80,6 +79,19 @@ struct Counters {
     unsigned long long gram_bytes;    // bytes the Gram growth reads (Q or atoms, b) and writes (G, h)
     unsigned long long fin_bytes;     // bytes the exact finish streams (Gram rows, atom columns, b)
     __host__ __device__ int act_n_of(int c) const { return act_n[c]; }
+};
+
+// What the host steers the outer loop by, in mapped host memory: written by the compaction that
+// ends an iteration's selection, while the rest of the iteration still runs.  seq is written
+// last; the host polls it, so no copy or synchronisation sits in the chain.
+struct HostView {
+    int act_next;    // signals with a master problem: the next active list before re-entries
+    int fin_n;       // signals sent to the exact finish
+    int fin_smax;    // the largest |S| among them
+    int grow_n;
+    int err;         // Counters::err so far
+    int reent[FIN_SLOTS];  // 1: the finish of this slot left a signal to merge (cleared by the host)
+    unsigned seq;    // selections completed (Counters::iters)
 };
 
 // Everything a kernel may touch, passed by value.
@@ -160,6 +172,7 @@ struct Dev {
     int* reent[FIN_SLOTS];       // finished signals to merge back into the active list, by slot
     int* list_apg;               // master-problem work list
     Counters* cnt;
+    HostView* view;              // mapped host memory, or null (no solve loop)
     __device__ const int* act_of(int c) const { return act[c]; }
 };
 
@@ -221,14 +234,15 @@ inline int res_blocks(int n) { return (n + RES_ROWS - 1) / RES_ROWS; }
 bool sel_chunked(const Dev& d, int act_n_ub);
 cudaError_t launch_select(const Dev& d, int cur, int no_grow, int act_n_ub, cudaStream_t s, int64_t* nl,
                           const PropArgs* pa = nullptr, int route = ROUTE_GEMM, int fuse_compact = 0,
-                          int chunked = 0);
+                          int chunked = 0, int slot = 0);
 // Identity route (eq. batchQ): scores beta_i - Q_S x_S into the compacted score rows.
 cudaError_t launch_corr_q(const Dev& d, int cur, int act_n_ub, cudaStream_t s, int64_t* nl);
 // beta_i = score row of signal i (after an FP32 correlation of the residual b_i).
 cudaError_t launch_save_beta(const Dev& d, int cur, int act_n_ub, cudaStream_t s, int64_t* nl);
 cudaError_t build_gram_q(const float* A32, int n, int m, float* Q, int* act, Counters* cnt, cudaStream_t s,
                          int64_t* nl);
-cudaError_t launch_compact(const Dev& d, int cur, cudaStream_t s, int64_t* nl);
+// slot: the finish list slot of the iteration (t % FIN_SLOTS).
+cudaError_t launch_compact(const Dev& d, int cur, int slot, cudaStream_t s, int64_t* nl);
 // The new rows and columns of each growing signal's Gram block (h of the new atoms was
 // written by the selection that appended them).
 // qmax: most atoms a signal can take this iteration (picks the tile width).
@@ -242,12 +256,10 @@ cudaError_t launch_gram_gather(const Dev& d, int ub, cudaStream_t s, int64_t* nl
 constexpr int FIN_CLUSTER_MAX = 8;
 constexpr int FIN_CLUSTER_MIN_N = 2048;
 cudaError_t launch_finish(const Dev& d, int slot, int ub, int est, int scap, cudaStream_t s, int64_t* nl, int sms);
-// Set the device counter mslots (the finished slots the next merge takes back).
-cudaError_t launch_set_merge(const Dev& d, int mask, cudaStream_t s, int64_t* nl);
-// Append reent[s] of every slot s in the device counter mslots to the active list of an
-// iteration with parity cur (rows for the GEMM included); the finishes that filled those
-// slots must be complete.  Advances the finish list slot to the one of this iteration.
-cudaError_t launch_merge(const Dev& d, int cur, int ub, cudaStream_t s, int64_t* nl);
+// Append reent[s] of every slot s in mask to the active list of an iteration with parity cur
+// (rows for the GEMM included); the finishes that filled those slots must be complete.
+// ub bounds their signals.
+cudaError_t launch_merge(const Dev& d, int cur, int mask, int ub, cudaStream_t s, int64_t* nl);
 // Master-problem launches: every signal of the work list, or only those whose Gram block fits
 // shared memory, or only those streamed from global memory.
 enum ApgClass : int { APG_ALL = 0, APG_SMEM = 1, APG_GLOBAL = 2 };
@@ -322,7 +334,8 @@ constexpr int APG_THREADS = 256;
 constexpr size_t FIN_SMEM_TWO_CTAS = 110 * 1024;  // dynamic shared memory that keeps 2 finish CTAs per SM
 constexpr size_t FIN_SMEM_MAX = 225 * 1024;       // the most one finish CTA takes
 constexpr int FIN_THREADS = 256;
-constexpr int FIN_THREADS_WIDE = 512;  // one finish CTA per SM (large active sets)
+constexpr int FIN_THREADS_WIDE = 512;  // one finish CTA per SM (large active sets, long signals)
+constexpr int FIN_WIDE_MIN_N = 4096;
 constexpr int FIN_MAX_PIVOTS = 16;
 constexpr int FIN_CG_MAXIT = 60;  // CG iterations per solve before the finish falls back to a factor
 constexpr int FIN_CG_MIN_S = 128; // active sets above this size (with a factor outside shared memory) use CG

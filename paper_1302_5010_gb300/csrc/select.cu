@@ -1188,14 +1188,16 @@ __device__ __forceinline__ void select_body(const Dev& d, int cur, int no_grow, 
 // iteration (one CTA): grow, finish, master problem, and the next active list.
 // The states were written by other CTAs of the same launch when the compaction
 // runs at the end of the selection, so they are read past L1.
-__device__ void compact_body(const Dev& d, int cur) {
+__device__ void compact_body(const Dev& d, int cur, int slot) {
     const int nact = d.cnt->act_n[cur];
     const int* act = d.act[cur];
     int* nxt = d.act[cur ^ 1];
     __shared__ int wsum[3][32];
     __shared__ int base[3];
+    __shared__ int smax_fin;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
     if (tid < 3) base[tid] = 0;
+    if (tid == 3) smax_fin = 0;
     if (tid < 96) wsum[tid / 32][tid % 32] = 0;
     __syncthreads();
     for (int c0 = 0; c0 < nact; c0 += nt) {
@@ -1205,6 +1207,7 @@ __device__ void compact_body(const Dev& d, int cur) {
         // the next active list: signals with a master problem to solve; the ones sent to the
         // exact finish leave it and come back through reent[] once their finish is done
         const int f[3] = {st == ST_GROW || st == ST_REFINE, st == ST_FINALIZE, st == ST_GROW || st == ST_REFINE};
+        if (st == ST_FINALIZE) atomicMax(&smax_fin, __ldcg(d.ssize + sig));
         if (st == ST_REFINE) d.state[sig] = ST_GROW;  // master problem again, no new atoms
         int pre[3];
         const unsigned lt = (1u << lane) - 1u;
@@ -1233,7 +1236,7 @@ __device__ void compact_body(const Dev& d, int cur) {
             if (f[q]) {
                 if (MPL_OOB(off < 0 || off >= d.p || sig < 0 || sig >= d.p, 504)) continue;
                 if (q == 0) { d.list_grow[off] = sig; d.list_apg[off] = sig; }
-                else if (q == 1) d.list_fin[d.cnt->fslot][off] = sig;
+                else if (q == 1) d.list_fin[slot][off] = sig;
                 else {
                     nxt[off] = sig;
                     if (d.pos) d.pos[sig] = off;  // its GEMM row next iteration
@@ -1250,23 +1253,37 @@ __device__ void compact_body(const Dev& d, int cur) {
         d.cnt->grow_n = base[0];
         d.cnt->apg_n = base[0];
         d.cnt->fin_n = base[1];
-        d.cnt->fin_par[d.cnt->fslot] = base[1];
+        d.cnt->fin_par[slot] = base[1];
         d.cnt->act_n[cur ^ 1] = base[2];
         d.cnt->apg_head = 0;
         d.cnt->apg_head2 = 0;
+        const unsigned it = ++d.cnt->iters;
+        if (d.view) {
+            // the host may launch the finish and the next iteration as soon as it sees seq: the
+            // lists (this CTA's, above) and the selections' results (fenced by their CTAs
+            // before the last one's turn, or by the kernel boundary) come before it
+            volatile HostView* v = d.view;
+            v->act_next = base[2];
+            v->fin_n = base[1];
+            v->fin_smax = smax_fin;
+            v->grow_n = base[0];
+            v->err = d.cnt->err;
+            __threadfence_system();
+            v->seq = it;
+        }
     }
 }
 
-__global__ void __launch_bounds__(1024) k_compact(Dev d, int cur) {
+__global__ void __launch_bounds__(1024) k_compact(Dev d, int cur, int slot) {
     pdl_enter();
-    compact_body(d, cur);
+    compact_body(d, cur, slot);
 }
 
 // The selection of one outer iteration; with fuse set, the last CTA to finish
 // (counted with a fenced atomic) also runs the compaction, saving a launch.
 template <bool CHUNKED>
 __global__ void __launch_bounds__(SEL_THREADS, 2) k_select(Dev d, int cur, int no_grow, PropArgs pa, int route,
-                                                           int fuse) {
+                                                           int fuse, int slot) {
     pdl_enter();
     select_body<CHUNKED>(d, cur, no_grow, pa, route);
     if (!fuse) return;
@@ -1279,8 +1296,8 @@ __global__ void __launch_bounds__(SEL_THREADS, 2) k_select(Dev d, int cur, int n
     __syncthreads();
     if (!last) return;
     __threadfence();
-    compact_body(d, cur);
     if (threadIdx.x == 0) d.cnt->sel_done = 0;
+    compact_body(d, cur, slot);
 }
 
 // Chunk maxima of the score rows (see fast_kth_chunks): warp w of signal position blockIdx.x
@@ -1362,7 +1379,7 @@ cudaError_t prepare_select() {
 }
 
 cudaError_t launch_select(const Dev& d, int cur, int no_grow, int act_n_ub, cudaStream_t s, int64_t* nl,
-                          const PropArgs* pa, int route, int fuse_compact, int chunked) {
+                          const PropArgs* pa, int route, int fuse_compact, int chunked, int slot) {
     if (act_n_ub <= 0) return cudaSuccess;
     PropArgs a{};
     if (pa) a = *pa;
@@ -1377,16 +1394,16 @@ cudaError_t launch_select(const Dev& d, int cur, int no_grow, int act_n_ub, cuda
         ++*nl;
     }
     e = chunked ? launch_chain(k_select<true>, dim3(act_n_ub), dim3(SEL_THREADS), sm, s, d, cur, no_grow, a, route,
-                               fuse_compact)
+                               fuse_compact, slot)
                 : launch_chain(k_select<false>, dim3(act_n_ub), dim3(SEL_THREADS), sm, s, d, cur, no_grow, a, route,
-                               fuse_compact);
+                               fuse_compact, slot);
     if (e != cudaSuccess) return e;
     ++*nl;
     return cudaGetLastError();
 }
 
-cudaError_t launch_compact(const Dev& d, int cur, cudaStream_t s, int64_t* nl) {
-    const cudaError_t e = launch_chain(k_compact, dim3(1), dim3(1024), 0, s, d, cur);
+cudaError_t launch_compact(const Dev& d, int cur, int slot, cudaStream_t s, int64_t* nl) {
+    const cudaError_t e = launch_chain(k_compact, dim3(1), dim3(1024), 0, s, d, cur, slot);
     if (e != cudaSuccess) return e;
     ++*nl;
     return cudaGetLastError();

@@ -163,8 +163,8 @@ __global__ void __launch_bounds__(256) k_init(Dev d) {
             d.cnt->bounds_site = 0;
             d.cnt->apg_elems = d.cnt->apg_gl_elems = 0ull;
             for (int q = 0; q < FIN_SLOTS; ++q) d.cnt->fin_par[q] = d.cnt->reent_n[q] = 0;
-            d.cnt->fslot = 0;
-            d.cnt->mslots = 0;
+            d.cnt->merge_done = 0;
+            d.cnt->iters = 0u;
             d.cnt->res_bytes = d.cnt->gram_bytes = d.cnt->fin_bytes = 0ull;
         }
     }
@@ -1304,13 +1304,13 @@ cudaError_t launch_residual(const Dev& d, int ub, cudaStream_t s, int64_t* nl) {
 
 // Per-signal statistics packed on the device into the host struct layout (one copy back).
 // ------------------------------------------------------------------ re-entry
-// Finished signals (reent[s] of the slots s in mslots, in slot order) go back to the end of
+// Finished signals (reent[s] of the slots s in mask, in slot order) go back to the end of
 // the active list of this iteration, with their rows in the GEMM's compacted BF16 residual
-// (the finish wrote the per-signal copy); the counters are updated by k_merge_count once
-// every row is in place.
-__global__ void __launch_bounds__(256) k_merge(Dev d, int cur) {
+// (the finish wrote the per-signal copy).  Launched only when a finish is done; the last CTA
+// updates the lengths, once every CTA has read them.
+__global__ void __launch_bounds__(256) k_merge(Dev d, int cur, int mask) {
     pdl_enter();
-    const int mask = d.cnt->mslots, n = d.n;
+    const int n = d.n;
     int base = d.cnt->act_n[cur];
     for (int q = 0; q < FIN_SLOTS; ++q) {
         if (!((mask >> q) & 1)) continue;
@@ -1331,45 +1331,24 @@ __global__ void __launch_bounds__(256) k_merge(Dev d, int cur) {
         }
         base += cnt;
     }
-}
-
-// Also advances the finish list slot of the selection that follows (t % FIN_SLOTS for outer
-// iteration t; k_init starts it at 0) and clears the merge mask the host set.
-__global__ void k_merge_count(Dev d, int cur) {
-    pdl_enter();
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        const int mask = d.cnt->mslots;
-        for (int q = 0; q < FIN_SLOTS; ++q) {
-            if (!((mask >> q) & 1)) continue;
-            d.cnt->act_n[cur] += d.cnt->reent_n[q];
-            d.cnt->reent_n[q] = 0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&d.cnt->merge_done, 1) == (int)gridDim.x - 1) {
+            for (int q = 0; q < FIN_SLOTS; ++q)
+                if ((mask >> q) & 1) d.cnt->reent_n[q] = 0;
+            d.cnt->act_n[cur] = base;
+            d.cnt->merge_done = 0;
         }
-        d.cnt->mslots = 0;
-        d.cnt->fslot = (d.cnt->fslot + 1) % FIN_SLOTS;
     }
 }
 
-// The finishes whose signals the next merge takes back (bit s: list slot s), from the host.
-__global__ void k_set_merge(Dev d, int mask) {
-    pdl_enter();
-    if (threadIdx.x == 0 && blockIdx.x == 0) d.cnt->mslots = mask;
-}
-
-cudaError_t launch_set_merge(const Dev& d, int mask, cudaStream_t s, int64_t* nl) {
-    const cudaError_t e = launch_chain(k_set_merge, dim3(1), dim3(32), 0, s, d, mask);
-    if (e != cudaSuccess) return e;
-    ++*nl;
-    return cudaGetLastError();
-}
-
-cudaError_t launch_merge(const Dev& d, int cur, int ub, cudaStream_t s, int64_t* nl) {
+cudaError_t launch_merge(const Dev& d, int cur, int mask, int ub, cudaStream_t s, int64_t* nl) {
     if (ub <= 0) return cudaSuccess;
     const int grid = ub < 608 ? ub : 608;
-    cudaError_t e = launch_chain(k_merge, dim3(grid), dim3(256), 0, s, d, cur);
+    const cudaError_t e = launch_chain(k_merge, dim3(grid), dim3(256), 0, s, d, cur, mask);
     if (e != cudaSuccess) return e;
-    e = launch_chain(k_merge_count, dim3(1), dim3(32), 0, s, d, cur);
-    if (e != cudaSuccess) return e;
-    *nl += 2;
+    ++*nl;
     return cudaGetLastError();
 }
 
