@@ -381,16 +381,17 @@ __device__ unsigned radix_kth(K key, int m, int kth, SelSmem& sh) {
 // from fill_cache.  Let jw = ceil(kth / warps); every warp has jw threads whose
 // largest key is at least the warp's jw-th largest thread maximum, so at least
 // kth distinct keys are >= T = the minimum of those over the warps: T is a lower
-// bound on the kth largest key.  The keys >= T (with their atoms) go to a list
+// bound on the kth largest key.  (Short rows leave the last warps without keys; they do not
+// count.)  The keys >= T (with their atoms) go to a list
 // in sh.key as (key << 32 | j); the kth largest is the entry with exactly
 // kth - 1 entries above it.  Returns false (the caller takes the radix passes)
 // when T is 0 or the list has more than blockDim.x entries.  On success *tlo = T
 // and *below = the largest key < T (for the bound on the atoms left out).
 __device__ bool fast_kth(const unsigned* keys, int m, int kth, unsigned tmax, SelSmem& sh, unsigned* kkey,
                          unsigned* tlo, unsigned* below) {
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    const int nw = min(nt >> 5, (m + 127) >> 7);  // warps that own keys (four per thread and round)
     const int jw = (kth + nw - 1) / nw;
-    if (jw > 32) return false;
     unsigned v = tmax;
     if (jw == 1) {
 #pragma unroll
@@ -567,7 +568,34 @@ __device__ bool fast_kth_chunks(const float* row, const uint32_t* msk, int m, co
                                 int sig) {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
     if (kth > nch) { CK_TRACE(sig, 1, 0, 0, 0); return false; }
-    const unsigned T = radix_kth(PlainKeys{tm}, nch, kth, sh);
+    // the maxima staged once in the row cache's space where they fit (one round trip to global
+    // memory, which is slow while other CTAs stream atoms through it), their kth largest by the
+    // list, or by the radix passes
+    const bool staged = nch <= SEL_ROWCACHE;
+    unsigned* tms = reinterpret_cast<unsigned*>(sh.row);
+    unsigned T = 0u;
+    bool found = false;
+    if (staged) {
+        unsigned tmax = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int c0 = own_atom(tid, nt, u, 0);
+            unsigned k4[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) k4[e] = c0 + e < nch ? __ldcg(tm + c0 + e) : 0u;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (c0 + e < nch) tms[c0 + e] = k4[e];
+                tmax = max(tmax, k4[e]);
+            }
+        }
+        __syncthreads();
+        unsigned lo_t, below_t;
+        found = fast_kth(tms, nch, kth, tmax, sh, &T, &lo_t, &below_t);
+        __syncthreads();
+    }
+    const unsigned* tk = staged ? tms : tm;
+    if (!found) T = radix_kth(PlainKeys{tk}, nch, kth, sh);
     if (T == 0u) { CK_TRACE(sig, 2, 0, 0, 0); return false; }
     const float tv = fmaxf((__uint_as_float(T) - band) * (1.f - 2e-6f), lo);
     const unsigned TL = tv > 0.f ? min(__float_as_uint(tv), T) : 1u;
@@ -577,7 +605,7 @@ __device__ bool fast_kth_chunks(const float* row, const uint32_t* msk, int m, co
     unsigned omax = 0;
     for (int cb = tid - lane; cb < nch; cb += nt) {
         const int c = cb + lane;
-        const unsigned mx = c < nch ? tm[c] : 0u;
+        const unsigned mx = c < nch ? tk[c] : 0u;
         const bool take = c < nch && mx >= TL;
         const unsigned bal = __ballot_sync(0xffffffffu, take);
         unsigned base = 0;
@@ -596,12 +624,22 @@ __device__ bool fast_kth_chunks(const float* row, const uint32_t* msk, int m, co
     if (cc > (unsigned)SEL_KCAP) { CK_TRACE(sig, 3, 0, 0, cc); return false; }  // uniform
     // their keys: one warp per chunk, lane l on atom l of the chunk (the front holds at most
     // nt entries, the back the other SEL_KCAP - nt)
-    for (unsigned q = warp; q < cc; q += nw) {
-        const int j0 = sh.idx[q] * SEL_CHUNK;
-        for (int u = 0; u < SEL_CHUNK; u += 32) {
-            const int j = j0 + u + lane;
+    static_assert(SEL_CHUNK == 32, "a lane per atom of a chunk");
+    constexpr int CQ = 4;  // chunks whose keys a warp reads together
+    for (unsigned q0 = warp; q0 < cc; q0 += CQ * nw) {
+        unsigned kq[CQ];
+        int jq[CQ];
+#pragma unroll
+        for (int u = 0; u < CQ; ++u) {
+            const unsigned q = q0 + u * nw;
+            jq[u] = q < cc ? sh.idx[q] * SEL_CHUNK + lane : m;
             int nf = 0;
-            const unsigned kj = j < m ? key_of(row, msk, j, &nf) : 0u;
+            kq[u] = jq[u] < m ? key_of(row, msk, jq[u], &nf) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < CQ; ++u) {
+            const int j = jq[u];
+            const unsigned kj = kq[u];
             const bool hiw = j < m && kj >= T;
             const bool low = j < m && kj >= TL && kj < T;
             const unsigned bh = __ballot_sync(0xffffffffu, hiw), bl = __ballot_sync(0xffffffffu, low);
@@ -1056,20 +1094,7 @@ __device__ __forceinline__ void select_body(const Dev& d, int cur, int no_grow, 
         sort_keys_desc(sh, n2, len3);
         if (tid == 0) {
             d.outer[i] += 1;
-            int q = 0;
-            const int room = min(d.smax - ss, pa.cap);
-            int* Si = d.S + (size_t)i * d.smax;
-            float* xi = d.xS + (size_t)i * d.smax;
-            uint32_t* mw = d.mask + (size_t)i * d.mw;
-            for (int t = 0; t < nv + n2 && q < room; ++t) {
-                const int j = t < nv ? __float_as_int(sh.sc[SEL_KCAP / 2 + t])
-                                     : (int)(0xffffffffu - (unsigned)(sh.key[t - nv] & 0xffffffffull));
-                if (MPL_OOB(j < 0 || j >= m || ss + q >= d.smax, 502)) break;
-                Si[ss + q] = j;
-                xi[ss + q] = 0.f;
-                mw[j >> 5] |= 1u << (j & 31);
-                ++q;
-            }
+            const int q = max(0, min(nv + n2, min(d.smax - ss, pa.cap)));
             d.ssize[i] = ss + q;
             d.snew[i] = q;
             if (d.explore) d.explore[i] = 0;
@@ -1080,7 +1105,17 @@ __device__ __forceinline__ void select_body(const Dev& d, int cur, int no_grow, 
         __syncthreads();
         // h of the appended atoms (the order of the proposal's list is not the candidates')
         const int qp = sh.qsel;
-        const int* Sp = d.S + (size_t)i * d.smax;
+        int* Sp = d.S + (size_t)i * d.smax;
+        uint32_t* mw = d.mask + (size_t)i * d.mw;
+        for (int t = tid; t < qp; t += blockDim.x) {
+            const int j = t < nv ? __float_as_int(sh.sc[SEL_KCAP / 2 + t])
+                                 : (int)(0xffffffffu - (unsigned)(sh.key[t - nv] & 0xffffffffull));
+            if (MPL_OOB(j < 0 || j >= m || ss + t >= d.smax, 502)) continue;
+            Sp[ss + t] = j;
+            d.xS[(size_t)i * d.smax + ss + t] = 0.f;
+            atomicOr(mw + (j >> 5), 1u << (j & 31));
+        }
+        __syncthreads();
         for (int a = warp; a < qp; a += nwarps) {
             float c, h;
             warp_doth_f32(d.A32 + (size_t)Sp[ss + a] * n, r32, b32, n, lane, &c, &h);
@@ -1133,16 +1168,6 @@ __device__ __forceinline__ void select_body(const Dev& d, int cur, int no_grow, 
             }
             if (d.explore) d.explore[i] = q > d.rho ? q : 0;  // prune to rho after the master problem
             if (q > 0) {
-                int* Si = d.S + (size_t)i * d.smax;
-                float* xi = d.xS + (size_t)i * d.smax;
-                uint32_t* mw = d.mask + (size_t)i * d.mw;
-                for (int a = 0; a < q; ++a) {
-                    const int j = (int)(0xffffffffu - (unsigned)(sh.key[a] & 0xffffffffull));
-                    if (MPL_OOB(j < 0 || j >= m || ss + a >= d.smax, 503)) break;
-                    Si[ss + a] = j;
-                    xi[ss + a] = 0.f;  // warm start: new entries at zero (Alg. 1)
-                    mw[j >> 5] |= 1u << (j & 31);
-                }
                 d.ssize[i] = ss + q;
                 d.snew[i] = q;
                 d.finalized[i] = 0;
@@ -1169,6 +1194,18 @@ __device__ __forceinline__ void select_body(const Dev& d, int cur, int no_grow, 
     // h of the appended atoms: a violator's rank among the sorted keys is its position after ss
     const int qs = sh.qsel;
     if (qs > 0) {
+        // the atoms appended in key order, a thread each (one thread's read-modify-writes of the
+        // membership words were a chain of global round trips)
+        int* Si = d.S + (size_t)i * d.smax;
+        float* xi = d.xS + (size_t)i * d.smax;
+        uint32_t* mw = d.mask + (size_t)i * d.mw;
+        for (int a = tid; a < qs; a += blockDim.x) {
+            const int j = (int)(0xffffffffu - (unsigned)(sh.key[a] & 0xffffffffull));
+            if (MPL_OOB(j < 0 || j >= m || ss + a >= d.smax, 503)) continue;
+            Si[ss + a] = j;
+            xi[ss + a] = 0.f;  // warm start: new entries at zero (Alg. 1)
+            atomicOr(mw + (j >> 5), 1u << (j & 31));
+        }
         for (unsigned c = tid; c < kc; c += blockDim.x) {
             if (!(sh.sc[c] > 0.f)) continue;
             const unsigned long long kcand = ((unsigned long long)__float_as_uint(sh.sc[c]) << 32) |
