@@ -55,9 +55,9 @@ struct mpl_ctx {
     cudaStream_t fin_st[FIN_SLOTS] = {};  // the exact finish of iteration t runs on fin_st[t % FIN_SLOTS],
                                           // overlapping the master problems and the next iterations
     cudaStream_t main = nullptr;  // graph-mode solves run here (captured streams cannot be the legacy one)
-    cudaStream_t side2 = nullptr; // master problems with blocks outside shared memory, beside the others
+    cudaStream_t side[2] = {};    // master problems with blocks outside registers, beside the others
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
-    cudaEvent_t ev_fork2 = nullptr, ev_join2 = nullptr;
+    cudaEvent_t ev_fork2 = nullptr, ev_join[2] = {};
     HostView* view = nullptr;                     // mapped pinned memory, written by the compaction
     bool in_solve = false;                        // a solve began and did not end (it returned an error)
     cudaEvent_t ev_fin[FIN_SLOTS] = {};           // the exact finish of the last iteration of each slot
@@ -474,9 +474,11 @@ void mpl_destroy(mpl_handle_t h) {
     for (cudaStream_t q : h->fin_st)
         if (q) cudaStreamDestroy(q);
     if (h->main) cudaStreamDestroy(h->main);
-    if (h->side2) cudaStreamDestroy(h->side2);
+    for (cudaStream_t q : h->side)
+        if (q) cudaStreamDestroy(q);
     if (h->ev_fork2) cudaEventDestroy(h->ev_fork2);
-    if (h->ev_join2) cudaEventDestroy(h->ev_join2);
+    for (cudaEvent_t e : h->ev_join)
+        if (e) cudaEventDestroy(e);
     if (h->ev_in) cudaEventDestroy(h->ev_in);
     if (h->ev_out) cudaEventDestroy(h->ev_out);
     for (cudaEvent_t e : h->ev_fin)
@@ -736,18 +738,17 @@ static cudaError_t launch_iteration(mpl_ctx* h, const Dev& d, int t, int act_ub,
     }
     if (pt) pt->end(3, e0, run);
     e0 = pt ? pt->begin_if(5, run) : nullptr;
-    if (apg_split(d, scap)) {
-        // blocks outside shared memory stream on a second stream while the shared-memory
-        // blocks are solved, so that neither class waits for the other's long poles
-        if ((e = cudaEventRecord(h->ev_fork2, run)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(h->side2, h->ev_fork2, 0)) != cudaSuccess) return e;
-        if ((e = launch_apg(d, act_ub, h->sms, scap, h->side2, nl, APG_GLOBAL)) != cudaSuccess) return e;
-        if ((e = cudaEventRecord(h->ev_join2, h->side2)) != cudaSuccess) return e;
-        if ((e = launch_apg(d, act_ub, h->sms, scap, run, nl, APG_SMEM)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(run, h->ev_join2, 0)) != cudaSuccess) return e;
-    } else if ((e = launch_apg(d, act_ub, h->sms, scap, run, nl)) != cudaSuccess) {
-        return e;
+    // each class of block sizes on a stream of its own, so that none waits for another's long poles
+    const int ncls = apg_classes(d, scap);
+    if (ncls > 1 && (e = cudaEventRecord(h->ev_fork2, run)) != cudaSuccess) return e;
+    for (int c = 1; c < ncls; ++c) {
+        if ((e = cudaStreamWaitEvent(h->side[c - 1], h->ev_fork2, 0)) != cudaSuccess) return e;
+        if ((e = launch_apg(d, act_ub, h->sms, scap, h->side[c - 1], nl, c)) != cudaSuccess) return e;
+        if ((e = cudaEventRecord(h->ev_join[c - 1], h->side[c - 1])) != cudaSuccess) return e;
     }
+    if ((e = launch_apg(d, act_ub, h->sms, scap, run, nl, APG_REG)) != cudaSuccess) return e;
+    for (int c = 1; c < ncls; ++c)
+        if ((e = cudaStreamWaitEvent(run, h->ev_join[c - 1], 0)) != cudaSuccess) return e;
     if (d.omega > 1 && (e = launch_smpl_prune(d, act_ub, run, nl)) != cudaSuccess) return e;
     if (pt) pt->end(5, e0, run);
     e0 = pt ? pt->begin_if(6, run) : nullptr;
@@ -801,8 +802,8 @@ static mpl_status_t ensure_streams(mpl_ctx* h) {
     int prio_lo = 0, prio_hi = 0;
     CK(cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi));
     for (cudaStream_t& q : h->fin_st) CK(cudaStreamCreateWithPriority(&q, cudaStreamNonBlocking, prio_lo));
-    CK(cudaStreamCreateWithPriority(&h->side2, cudaStreamNonBlocking, prio_hi));
-    cudaEvent_t* evs[] = {&h->ev_fork2, &h->ev_join2, &h->ev_in, &h->ev_out};
+    for (cudaStream_t& q : h->side) CK(cudaStreamCreateWithPriority(&q, cudaStreamNonBlocking, prio_hi));
+    cudaEvent_t* evs[] = {&h->ev_fork2, &h->ev_join[0], &h->ev_join[1], &h->ev_in, &h->ev_out};
     for (cudaEvent_t* e : evs) CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
     for (cudaEvent_t& e : h->ev_fin) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     CK(cudaStreamCreateWithPriority(&h->main, cudaStreamNonBlocking, prio_hi));

@@ -64,7 +64,8 @@ struct Counters {
     unsigned iters;  // selections completed by this solve
     int apg_n;       // signals in the master-problem list (grow + failed finishes)
     int apg_head;    // work-queue head of the persistent master-problem kernel
-    int apg_head2;   // head of its second queue (blocks streamed from global memory)
+    int apg_head2;   // heads of its other queues: blocks streamed from global memory,
+    int apg_head3;   // blocks in shared memory (apg_head: blocks in registers)
     int err;         // first device-side error code (0 = none)
     int sel_fallback;// candidate-buffer overflows in the selection
     unsigned long long cols;  // signal columns processed by the correlation (all iterations)
@@ -260,13 +261,13 @@ cudaError_t launch_finish(const Dev& d, int slot, int ub, int est, int scap, cud
 // (rows for the GEMM included); the finishes that filled those slots must be complete.
 // ub bounds their signals.
 cudaError_t launch_merge(const Dev& d, int cur, int mask, int ub, cudaStream_t s, int64_t* nl);
-// Master-problem launches: every signal of the work list, or only those whose Gram block fits
-// shared memory, or only those streamed from global memory.
-enum ApgClass : int { APG_ALL = 0, APG_SMEM = 1, APG_GLOBAL = 2 };
-cudaError_t launch_apg(const Dev& d, int ub, int sms, int vcap, cudaStream_t s, int64_t* nl, int cls = APG_ALL);
-// True when blocks up to the bound vcap may outgrow shared memory: the caller then runs an
-// APG_SMEM and an APG_GLOBAL launch (concurrently) instead of one APG_ALL launch.
-bool apg_split(const Dev& d, int vcap);
+// Master-problem launches by the size of a signal's block: in registers (up to APG_REG_S atoms), in
+// shared memory (up to APG_SMEM_S), or streamed from global memory.
+enum ApgClass : int { APG_REG = 0, APG_SMEM = 1, APG_GLOBAL = 2 };
+cudaError_t launch_apg(const Dev& d, int ub, int sms, int vcap, cudaStream_t s, int64_t* nl, int cls);
+// How many of the classes (in their order) blocks up to the bound vcap can reach: the caller
+// launches those, side by side.
+int apg_classes(const Dev& d, int vcap);
 cudaError_t launch_residual(const Dev& d, int ub, cudaStream_t s, int64_t* nl);
 // Algorithm 2: keep the rho explored atoms with the largest |u| (compacts S, x_S, h, G).
 cudaError_t launch_smpl_prune(const Dev& d, int ub, cudaStream_t s, int64_t* nl);
@@ -327,7 +328,8 @@ constexpr int SEL_THREADS = 512;
 // reading, so the option stops here, at the value the GPU tests exercise.
 constexpr int WARM_W_MAX = 64;
 constexpr int SEL_ROWCACHE_ATOMS = 8192;  // score rows up to this length are cached in shared memory
-// Master problem: Gram block kept in shared memory up to this size.
+// Master problem: Gram block kept in registers up to the first size, in shared memory up to the second.
+constexpr int APG_REG_S = 128;
 constexpr int APG_SMEM_S = 200;
 constexpr int APG_THREADS = 256;
 // Exact finish: FP32 factor in shared memory up to this support size (global beyond).

@@ -1294,6 +1294,7 @@ __device__ void compact_body(const Dev& d, int cur, int slot) {
         d.cnt->act_n[cur ^ 1] = base[2];
         d.cnt->apg_head = 0;
         d.cnt->apg_head2 = 0;
+        d.cnt->apg_head3 = 0;
         const unsigned it = ++d.cnt->iters;
         if (d.view) {
             // the host may launch the finish and the next iteration as soon as it sees seq: the

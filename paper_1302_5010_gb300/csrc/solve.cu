@@ -14,6 +14,8 @@
 //   k_smpl_prune  Algorithm 2's pruning of the explored atoms back to rho
 // (the Gram growth read out of Q instead of k_gram is in corr_q.cu.)  The chain's
 // kernels start with pdl_enter (programmatic dependent launch).
+#include <algorithm>
+
 #include "mpl_internal.cuh"
 
 namespace mpl {
@@ -153,7 +155,8 @@ __global__ void __launch_bounds__(256) k_init(Dev d) {
         if (i == 0) {
             d.cnt->act_n[0] = d.p;
             d.cnt->act_n[1] = 0;
-            d.cnt->grow_n = d.cnt->fin_n = d.cnt->apg_n = d.cnt->apg_head = d.cnt->apg_head2 = 0;
+            d.cnt->grow_n = d.cnt->fin_n = d.cnt->apg_n = 0;
+            d.cnt->apg_head = d.cnt->apg_head2 = d.cnt->apg_head3 = 0;
             d.cnt->err = 0;
             d.cnt->sel_fallback = 0;
             d.cnt->cols = 0ull;
@@ -384,45 +387,8 @@ template <int BM, int BN>
 constexpr size_t gram_smem() { return (size_t)GS * (BM + BN) * GPAD * sizeof(float); }
 
 // ------------------------------------------------------------------ APG
-// Gram block in shared memory when s <= gcap (<= APG_SMEM_S), else read from
-// global memory (L2).  Dynamic shared memory: [G gcap^2 | 6 vectors of vcap].
-// y = G x with TPR threads per row (s <= 256 / TPR): lane = row slot + (256 / TPR / 8)
-// ... the TPR threads of a row sit 32 / TPR lanes apart and take every TPR-th
-// column; their partial sums meet in a fixed butterfly.  With the packed leading
-// dimension ld = 32 / TPR (mod 32) the TPR column phases fall in disjoint banks.
-// With h != nullptr the thread that writes y_r also returns its share of the
-// restricted objective, lambda |x_r| + x_r (y_r / 2 - h_r) (summed over its rows).
-template <int TPR>
-__device__ __forceinline__ float gram_mv_split(const float* __restrict__ G, int ld, int s, const float* __restrict__ x,
-                                               float* __restrict__ y, const float* h = nullptr, float lam = 0.f) {
-    constexpr int RW = 32 / TPR;  // rows per warp
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int p = lane / RW, r = warp * RW + (lane % RW);
-    float a = 0.f;
-    if (r < s)
-        for (int c = p; c < s; c += TPR) a = fmaf(G[(size_t)c * ld + r], x[c], a);
-#pragma unroll
-    for (int o = RW; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    float part = 0.f;
-    if (p == 0 && r < s) {
-        y[r] = a;
-        if (h) part = lam * fabsf(x[r]) + x[r] * (0.5f * a - h[r]);
-    }
-    return part;
-}
-
-// Packed leading dimension of an s x s block for gram_mv_split (see above).
-__host__ __device__ __forceinline__ int apg_ld(int s) {
-    if (s <= 64) return s + ((8 - s) & 31);    // = 8 (mod 32), TPR 4
-    if (s <= 128) return s + ((16 - s) & 31);  // = 16 (mod 32), TPR 2
-    return s;
-}
-
-// Floats reserved for a packed block of up to gcap atoms (padded rows included).
-__host__ __device__ __forceinline__ size_t apg_area(int gcap) {
-    const size_t g = (size_t)gcap, h = (size_t)(gcap < 128 ? gcap : 128);
-    return g * g > h * (h + 32) ? g * g : h * (h + 32);
-}
+// Blocks of more than APG_REG_S atoms: in shared memory when s <= gcap (<= APG_SMEM_S), else streamed
+// from global memory (L2).  Dynamic shared memory: [G gcap^2 | 6 vectors of vcap].
 
 __device__ __forceinline__ float gram_mv(const float* __restrict__ G, int ld, int s, const float* __restrict__ x,
                                          float* __restrict__ y, const float* h = nullptr, float lam = 0.f) {
@@ -596,7 +562,7 @@ __device__ __forceinline__ void block_sum3(float& a, float& b, float& c, float* 
 }
 
 // STREAM: the APG_GLOBAL launch (every block streamed from global memory by warp rows);
-// otherwise blocks in shared memory (or, past gcap, read by the thread-per-row product).
+// otherwise blocks in shared memory.
 template <bool STREAM>
 __global__ void __launch_bounds__(APG_THREADS) k_apg(Dev d, int vcap, int gcap, int cls) {
     pdl_enter();
@@ -605,11 +571,11 @@ __global__ void __launch_bounds__(APG_THREADS) k_apg(Dev d, int vcap, int gcap, 
     const int tid = threadIdx.x;
     const int smax = d.smax;
     if (tid == 0) {
-        float* base = gsm + apg_area(gcap);
+        float* base = gsm + (size_t)gcap * gcap;
         sh.u = base; sh.up = base + vcap; sh.Gu = base + 2 * vcap;
         sh.Gup = base + 3 * vcap; sh.h = base + 4 * vcap; sh.v = base + 5 * vcap;
     }
-    int* head = cls == APG_GLOBAL ? &d.cnt->apg_head2 : &d.cnt->apg_head;
+    int* head = cls == APG_GLOBAL ? &d.cnt->apg_head2 : &d.cnt->apg_head3;
     for (;;) {
         if (tid == 0) sh.item = atomicAdd(head, 1);
         __syncthreads();
@@ -618,7 +584,7 @@ __global__ void __launch_bounds__(APG_THREADS) k_apg(Dev d, int vcap, int gcap, 
         const int i = d.list_apg[it];
         const int s = d.ssize[i];
         // a class launch takes only its own signals (the other launch takes the rest)
-        if ((cls == APG_SMEM && s > gcap) || (cls == APG_GLOBAL && s <= APG_SMEM_S)) {
+        if (cls == APG_SMEM ? (s <= APG_REG_S || s > gcap) : s <= APG_SMEM_S) {
             __syncthreads();  // every thread has read sh.item before thread 0 takes the next
             continue;
         }
@@ -631,10 +597,9 @@ __global__ void __launch_bounds__(APG_THREADS) k_apg(Dev d, int vcap, int gcap, 
             __syncthreads();
             continue;
         }
-        const bool insm = s <= gcap;
-        const float* G = insm ? gsm : Gg;
-        const int ld = insm ? apg_ld(s) : smax;
-        if (insm) {
+        const float* G = STREAM ? Gg : gsm;
+        const int ld = STREAM ? smax : s;
+        if (!STREAM) {
             // eight loads in flight per thread before their stores
             for (int e0 = tid; e0 < s * s; e0 += 8 * blockDim.x) {
                 float v[8];
@@ -656,26 +621,16 @@ __global__ void __launch_bounds__(APG_THREADS) k_apg(Dev d, int vcap, int gcap, 
                 }
             }
         }
-        // the block's matrix-vector product: split rows while the block is small, warp rows
-        // streamed as float4 slices from global memory when it is not in shared memory
+        // the block's matrix-vector product: a row per thread in shared memory, warp rows streamed
+        // as float4 slices from global memory
         auto mv = [&](const float* x, float* y) {
-            if constexpr (STREAM) {
-                gram_mv_stream(G, ld, s, x, y);
-            } else {
-                if (insm && s <= 64) gram_mv_split<4>(G, ld, s, x, y);
-                else if (insm && s <= 128) gram_mv_split<2>(G, ld, s, x, y);
-                else gram_mv(G, ld, s, x, y);
-            }
+            if constexpr (STREAM) gram_mv_stream(G, ld, s, x, y);
+            else gram_mv(G, ld, s, x, y);
         };
         // y = G x and this thread's share of the restricted objective at x
         auto mvF = [&](const float* x, float* y) -> float {
-            if constexpr (STREAM) {
-                return gram_mv_stream(G, ld, s, x, y, sh.h, lam);
-            } else {
-                if (insm && s <= 64) return gram_mv_split<4>(G, ld, s, x, y, sh.h, lam);
-                if (insm && s <= 128) return gram_mv_split<2>(G, ld, s, x, y, sh.h, lam);
-                return gram_mv(G, ld, s, x, y, sh.h, lam);
-            }
+            if constexpr (STREAM) return gram_mv_stream(G, ld, s, x, y, sh.h, lam);
+            else return gram_mv(G, ld, s, x, y, sh.h, lam);
         };
         float* xi = d.xS + (size_t)i * smax;
         float* ritz = d.ritz + (size_t)i * smax;
@@ -833,7 +788,7 @@ __global__ void __launch_bounds__(APG_THREADS) k_apg(Dev d, int vcap, int gcap, 
             const unsigned long long ss = (unsigned long long)s * (unsigned long long)s;
             const unsigned long long nmv = (unsigned long long)(npow + 1 + iters);
             atomicAdd(&d.cnt->apg_elems, ss * nmv);
-            atomicAdd(&d.cnt->apg_gl_elems, insm ? ss : ss * nmv);
+            atomicAdd(&d.cnt->apg_gl_elems, STREAM ? ss * nmv : ss);
             // early stopping, eq. (stop_con): decrease of f over this outer iteration's
             // master problem (F0 is f at x^{t-1}, new entries at zero)
             if (d.early && d.stop_eps >= 0.f && d.snew[i] > 0 &&
@@ -841,6 +796,248 @@ __global__ void __launch_bounds__(APG_THREADS) k_apg(Dev d, int vcap, int gcap, 
                 d.early[i] = 1;
         }
         __syncthreads();
+    }
+}
+
+// ------------------------------------------------------------------ APG, blocks in registers
+// The same master problem for blocks of at most APG_REG_S atoms, with the Gram block in registers.
+// With the block in shared memory an iteration took 3300 cycles at 85 atoms: every product reads
+// the whole block from shared memory (one chain of dependent loads and FMAs per row), and
+// so do its five vectors.  Here thread (row r, half h) keeps NC entries of row r (the float4
+// column groups 8 k + 4 h) and row r's entries of the vectors; only the product's operand
+// goes through shared memory, where a warp reads it as broadcast float4, and an iteration
+// has two barriers.  WARP: blocks of at most 32 atoms, a row per lane and a signal per
+// warp, no block barrier at all.  Face-shaped batch (2048 signals, 85 atoms and 556 iterations a
+// signal): 8.1 -> 3.0 ms in master problems; 256 signals on 1024 x 8192: 0.10 -> 0.06 ms.
+// Rows and columns past s are zero, so they add nothing to any sum.
+template <int NC, bool WARP>
+struct ApgReg {
+    static constexpr int ROWS = WARP ? 32 : 2 * NC;
+    static constexpr int NT = WARP ? 32 : 2 * ROWS;  // threads per signal
+    static constexpr int NWARP = NT / 32;
+};
+constexpr int APG_WARPS = 4;  // signals per CTA of the warp variant
+
+// Shared memory of one signal's group of threads (x is read as float4: aligned, also as an array
+// element).
+struct alignas(16) ApgRegShared {
+    float x[APG_REG_S];
+    float red[3][8];
+    int item;
+};
+
+static_assert(sizeof(ApgRegShared) % 16 == 0 && offsetof(ApgRegShared, x) == 0, "float4 reads of x");
+
+template <int NC, bool WARP>
+__device__ void apg_reg_signal(const Dev& d, int i, int tid, ApgRegShared& sh) {
+    using T = ApgReg<NC, WARP>;
+    const int lane = tid & 31, warp = tid >> 5;
+    const int r = WARP ? tid : tid >> 1, h = WARP ? 0 : (tid & 1);
+    constexpr int CG = WARP ? 4 : 8;  // columns from one of this thread's float4 groups to its next
+    const int s = d.ssize[i], smax = d.smax;
+    const float lam = d.lam[i], eps = d.eps[i];
+    const float* Gg = d.G + (size_t)i * smax * smax;
+    const bool own = r < s;          // (both halves of a row hold its vector entries)
+    const bool lead = own && h == 0; // ... and the first one counts them
+    auto sync = [&]() {
+        if (WARP) __syncwarp();
+        else __syncthreads();
+    };
+    // sums over the rows, the same in every thread; a barrier separates two calls' use of red
+    auto sum3 = [&](float& a, float& b, float& c) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, o);
+            b += __shfl_xor_sync(0xffffffffu, b, o);
+            c += __shfl_xor_sync(0xffffffffu, c, o);
+        }
+        if (WARP) return;
+        if (lane == 0) { sh.red[0][warp] = a; sh.red[1][warp] = b; sh.red[2][warp] = c; }
+        __syncthreads();
+        a = b = c = 0.f;
+#pragma unroll
+        for (int w = 0; w < T::NWARP; ++w) { a += sh.red[0][w]; b += sh.red[1][w]; c += sh.red[2][w]; }
+    };
+    auto sum = [&](float a) -> float {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (WARP) return a;
+        if (lane == 0) sh.red[0][warp] = a;
+        __syncthreads();
+        a = 0.f;
+#pragma unroll
+        for (int w = 0; w < T::NWARP; ++w) a += sh.red[0][w];
+        return a;
+    };
+    // the block: every load in flight at once
+    float4 g[NC / 4];
+    const float* grow = Gg + (size_t)(own ? r : 0) * smax;
+    if ((smax & 3) == 0) {
+#pragma unroll
+        for (int k = 0; k < NC / 4; ++k) {
+            const int c = CG * k + 4 * h;
+            g[k] = own && c < s ? __ldg(reinterpret_cast<const float4*>(grow + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int k = 0; k < NC / 4; ++k) {  // (entries past s are left over from larger sets)
+            const int c = CG * k + 4 * h;
+            if (c + 1 >= s) g[k].y = 0.f;
+            if (c + 2 >= s) g[k].z = 0.f;
+            if (c + 3 >= s) g[k].w = 0.f;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < NC / 4; ++k) {
+            const int c = CG * k + 4 * h;
+            g[k].x = own && c < s ? __ldg(grow + c) : 0.f;
+            g[k].y = own && c + 1 < s ? __ldg(grow + c + 1) : 0.f;
+            g[k].z = own && c + 2 < s ? __ldg(grow + c + 2) : 0.f;
+            g[k].w = own && c + 3 < s ? __ldg(grow + c + 3) : 0.f;
+        }
+    }
+    // (G x)_r of the vector whose entries the rows pass; ends without a barrier
+    auto mv = [&](float x) -> float {
+        if (h == 0) sh.x[r] = x;
+        sync();
+        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+        for (int k = 0; k < NC / 4; ++k) {
+            const float4 v = *reinterpret_cast<const float4*>(&sh.x[CG * k + 4 * h]);
+            a0 = fmaf(g[k].x, v.x, a0);
+            a1 = fmaf(g[k].y, v.y, a1);
+            a2 = fmaf(g[k].z, v.z, a2);
+            a3 = fmaf(g[k].w, v.w, a3);
+        }
+        float y = (a0 + a1) + (a2 + a3);
+        if (!WARP) y += __shfl_xor_sync(0xffffffffu, y, 1);
+        return y;
+    };
+    float* xi = d.xS + (size_t)i * smax;
+    float* ritz = d.ritz + (size_t)i * smax;
+    const int prev = s - d.snew[i];  // ritz vector valid for the first `prev` entries
+    const bool warm = prev > 0 && d.outer[i] > 1;
+    float u = own ? xi[r] : 0.f;
+    const float hv = own ? d.h[(size_t)i * smax + r] : 0.f;
+    float pv = !own ? 0.f : (r < prev && d.outer[i] > 1 ? ritz[r] : 1.f);
+    // step size: power iteration for lambda_max(G), as in k_apg
+    float theta = 1.f;
+    const int npow = !(lam > 0.f) ? 0 : (warm ? 3 : 8);
+    for (int pi = 0; pi < npow; ++pi) {
+        const float w = mv(pv);
+        if ((pi & 3) == 3 || pi == npow - 1) {
+            float vv = lead ? pv * pv : 0.f, vg = lead ? pv * w : 0.f, gg = lead ? w * w : 0.f;
+            sum3(vv, vg, gg);
+            theta = vv > 0.f ? vg / vv : 1.f;
+            pv = w * (gg > 0.f ? rsqrtf(gg) : 0.f);
+        } else {
+            pv = w;
+        }
+        sync();
+    }
+    if (lead) ritz[r] = pv;
+    float L = fmaxf(1.05f * theta, 1e-30f);
+    // F(u) and G u at the warm start
+    float Gu = mv(u);
+    float up = u, Gup = Gu;
+    float F = sum(lead ? lam * fabsf(u) + u * (0.5f * Gu - hv) : 0.f);
+    const float F0 = F;
+    float t = 1.f, beta = 0.f;
+    int iters = 0, restarts_in_row = 0;
+    if (!(lam > 0.f)) {
+        // lambda = 0: least squares by conjugate gradients from the warm start
+        float res = own ? hv - Gu : 0.f, dir = res;
+        sync();
+        float rr = lead ? res * res : 0.f, hh = lead ? hv * hv : 0.f, z0 = 0.f;
+        sum3(rr, hh, z0);
+        const float stop2 = eps * eps * hh;
+        const int cg_max = min(d.inner_max, 4 * s + 20);
+        for (int k = 0; k < cg_max && rr > stop2; ++k) {
+            sync();
+            const float q = mv(dir);
+            const float pgp = sum(lead ? dir * q : 0.f);
+            if (!(pgp > 0.f)) break;
+            const float alpha = rr / pgp;
+            u += alpha * dir;
+            Gu += alpha * q;
+            res -= alpha * q;
+            sync();
+            const float rn = sum(lead ? res * res : 0.f);
+            const float bcg = rn / rr;
+            rr = rn;
+            dir = res + bcg * dir;
+            ++iters;
+        }
+        sync();
+        F = sum(lead ? u * (0.5f * Gu - hv) : 0.f);
+    }
+    for (int k = 0; lam > 0.f && k < d.inner_max; ++k) {
+        // extrapolate, prox-gradient step (the one product is G u of the new point)
+        const float invL = 1.f / L;
+        const float y = u + beta * (u - up);
+        const float gy = Gu + beta * (Gu - Gup) - hv;
+        const float z = own ? softf(y - gy * invL, lam * invL) : 0.f;
+        const float u0 = u, Gu0 = Gu;
+        if (WARP) __syncwarp();  // (in a block the last sum's barrier follows every read of x)
+        const float Gz = mv(z);
+        const float Fn = sum(lead ? lam * fabsf(z) + z * (0.5f * Gz - hv) : 0.f);
+        ++iters;
+        if (Fn > F) {
+            // function-value restart: stay at the current point, momentum off; a plain step that
+            // still increases F means L was too small
+            const bool genuine = (Fn - F) > 1e-4f * fmaxf(F0 - F, 1e-30f);
+            if (beta == 0.f && genuine) L *= 2.f;
+            up = u0;
+            Gup = Gu0;
+            beta = 0.f;
+            t = 1.f;
+            if (++restarts_in_row >= 3) break;  // stalled at FP32 resolution
+            continue;
+        }
+        up = u0;
+        Gup = Gu0;
+        u = z;
+        Gu = Gz;
+        restarts_in_row = 0;
+        const float dec = F - Fn, tot = F0 - Fn;
+        F = Fn;
+        // relative-decrease stop of eq. (inner)
+        if (tot <= 0.f ? dec <= 0.f : dec <= eps * tot) break;
+        const float tn = 0.5f * (1.f + sqrtf(1.f + 4.f * t * t));
+        beta = (t - 1.f) / tn;
+        t = tn;
+    }
+    if (lead) xi[r] = u;
+    if (tid == 0) {
+        d.inner[i] += iters;
+        const unsigned long long ss = (unsigned long long)s * (unsigned long long)s;
+        atomicAdd(&d.cnt->apg_elems, ss * (unsigned long long)(npow + 1 + iters));
+        atomicAdd(&d.cnt->apg_gl_elems, ss);
+        // early stopping, eq. (stop_con)
+        if (d.early && d.stop_eps >= 0.f && d.snew[i] > 0 &&
+            F0 - F <= d.stop_eps * fabsf((float)d.rho * d.f0[i]))
+            d.early[i] = 1;
+    }
+}
+
+// Persistent CTAs (or warps) over the master-problem list; signals with more than NC's rows (or
+// more than the class takes) are left to the other launches of the iteration.
+template <int NC, bool WARP, int MINB>
+__global__ void __launch_bounds__(WARP ? 32 * APG_WARPS : 4 * NC, MINB) k_apg_reg(Dev d) {
+    pdl_enter();
+    __shared__ __align__(16) ApgRegShared sha[WARP ? APG_WARPS : 1];
+    ApgRegShared& sh = sha[WARP ? threadIdx.x >> 5 : 0];
+    const int tid = WARP ? threadIdx.x & 31 : threadIdx.x;
+    for (;;) {
+        if (tid == 0) sh.item = atomicAdd(&d.cnt->apg_head, 1);
+        if (WARP) __syncwarp();
+        else __syncthreads();
+        const int it = sh.item;
+        if (it >= d.cnt->apg_n) break;
+        const int i = d.list_apg[it];
+        if (d.ssize[i] <= ApgReg<NC, WARP>::ROWS) apg_reg_signal<NC, WARP>(d, i, tid, sh);
+        // every thread has read sh.item (and finished with sh) before the next one is taken
+        if (WARP) __syncwarp();
+        else __syncthreads();
     }
 }
 
@@ -1252,7 +1449,7 @@ extern "C" int mpl_debug_apg_trace(long long* out, int count, int reset) {
 cudaError_t prepare_apg() {
     static bool attr = false;
     if (attr) return cudaSuccess;
-    const int mx = (int)((apg_area(APG_SMEM_S) + 6 * 1024) * sizeof(float));
+    const int mx = (int)(((size_t)APG_SMEM_S * APG_SMEM_S + 6 * 1024) * sizeof(float));
     cudaError_t e = cudaFuncSetAttribute(k_apg<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_apg<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
     if (e == cudaSuccess) attr = true;
@@ -1268,27 +1465,48 @@ static int apg_vcap(const Dev& d, int vcap) {
     return vcap < cap4 ? vcap : cap4;
 }
 
-bool apg_split(const Dev& d, int vcap) { return apg_vcap(d, vcap) > APG_SMEM_S; }
+int apg_classes(const Dev& d, int vcap) {
+    vcap = apg_vcap(d, vcap);
+    return vcap <= APG_REG_S ? 1 : (vcap <= APG_SMEM_S ? 2 : 3);
+}
+
+// The register variants by the bound on |S|: rows of a warp, then 64, 96 and 128 rows (the more
+// rows, the more registers a thread and the fewer CTAs an SM holds).
+template <int NC, bool WARP, int MINB>
+static cudaError_t launch_apg_reg_t(const Dev& d, int ub, int sms, cudaStream_t s) {
+    constexpr int nt = WARP ? 32 * APG_WARPS : 4 * NC;
+    int per_sm = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_apg_reg<NC, WARP, MINB>, nt, 0);
+    if (e != cudaSuccess) return e;
+    const int need = WARP ? (ub + APG_WARPS - 1) / APG_WARPS : ub;
+    const int grid = std::min(sms * std::max(per_sm, 1), need);
+    return launch_chain(k_apg_reg<NC, WARP, MINB>, dim3(grid), dim3(nt), 0, s, d);
+}
 
 cudaError_t launch_apg(const Dev& d, int ub, int sms, int vcap, cudaStream_t s, int64_t* nl, int cls) {
     if (ub <= 0) return cudaSuccess;
     vcap = apg_vcap(d, vcap);
-    cudaError_t ep = prepare_apg();
-    if (ep != cudaSuccess) return ep;
-    // APG_ALL: one launch, blocks up to the bound (at most APG_SMEM_S) in shared memory;
-    // APG_SMEM: the blocks that fit shared memory; APG_GLOBAL: the others, without the block
-    // area, so that several CTAs per SM stream their blocks from L2/HBM
-    const int gcap = cls == APG_GLOBAL ? 0 : (vcap < APG_SMEM_S ? vcap : APG_SMEM_S);
-    const size_t dyn = (apg_area(gcap) + 6 * (size_t)vcap) * sizeof(float);
-    int per_sm = 0;
-    const bool stream = cls == APG_GLOBAL;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, stream ? k_apg<true> : k_apg<false>,
-                                                                  APG_THREADS, dyn);
-    if (e != cudaSuccess) return e;
-    int grid = sms * (per_sm > 0 ? per_sm : 1);
-    if (grid > ub) grid = ub;
-    e = stream ? launch_chain(k_apg<true>, dim3(grid), dim3(APG_THREADS), dyn, s, d, vcap, gcap, cls)
-               : launch_chain(k_apg<false>, dim3(grid), dim3(APG_THREADS), dyn, s, d, vcap, gcap, cls);
+    cudaError_t e;
+    if (cls == APG_REG) {
+        e = vcap <= 32   ? launch_apg_reg_t<32, true, 4>(d, ub, sms, s)
+            : vcap <= 64 ? launch_apg_reg_t<32, false, 5>(d, ub, sms, s)
+            : vcap <= 96 ? launch_apg_reg_t<48, false, 3>(d, ub, sms, s)
+                         : launch_apg_reg_t<64, false, 2>(d, ub, sms, s);
+    } else {
+        if ((e = prepare_apg()) != cudaSuccess) return e;
+        // APG_SMEM: the blocks past the registers that fit shared memory; APG_GLOBAL: the others,
+        // without the block area, so that several CTAs per SM stream their blocks from L2/HBM
+        const bool stream = cls == APG_GLOBAL;
+        const int gcap = stream ? 0 : (vcap < APG_SMEM_S ? vcap : APG_SMEM_S);
+        const size_t dyn = ((size_t)gcap * gcap + 6 * (size_t)vcap) * sizeof(float);
+        int per_sm = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, stream ? k_apg<true> : k_apg<false>, APG_THREADS,
+                                                          dyn);
+        if (e != cudaSuccess) return e;
+        const int grid = std::min(sms * std::max(per_sm, 1), ub);
+        e = stream ? launch_chain(k_apg<true>, dim3(grid), dim3(APG_THREADS), dyn, s, d, vcap, gcap, cls)
+                   : launch_chain(k_apg<false>, dim3(grid), dim3(APG_THREADS), dyn, s, d, vcap, gcap, cls);
+    }
     if (e != cudaSuccess) return e;
     ++*nl;
     return cudaGetLastError();
