@@ -14,6 +14,11 @@
 //   warps 2-5  epilogue: tcgen05.ld of the accumulator (each warp its 32-lane
 //           quarter = 32 atoms), coalesced FP32 stores of the score rows
 //           C[k*m + j], then release the accumulator.
+// A tile past the last whole BN signals is as narrow as its signals: the residual box is the
+// smallest of 64, 128 and BN rows that holds them, and N is their count rounded up to 16.  The
+// active list shrinks from one outer iteration to the next, and a 256-wide tile took its full
+// tensor time for a handful of signals (4096 x 65536 with 2 of 1024 signals active: 350 us where
+// reading the dictionary takes 80).
 // Every mbarrier wait is bounded; on expiry the CTA records DERR_TIMEOUT and
 // drains before it frees its TMEM: the producer waits (bounded) for every
 // stage whose TMA loads it issued, the MMA thread commits to a drain barrier
@@ -52,9 +57,30 @@ struct TcSmem {
     static_assert((2 * STAGES + 5) * 8 + 8 <= 256, "barriers, TMEM slot and abort flag fit their area");
 };
 
+// Tile t of the persistent walk: atom tile *tm, signal tile *tn.  Signal tiles vary fastest (they
+// share the atom tile in L2), rotated by one from each round of the grid to the next, so that
+// the narrow last tile does not always fall to the same CTAs.
+__device__ __forceinline__ void tile_of(int t, int tiles_n, int* tm, int* tn) {
+    *tm = t / tiles_n;
+    const int x = t - *tm * tiles_n;
+    *tn = (x + (*tm * tiles_n) / (int)gridDim.x) % tiles_n;
+}
+
+// Rows of the residual box of a tile with rem signals left, and the MMA's N.
+template <int BN>
+__device__ __forceinline__ int box_of(int rem) {
+    if (BN > 64 && rem <= 64) return 64;
+    if (BN > 128 && rem <= 128) return 128;
+    return BN;
+}
+template <int BN>
+__device__ __forceinline__ int n_of(int rem) { return min(BN, (rem + 15) & ~15); }
+
+// tm64, tm128, tmR: the residual rows in boxes of 64, 128 and BN rows.
 template <int BN, int STAGES>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-    k_corr_bf16(Dev d, int cur, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmR) {
+    k_corr_bf16(Dev d, int cur, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tm64,
+                const __grid_constant__ CUtensorMap tm128, const __grid_constant__ CUtensorMap tmR) {
     pdl_enter();
     using L = TcSmem<BN, STAGES>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -106,14 +132,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             uint32_t ph = 0;
             uint32_t armed = 0, armed_par = 0;  // stages with loads issued, and the phase they complete
             for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
-                const int tm = t / tiles_n, tn = t - tm * tiles_n;
+                int tm, tn;
+                tile_of(t, tiles_n, &tm, &tn);
+                const int bw = box_of<BN>(act_n - tn * BN);
+                const CUtensorMap* map = bw == BN ? &tmR : (bw == 64 ? &tm64 : &tm128);
                 for (int kb = 0; kb < nk; ++kb) {
                     if (!mbar_wait(&empty[stage], ph ^ 1u, abort_flag)) { give_up(); break; }
                     uint8_t* sa = base + stage * L::STAGE_BYTES;
                     uint8_t* sb = sa + L::A_BYTES;
-                    mbar_expect_tx(&full[stage], L::STAGE_BYTES);
+                    mbar_expect_tx(&full[stage], L::A_BYTES + (uint32_t)bw * (TC_BK * 2));
                     tma_load_2d(sa, &tmA, &full[stage], kb * TC_BK, tm * TC_BM);
-                    tma_load_2d(sb, &tmR, &full[stage], kb * TC_BK, tn * BN);
+                    tma_load_2d(sb, map, &full[stage], kb * TC_BK, tn * BN);
                     armed |= 1u << stage;
                     armed_par = (armed_par & ~(1u << stage)) | (ph << stage);
                     if (++stage == STAGES) { stage = 0; ph ^= 1u; }
@@ -128,7 +157,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(TC_BM, BN);
             int stage = 0, it = 0;
             uint32_t ph = 0;
             for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x, ++it) {
@@ -136,6 +164,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 const uint32_t aph = (uint32_t)((it >> 1) & 1);
                 if (!mbar_wait(&tempty[acc], aph ^ 1u, abort_flag)) { give_up(); break; }
                 fence_after();
+                int tm, tn;
+                tile_of(t, tiles_n, &tm, &tn);
+                const uint32_t idesc = idesc_bf16(TC_BM, n_of<BN>(act_n - tn * BN));
                 const uint32_t dt = tmem + (uint32_t)(acc * BN);
                 bool ok = true;
                 for (int kb = 0; kb < nk; ++kb) {
@@ -167,7 +198,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const int q = warp & 3;
         int it = 0;
         for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x, ++it) {
-            const int tm = t / tiles_n, tn = t - tm * tiles_n;
+            int tm, tn;
+            tile_of(t, tiles_n, &tm, &tn);
+            const int ncol = n_of<BN>(act_n - tn * BN);
             const int acc = it & 1;
             const uint32_t aph = (uint32_t)((it >> 1) & 1);
             bool ok = true;
@@ -178,7 +211,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             const int atom = tm * TC_BM + q * 32 + lane;
             const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
 #pragma unroll 1
-            for (int c0 = 0; c0 < BN; c0 += 16) {
+            for (int c0 = 0; c0 < ncol; c0 += 16) {
                 float v[16];
                 tmem_ld16(tbase + (uint32_t)c0, v);
                 const int sig0 = tn * BN + c0;
@@ -255,7 +288,7 @@ cudaError_t launch_bn(const Dev& d, int cur, const CUtensorMap* maps, int act_n_
     const int tiles = ((d.m + TC_BM - 1) / TC_BM) * ((act_n_ub + BN - 1) / BN);
     const int grid = tiles < sms ? tiles : sms;
     return launch_chain(k_corr_bf16<BN, TcStages<BN>::v>, dim3(grid), dim3(TC_THREADS), (size_t)L::TOTAL, s, d, cur,
-                        maps[0], maps[1 + bn_slot(BN)]);
+                        maps[0], maps[1], maps[2], maps[1 + bn_slot(BN)]);
 }
 
 }  // namespace
