@@ -17,18 +17,16 @@
 // A^T r: these O(n|P|) sums run in double-FP32 arithmetic (error-free
 // products and sums via FMA, ~2^-44 relative) on the FP32 pipe, since GB300's
 // FP64 rate is a small fraction of its FP32 rate.  The factor is FP32 (the
-// refinement with exact residuals restores full accuracy), updated in place when
-// an atom leaves or joins P; an FP64 factor, and then an exactly recomputed Gram
-// block, take over when the refinement stops contracting.  The certified KKT
+// refinement with exact residuals restores full accuracy); an FP64 factor, and then an
+// exactly recomputed Gram block, take over when the refinement stops contracting.  The certified KKT
 // violation on S and the exact residual (FP32 hi/lo pair and FP64) are stored;
 // the next worst-case analysis certifies the atoms outside S (eq. 8).
 //
 // One CTA per signal (256 threads, two CTAs per SM; 512 when the shared-memory
 // layout allows only one).  Shared memory is sized by the host from its bound on
 // |S|; the FP32 factor lives in shared memory when the bound fits there at two
-// CTAs per SM (panel Cholesky), else in the signal's global workspace (tiled
-// Cholesky staged through shared memory); the FP64 factor always uses the
-// workspace.
+// CTAs per SM, else in the signal's global workspace (its panels staged through
+// shared memory either way); the FP64 factor always uses the workspace.
 #include "mpl_internal.cuh"
 
 namespace mpl {
@@ -123,15 +121,13 @@ __device__ __forceinline__ double bsum(double v, double* red) {
 
 
 
-// Blocked right-looking Cholesky by the whole CTA, panels of W columns: one
-// thread factors the W x W diagonal block, the threads take the panel's rows
+// Right-looking Cholesky by the whole CTA, panels of W columns (the FP64 fallback, in global
+// memory): one thread factors the W x W diagonal block, the threads take the panel's rows
 // below it, then the trailing lower triangle gets the rank-W update with its
-// elements spread evenly over the CTA.  Three CTA barriers per panel.  With the
-// factor in global memory (stage != null) the panel is kept in shared memory
-// and wide panels (fewer passes over the trailing triangle) pay off.
+// elements spread evenly over the CTA.  Three CTA barriers per panel.
 // Returns 0 or -1 (non-positive pivot); flag likewise.
 template <typename T, int W>
-__device__ __noinline__ int chol_panel(T* M, int ld, int np, T* rdiag, int* flag, T* stage = nullptr) {
+__device__ __noinline__ int chol_panel(T* M, int ld, int np, T* rdiag, int* flag) {
     const int tid = threadIdx.x, nt = blockDim.x;
     // (r', c') of this thread's first TPOS elements of any trailing triangle (the
     // row-major enumeration does not depend on the triangle's size)
@@ -182,7 +178,6 @@ __device__ __noinline__ int chol_panel(T* M, int ld, int np, T* rdiag, int* flag
                     for (int q = 0; q < k; ++q) v -= l[q] * Rk[q];
                     l[k] = v * rdiag[j + k];
                     Rr[k] = l[k];
-                    if (stage) stage[(size_t)r * W + k] = l[k];
                 }
             }
         }
@@ -191,40 +186,6 @@ __device__ __noinline__ int chol_panel(T* M, int ld, int np, T* rdiag, int* flag
         // the first elements of a thread reuse the positions worked out before the loop
         const int b0 = j + w, nr = np - b0;
         const int tot = nr * (nr + 1) / 2;
-        if (stage) {
-            // factor in global memory: the panel comes from shared memory and each
-            // thread keeps four element loads in flight before its stores
-            for (int e0 = tid; e0 < tot; e0 += 4 * nt) {
-                int rr4[4], cc4[4];
-                T a4[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int e = e0 + u * nt;
-                    rr4[u] = -1;
-                    if (e < tot) {
-                        int rr = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-                        while ((rr + 1) * (rr + 2) / 2 <= e) ++rr;
-                        while (rr * (rr + 1) / 2 > e) --rr;
-                        rr4[u] = b0 + rr;
-                        cc4[u] = b0 + (e - rr * (rr + 1) / 2);
-                        a4[u] = M[(size_t)rr4[u] * ld + cc4[u]];
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (rr4[u] < 0) continue;
-                    const T* Lr = stage + (size_t)rr4[u] * W;
-                    const T* Lc = stage + (size_t)cc4[u] * W;
-                    T acc = a4[u];
-#pragma unroll
-                    for (int k = 0; k < W; ++k)
-                        if (k < w) acc -= Lr[k] * Lc[k];
-                    M[(size_t)rr4[u] * ld + cc4[u]] = acc;
-                }
-            }
-            __syncthreads();
-            continue;
-        }
         for (int e = tid, k8 = 0; e < tot; e += nt, ++k8) {
             int rr, cc;
             if (k8 < TPOS) {
@@ -249,29 +210,6 @@ __device__ __noinline__ int chol_panel(T* M, int ld, int np, T* rdiag, int* flag
     }
     if (tid == 0) *flag = 0;
     return 0;
-}
-
-// (L L^T) v = v by one warp, dot-product form (lanes split each sum).
-template <typename T>
-__device__ void solve_warp(const T* M, int ld, int np, const T* rdiag, T* v) {
-    const int lane = threadIdx.x & 31;
-    for (int j = 0; j < np; ++j) {  // forward: L y = v
-        const T* Lj = M + (size_t)j * ld;
-        T acc = T(0);
-        for (int q = lane; q < j; q += 32) acc += Lj[q] * v[q];
-#pragma unroll
-        for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) v[j] = (v[j] - acc) * rdiag[j];
-        __syncwarp();
-    }
-    for (int j = np - 1; j >= 0; --j) {  // backward: L^T x = y
-        T acc = T(0);
-        for (int q = j + 1 + lane; q < np; q += 32) acc += M[(size_t)q * ld + j] * v[q];
-#pragma unroll
-        for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) v[j] = (v[j] - acc) * rdiag[j];
-        __syncwarp();
-    }
 }
 
 // (L L^T) v = v by one warp for np <= 64, column sweeps with the right-hand
@@ -306,29 +244,17 @@ __device__ void solve_warp_reg(const T* M, int ld, int np, const T* rdiag, T* v)
 // block with the right-hand side in registers, then all threads apply the block to
 // the remaining unknowns (rows of L below it going forward, its columns going back).
 template <typename T>
-__device__ void fwd_cta(const T* M, int ld, int np, const T* rdiag, T* v, T* scr = nullptr) {
+__device__ void solve_cta(const T* M, int ld, int np, const T* rdiag, T* v) {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
     for (int b0 = 0; b0 < np; b0 += 32) {  // forward: L y = v
         const int bw = min(32, np - b0);
-        // the diagonal block: from M, or (a factor in global memory) from a shared-memory
-        // copy, so that warp 0's dependent chain waits on shared memory, not on L2
         const T* D = M + (size_t)b0 * ld + b0;
-        int dld = ld;
-        if (scr) {
-            for (int e = tid; e < bw * bw; e += nt) {
-                const int r = e / bw, c = e - r * bw;
-                if (c < r) scr[r * 33 + c] = D[(size_t)r * ld + c];
-            }
-            __syncthreads();
-            D = scr;
-            dld = 33;
-        }
         if (tid < 32) {
             T y = lane < bw ? v[b0 + lane] : T(0);
             for (int j = 0; j < bw; ++j) {
                 const T yj = __shfl_sync(0xffffffffu, y, j) * rdiag[b0 + j];
                 if (lane == j) y = yj;
-                if (lane > j && lane < bw) y -= D[(size_t)lane * dld + j] * yj;
+                if (lane > j && lane < bw) y -= D[(size_t)lane * ld + j] * yj;
             }
             if (lane < bw) v[b0 + lane] = y;
         }
@@ -342,33 +268,15 @@ __device__ void fwd_cta(const T* M, int ld, int np, const T* rdiag, T* v, T* scr
         }
         __syncthreads();
     }
-}
-
-// scr: null, or 32 x 33 elements of shared memory for the diagonal blocks (worth it
-// when M is in global memory).
-template <typename T>
-__device__ void solve_cta(const T* M, int ld, int np, const T* rdiag, T* v, T* scr = nullptr) {
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-    fwd_cta(M, ld, np, rdiag, v, scr);
     for (int b1 = np; b1 > 0; b1 -= 32) {  // backward: L^T x = y
         const int b0 = max(0, b1 - 32), bw = b1 - b0;
         const T* D = M + (size_t)b0 * ld + b0;
-        int dld = ld;
-        if (scr) {
-            for (int e = tid; e < bw * bw; e += nt) {
-                const int r = e / bw, c = e - r * bw;
-                if (c < r) scr[r * 33 + c] = D[(size_t)r * ld + c];
-            }
-            __syncthreads();
-            D = scr;
-            dld = 33;
-        }
         if (tid < 32) {
             T y = lane < bw ? v[b0 + lane] : T(0);
             for (int j = bw - 1; j >= 0; --j) {
                 const T xj = __shfl_sync(0xffffffffu, y, j) * rdiag[b0 + j];
                 if (lane == j) y = xj;
-                if (lane < j) y -= D[(size_t)j * dld + lane] * xj;
+                if (lane < j) y -= D[(size_t)j * ld + lane] * xj;
             }
             if (lane < bw) v[b0 + lane] = y;
         }
@@ -383,7 +291,7 @@ __device__ void solve_cta(const T* M, int ld, int np, const T* rdiag, T* v, T* s
     }
 }
 
-// Block version: warp 0 runs the sweeps (each sum is split over its lanes).
+// The FP64 solve: one warp for small supports, else the CTA.
 template <typename T>
 __device__ void solve_block(const T* M, int ld, int np, const T* rdiag, T* v) {
     if (np > 64) {
@@ -394,137 +302,252 @@ __device__ void solve_block(const T* M, int ld, int np, const T* rdiag, T* v) {
     __syncthreads();
 }
 
-// Factor of G_PP: FP32 in shared memory (the Gram block itself is only
+// Factor of G_PP: FP32, in shared memory where it fits (the Gram block itself is only
 // FP32-accurate; refinement with exact residuals recovers full accuracy), or
 // FP64 in the global workspace when FP32 refinement stagnates.  Every thread
 // of the CTA returns the same result.
-constexpr int FAC_TILE_W = 16;  // panel width of the tiled factorisation (factor in global memory)
+constexpr int FAC_W = 16;  // block width of the FP32 factorisation
 
-// Floats of shared-memory staging for a global-memory factor of up to scap rows: the
-// panel (FAC_TILE_W x scap rounded up to the 64-row tiles), its diagonal block, slack.
+// Floats of shared-memory staging for a factor of up to scap rows: the k-major panel
+// (fac_ps of at most scap - FAC_W rows, FAC_W columns) and the slack to align it.
 __host__ __device__ inline int fac_stage_floats(int scap) {
-    return FAC_TILE_W * ((scap + 63) / 64) * 64 + FAC_TILE_W * (FAC_TILE_W + 1) + 16;
+    return FAC_W * ((scap + 63) / 64) * 64 + FAC_W * (FAC_W + 1) + 16;
+}
+// Entries of an FP32 vector on the support: whole blocks.
+__host__ __device__ inline int fac_vec(int scap) { return (scap + FAC_W - 1) & ~(FAC_W - 1); }
+// Stride of the staged panel: a multiple of 4 (float4 reads) and 4 (mod 32), so that the 16
+// columns of a row go to eight banks.
+__device__ __forceinline__ int fac_ps(int nr) { return ((nr + 31) / 32) * 32 + 4; }
+
+// The FAC_W x FAC_W block at (j0, j0) by the first 256 threads of the CTA, thread (i, j) on one
+// entry: for j <= i of the block (which becomes L), for j > i of the strict lower triangle of
+// the unit factor's inverse, entry (j, i) (the elimination of [A | I]).  L is written over the lower
+// triangle and L^{-1}, transposed, over the upper one, so that the panel below and both sweeps
+// of a solve multiply by the inverse instead of running a chain through the block; rdiag takes
+// 1 / L_kk.  Step k publishes the entries of column k (and, of the inverse, of row k), one barrier
+// each (two buffers in turn); its chain is that barrier, one shared-memory load, a
+// reciprocal and two FMAs, so nothing in it branches (with divergent branches around the loads
+// a step took 520 cycles).
+// w < FAC_W: the last rows are the identity's.  buf: 2 x 2 x FAC_W floats of shared memory.  Every
+// thread returns the same: 0, or 1 when a pivot is not positive.
+__device__ __forceinline__ int fac_diag(float* M, int ld, int j0, int w, float* rdiag, float* buf) {
+    const int tid = threadIdx.x, i = tid >> 4, j = tid & (FAC_W - 1);
+    const bool mine = tid < FAC_W * FAC_W, low = j <= i;
+    const int r = low ? i : j, c = low ? j : i;  // of the block (low), or of the inverse
+    float e = i == j ? 1.f : 0.f;
+    if (mine && low && i < w) e = M[(size_t)(j0 + i) * ld + j0 + j];
+    float pr = 1.f, pc = 1.f;  // the pivots of row r and column c
+    const float* other = buf + (low ? c : FAC_W + c);
+    float* pub = buf + (low ? i : FAC_W + i);
+    int bad = 0;
+#pragma unroll 2
+    for (int k = 0; k < FAC_W; ++k) {
+        const int off = (k & 1) * 2 * FAC_W;
+        if (mine && j == k) pub[off] = e;
+        __syncthreads();
+        const float piv = buf[off + k], a = buf[off + (mine ? r : 0)];
+        float b = mine ? other[off] : 0.f;
+        if (c == k) b = low ? 0.f : 1.f;  // (column k itself is final; the inverse's unit diagonal)
+        float rcp = __fdividef(1.f, piv);
+        rcp = fmaf(rcp, fmaf(-piv, rcp, 1.f), rcp);
+        const bool on = r > k && (low ? c > k : c <= k);
+        e = on ? fmaf(-(a * rcp), b, e) : e;
+        pr = r == k ? piv : pr;
+        pc = c == k ? piv : pc;
+        bad |= !(piv > 0.f);
+    }
+    if (mine && r < w) {
+        // L_ij = a_ij / sqrt(pivot_j);  L^{-1}_rc = (unit inverse) / sqrt(pivot_r), at (c, r)
+        const float q = 1.f / sqrtf(low ? pc : pr);
+        if (i == j) rdiag[j0 + i] = q;
+        M[(size_t)(j0 + i) * ld + j0 + j] = e * q;
+    }
+    return bad;
 }
 
-// Blocked right-looking Cholesky of a factor in global memory, by the CTA, panels of
-// W = FAC_TILE_W columns.  Per panel: the W x W diagonal block is factored by warp 0
-// in shared memory; each thread takes panel rows below it (forward substitution
-// against the block, W values in registers) and writes them to M and, k-major, to the
-// shared staging area; then the trailing lower triangle gets the rank-W update in
-// 64 x 64 tiles, each thread a 4 x 4 register block fed by float4 reads of the staged
-// panel, with the tile's 16 global values loaded before the products.  Per element the
-// trailing triangle is read and written once per W columns (np^3 / (3W) touches in
-// all) instead of once per 4 or 8.  stage: fac_stage_floats(rows) floats, 16-byte
-// aligned.  Returns 0 or -1 (non-positive pivot); flag likewise.
-// (blockDim.x a multiple of 256: each 256 threads take one 64 x 64 tile at a time as
-// 16 x 16 blocks of 4 x 4)
-__device__ __noinline__ int chol_tiled(float* M, int ld, int np, float* rdiag, int* flag, float* stage) {
-    constexpr int W = FAC_TILE_W, DS = W + 1;
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
-    float* D = stage;                 // W x W diagonal block, stride DS
-    // k-major panel PT[k * PS + (r - j1)], 16-byte aligned for the float4 reads
-    float* PT = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(stage + W * DS) + 15) & ~(uintptr_t)15);
-    const int ty = (tid & 255) >> 4, tx = tid & 15;  // 16 x 16 threads of 4 x 4 blocks per tile
-    const int sub = tid >> 8, nsub = nt >> 8;        // tiles in flight at once
-    for (int j0 = 0; j0 < np; j0 += W) {
-        const int w = min(W, np - j0), j1 = j0 + w, nr = np - j1;
-        const int PS = ((nr + 63) / 64) * 64;
-        for (int e = tid; e < w * w; e += nt) {
-            const int r = e / w, c = e - r * w;
-            if (c <= r) D[r * DS + c] = M[(size_t)(j0 + r) * ld + j0 + c];
-        }
+// Entries (k, q), q < FAC_W, of the inverse of the diagonal block at j0 (zero for q > k), or with TR
+// entries (q, k) (zero for q < k); bw: the block's rows.  All loads are issued together.
+template <bool TR>
+__device__ __forceinline__ void fac_inv_row(const float* M, int ld, int j0, int bw, const float* rdiag, int k,
+                                            float (&iv)[FAC_W]) {
+    const float dk = rdiag[j0 + min(k, bw - 1)];
+#pragma unroll
+    for (int q = 0; q < FAC_W; ++q) {
+        const int qq = min(q, bw - 1), kk = min(k, bw - 1);
+        iv[q] = TR ? M[(size_t)(j0 + kk) * ld + j0 + qq] : M[(size_t)(j0 + qq) * ld + j0 + kk];
+    }
+#pragma unroll
+    for (int q = 0; q < FAC_W; ++q) {
+        const bool in = k < bw && q < bw && (TR ? q > k : q < k);
+        iv[q] = in ? iv[q] : (q == k && k < bw ? dk : 0.f);
+    }
+}
+
+// Blocked factorisation G = W D W^T of an FP32 block by the CTA, blocks of FAC_W columns: D the
+// diagonal blocks L L^T (fac_diag keeps L^{-1}), W unit lower triangular by blocks.  The panel
+// below a block is A21 L^{-T} (staged k-major for the trailing update, in 4 x 4 register blocks
+// fed by float4 reads) times L^{-1}, which is W and what M keeps: a solve's sweeps then only
+// subtract products with W, and no chain through a diagonal block sits between two of them.
+// SM: M is in shared memory.  stage: fac_stage_floats(rows) floats of shared memory.  Returns 0 or -1
+// (non-positive pivot).
+template <bool SM>
+__device__ __noinline__ int chol_blocked(float* M, int ld, int np, float* rdiag, float* stage) {
+    __shared__ float buf[4 * FAC_W];
+    if (SM) __builtin_assume(__isShared(M));
+    __builtin_assume(__isShared(rdiag));
+    __builtin_assume(__isShared(stage));
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+    float* PT = stage + ((16u - (unsigned)__cvta_generic_to_shared(stage)) & 15u) / 4u;
+    for (int j0 = 0; j0 < np; j0 += FAC_W) {
+        const int w = min(FAC_W, np - j0), j1 = j0 + w, nr = np - j1;
+        const int PS = fac_ps(nr);
+        const int bad = fac_diag(M, ld, j0, w, rdiag, buf);
         __syncthreads();
-        if (warp == 0) {
-            int bad = 0;
-            for (int k = 0; k < w; ++k) {
-                const float dkk = D[k * DS + k];
-                if (!(dkk > 0.f)) { bad = 1; break; }  // the same value on every lane
-                const float dg = sqrtf(dkk), inv = 1.f / dg;
-                __syncwarp();
-                if (lane == k) { D[k * DS + k] = dg; rdiag[j0 + k] = inv; }
-                if (lane > k && lane < w) D[lane * DS + k] *= inv;
-                __syncwarp();
-                if (lane > k && lane < w) {
-                    const float lk = D[lane * DS + k];
-                    for (int c = k + 1; c <= lane; ++c) D[lane * DS + c] -= lk * D[c * DS + k];
+        if (bad) return -1;
+        if (nr == 0) break;
+        {
+            // lane k of a half-warp forms column k of its row (w == FAC_W here: only the last block
+            // is narrower, and nothing is below it)
+            const int k = lane & (FAC_W - 1), hw = lane >> 4;
+            float iv[FAC_W], it[FAC_W];
+            fac_inv_row<false>(M, ld, j0, FAC_W, rdiag, k, iv);
+            fac_inv_row<true>(M, ld, j0, FAC_W, rdiag, k, it);
+            for (int r0 = 2 * warp; r0 < nr; r0 += 2 * nw) {
+                const int r = r0 + hw;
+                float* e = M + (size_t)(j1 + min(r, nr - 1)) * ld + j0 + k;
+                const float av = *e;
+                float l0 = 0.f, l1 = 0.f;
+#pragma unroll
+                for (int q = 0; q < FAC_W; q += 2) {
+                    l0 = fmaf(__shfl_sync(0xffffffffu, av, (hw << 4) + q), iv[q], l0);
+                    l1 = fmaf(__shfl_sync(0xffffffffu, av, (hw << 4) + q + 1), iv[q + 1], l1);
                 }
-                __syncwarp();
-            }
-            if (lane == 0) *flag = bad;
-        }
-        __syncthreads();
-        if (*flag) return -1;
-        for (int e = tid; e < w * w; e += nt) {
-            const int r = e / w, c = e - r * w;
-            if (c <= r) M[(size_t)(j0 + r) * ld + j0 + c] = D[r * DS + c];
-        }
-        // panel rows below the block
-        for (int r = j1 + tid; r < np; r += nt) {
-            float* Rr = M + (size_t)r * ld + j0;
-            float l[W];
+                const float l = l0 + l1;
+                float w0 = 0.f, w1 = 0.f;
 #pragma unroll
-            for (int k = 0; k < W; ++k) l[k] = k < w ? Rr[k] : 0.f;
-#pragma unroll
-            for (int k = 0; k < W; ++k) {
-                if (k < w) {
-                    float v = l[k];
-#pragma unroll
-                    for (int q = 0; q < k; ++q) v -= l[q] * D[k * DS + q];
-                    l[k] = v * rdiag[j0 + k];
+                for (int q = 0; q < FAC_W; q += 2) {
+                    w0 = fmaf(__shfl_sync(0xffffffffu, l, (hw << 4) + q), it[q], w0);
+                    w1 = fmaf(__shfl_sync(0xffffffffu, l, (hw << 4) + q + 1), it[q + 1], w1);
                 }
-            }
-#pragma unroll
-            for (int k = 0; k < W; ++k) {
-                if (k < w) {
-                    Rr[k] = l[k];
-                    PT[k * PS + (r - j1)] = l[k];
+                if (r < nr) {
+                    *e = w0 + w1;
+                    PT[k * PS + r] = l;
                 }
             }
         }
         __syncthreads();
-        // trailing triangle: 64 x 64 tiles (ti >= tj), element (r, c) with c <= r
-        const int T = (nr + 63) / 64;
-        for (int t = sub; t < T * (T + 1) / 2; t += nsub) {
-            int ti = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
-            while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
-            while (ti * (ti + 1) / 2 > t) --ti;
-            const int tj = t - ti * (ti + 1) / 2;
-            const int rr0 = ti * 64 + ty * 4, cc0 = tj * 64 + tx * 4;  // offsets from j1
+        // trailing triangle: 4 x 4 blocks (ti >= tj), element (r, c) with c <= r
+        const int T = (nr + 3) >> 2;
+        for (int e = tid; e < T * (T + 1) / 2; e += nt) {
+            int ti = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+            while ((ti + 1) * (ti + 2) / 2 <= e) ++ti;
+            while (ti * (ti + 1) / 2 > e) --ti;
+            const int rr = 4 * ti, cc = 4 * (e - ti * (ti + 1) / 2);
             float a[4][4];
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const int r = rr0 + u, c = cc0 + v;
-                    a[u][v] = (r < nr && c <= r) ? M[(size_t)(j1 + r) * ld + j1 + c] : 0.f;
-                }
-            float acc[4][4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
-            for (int k = 0; k < w; ++k) {
-                const float4 x = *reinterpret_cast<const float4*>(PT + k * PS + rr0);
-                const float4 y = *reinterpret_cast<const float4*>(PT + k * PS + cc0);
+                for (int v = 0; v < 4; ++v)  // (clamped: entries past the triangle are not stored)
+                    a[u][v] = M[(size_t)(j1 + min(rr + u, nr - 1)) * ld + j1 + min(cc + v, nr - 1)];
+#pragma unroll 4
+            for (int k = 0; k < FAC_W; ++k) {
+                const float4 x = *reinterpret_cast<const float4*>(PT + k * PS + rr);
+                const float4 y = *reinterpret_cast<const float4*>(PT + k * PS + cc);
                 const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(xs[u], ys[v], acc[u][v]);
+                    for (int v = 0; v < 4; ++v) a[u][v] = fmaf(-xs[u], ys[v], a[u][v]);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const int r = rr0 + u, c = cc0 + v;
-                    if (r < nr && c <= r) M[(size_t)(j1 + r) * ld + j1 + c] = a[u][v] - acc[u][v];
-                }
+                for (int v = 0; v < 4; ++v)
+                    if (rr + u < nr && cc + v <= rr + u) M[(size_t)(j1 + rr + u) * ld + j1 + cc + v] = a[u][v];
         }
         __syncthreads();
     }
     return 0;
 }
 
+// v <- (W D W^T)^{-1} v with the factor of chol_blocked, by the CTA: a forward sweep, the diagonal blocks
+// (a half-warp each, all at once), a backward sweep.  A sweep's step subtracts a block's 16
+// unknowns from the remaining ones, a thread per unknown: one barrier, one round of
+// shared-memory loads (the rows of W are read ahead) and 16 FMAs.  v: shared memory, 16-byte
+// aligned, (np + 15) & ~15 entries readable.
+template <bool SM>
+__device__ __noinline__ void solve_blocked(const float* M, int ld, int np, const float* rdiag, float* v) {
+    if (SM) __builtin_assume(__isShared(M));
+    __builtin_assume(__isShared(rdiag));
+    __builtin_assume(__isShared(v));
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+    auto apply = [&](const float (&l)[FAC_W], int b0) -> float {
+        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+        for (int c = 0; c < FAC_W; c += 4) {
+            const float4 y = *reinterpret_cast<const float4*>(v + b0 + c);
+            a0 = fmaf(l[c], y.x, a0);
+            a1 = fmaf(l[c + 1], y.y, a1);
+            a2 = fmaf(l[c + 2], y.z, a2);
+            a3 = fmaf(l[c + 3], y.w, a3);
+        }
+        return (a0 + a1) + (a2 + a3);
+    };
+    // forward: v_r -= W_rb v_b
+    for (int b0 = 0; b0 + FAC_W < np; b0 += FAC_W) {
+        for (int r0 = b0 + FAC_W; r0 < np; r0 += nt) {
+            const int r = r0 + tid;
+            if (r >= np) continue;
+            float l[FAC_W];
+            const float* Wr = M + (size_t)r * ld + b0;
+#pragma unroll
+            for (int c = 0; c < FAC_W; ++c) l[c] = Wr[c];
+            v[r] -= apply(l, b0);
+        }
+        __syncthreads();
+    }
+    // the diagonal blocks: v_b <- L_b^{-T} L_b^{-1} v_b
+    for (int blk = 2 * warp + (lane >> 4); ; blk += 2 * nw) {
+        const int b0 = blk * FAC_W;
+        // (both half-warps leave together: the shuffles need the whole warp)
+        if ((blk - (lane >> 4)) * FAC_W >= np) break;
+        const int bw = max(1, min(FAC_W, np - b0)), k = lane & (FAC_W - 1), hw = lane & FAC_W;
+        const int bb = min(b0, ((np - 1) / FAC_W) * FAC_W);
+        float iv[FAC_W];
+        fac_inv_row<false>(M, ld, bb, min(bw, np - bb), rdiag, k, iv);
+        const float vk = b0 < np && k < bw ? v[b0 + k] : 0.f;
+        float y0 = 0.f, y1 = 0.f;
+#pragma unroll
+        for (int q = 0; q < FAC_W; q += 2) {
+            y0 = fmaf(iv[q], __shfl_sync(0xffffffffu, vk, hw + q), y0);
+            y1 = fmaf(iv[q + 1], __shfl_sync(0xffffffffu, vk, hw + q + 1), y1);
+        }
+        const float y = y0 + y1;
+        fac_inv_row<true>(M, ld, bb, min(bw, np - bb), rdiag, k, iv);
+        float x0 = 0.f, x1 = 0.f;
+#pragma unroll
+        for (int q = 0; q < FAC_W; q += 2) {
+            x0 = fmaf(iv[q], __shfl_sync(0xffffffffu, y, hw + q), x0);
+            x1 = fmaf(iv[q + 1], __shfl_sync(0xffffffffu, y, hw + q + 1), x1);
+        }
+        if (b0 < np && k < bw) v[b0 + k] = x0 + x1;
+    }
+    // (entries of the last block past np are multiplied by zero below: they must be finite)
+    for (int e = np + tid; e < ((np + FAC_W - 1) & ~(FAC_W - 1)); e += nt) v[e] = 0.f;
+    __syncthreads();
+    // backward: v_c -= sum over the block's rows of W_rc v_r
+    for (int b0 = ((np - 1) / FAC_W) * FAC_W; b0 > 0; b0 -= FAC_W) {
+        const int bw = min(FAC_W, np - b0);
+        for (int c = tid; c < b0; c += nt) {
+            float l[FAC_W];
+            const float* Wc = M + (size_t)b0 * ld + c;
+#pragma unroll
+            for (int q = 0; q < FAC_W; ++q) l[q] = Wc[(size_t)min(q, bw - 1) * ld];
+            v[c] -= apply(l, b0);
+        }
+        __syncthreads();
+    }
+}
 
 struct Factor {
     float* Mf;       // FP32 factor, leading dimension ldf
@@ -532,17 +555,17 @@ struct Factor {
     double* Md;      // FP64 factor (global workspace), leading dimension ldd
     double* rdd;     // reciprocal diagonal for the FP64 factor
     float* vf;       // FP32 right-hand side scratch
-    float* stage;    // staging (fac_stage_floats) for an FP32 factor in global memory, else null
+    float* stage;    // staging of the FP32 factorisation (fac_stage_floats)
     int stage_n;     // floats at stage
     int ldf, ldd;
+    int in_sm;       // the FP32 factor is in shared memory
     int fp64;        // which factor is current
 };
 
 __device__ int factor(Factor& F, int np, int* flag) {
-    if (!F.fp64) {
-        if (F.stage) return chol_tiled(F.Mf, F.ldf, np, F.rdf, flag, F.stage);
-        return chol_panel<float, 4>(F.Mf, F.ldf, np, F.rdf, flag);
-    }
+    if (!F.fp64)
+        return F.in_sm ? chol_blocked<true>(F.Mf, F.ldf, np, F.rdf, F.stage)
+                       : chol_blocked<false>(F.Mf, F.ldf, np, F.rdf, F.stage);
     return chol_panel<double, 4>(F.Md, F.ldd, np, F.rdd, flag);
 }
 
@@ -551,13 +574,8 @@ __device__ void fsolve(const Factor& F, int np, double* v) {
     if (!F.fp64) {
         for (int a = threadIdx.x; a < np; a += blockDim.x) F.vf[a] = (float)v[a];
         __syncthreads();
-        if (np > 64) {
-            // the staging area is free outside factorisations: the diagonal blocks go there
-            solve_cta(F.Mf, F.ldf, np, F.rdf, F.vf, F.stage_n >= 32 * 33 ? F.stage : nullptr);
-        } else {
-            if (threadIdx.x < 32) solve_warp_reg(F.Mf, F.ldf, np, F.rdf, F.vf);
-            __syncthreads();
-        }
+        if (F.in_sm) solve_blocked<true>(F.Mf, F.ldf, np, F.rdf, F.vf);
+        else solve_blocked<false>(F.Mf, F.ldf, np, F.rdf, F.vf);
         for (int a = threadIdx.x; a < np; a += blockDim.x) v[a] = (double)F.vf[a];
         __syncthreads();
         return;
@@ -579,9 +597,6 @@ struct FinShared {
     double red[32];
     int ival[4];
     double dval[4];
-    int fac_np;  // rows of the FP32 factor that match P in its order (-1: rebuild next step)
-    float cs[2]; // rotation of the factor update
-    float rot[2][2];  // rotations of the CTA-wide update, alternating slots
     int cg;      // 1: solves by conjugate gradients on the Gram block (no factor)
     uint64_t cbar[2];  // cluster barriers of a clustered finish (C arrivals per phase; phases alternate)
 };
@@ -601,272 +616,6 @@ __device__ int build_support(int s, FinShared& sh) {
     }
     __syncthreads();
     return sh.ival[1];
-}
-
-// Incremental changes of the FP32 factor of G_PP when the support loses or
-// gains one atom, instead of refactoring: by warp 0 up to FAC_INC_MAX atoms, by the
-// whole CTA above that.
-constexpr int FAC_INC_MAX = 64;
-
-// Drop factor row/column k: the trailing factor absorbs the dropped column by a
-// rank-one update (L33' L33'^T = L33 L33^T + l l^T, rotations by warp 0), then
-// rows and columns after k move up by one; P and the reciprocal diagonal follow.
-__device__ __noinline__ void fac_remove(FinShared& sh, int k, int np) {
-    float* M = sh.F.Mf;
-    const int ld = sh.F.ldf;
-    const int m = np - k - 1;
-    const int tid = threadIdx.x, lane = tid & 31;
-    if (tid < 32) {
-        // lane owns entries lane and lane + 32 of the dropped column below the diagonal
-        float x0 = lane < m ? M[(size_t)(k + 1 + lane) * ld + k] : 0.f;
-        float x1 = lane + 32 < m ? M[(size_t)(k + 33 + lane) * ld + k] : 0.f;
-        for (int j = 0; j < m; ++j) {
-            const int J = k + 1 + j;
-            const float xj = __shfl_sync(0xffffffffu, j < 32 ? x0 : x1, j & 31);
-            const float ljj = M[(size_t)J * ld + J];
-            const float r = sqrtf(ljj * ljj + xj * xj);
-            const float c = r / ljj, sn = xj / ljj;
-            __syncwarp();
-            if (lane == 0) { M[(size_t)J * ld + J] = r; sh.F.rdf[J] = 1.f / r; }
-            if (lane > j && lane < m) {
-                float* L = M + (size_t)(k + 1 + lane) * ld + J;
-                const float ln = (*L + sn * x0) / c;
-                *L = ln;
-                x0 = c * x0 - sn * ln;
-            }
-            if (lane + 32 > j && lane + 32 < m) {
-                float* L = M + (size_t)(k + 33 + lane) * ld + J;
-                const float ln = (*L + sn * x1) / c;
-                *L = ln;
-                x1 = c * x1 - sn * ln;
-            }
-            __syncwarp();
-        }
-    }
-    __syncthreads();
-    // move rows/columns after k by one (each thread stages up to 16 entries of one row)
-    const int r = tid >> 2, cq = tid & 3;
-    float v[16];
-    const bool live = r < np - 1;
-    const int rs = r < k ? r : r + 1;
-#pragma unroll
-    for (int u = 0; u < 16; ++u) {
-        const int c = cq + 4 * u;
-        v[u] = (live && c <= r) ? M[(size_t)rs * ld + (c < k ? c : c + 1)] : 0.f;
-    }
-    float rd = 0.f;
-    int pr = 0;
-    if (tid < np - 1) { rd = sh.F.rdf[tid < k ? tid : tid + 1]; pr = sh.P[tid < k ? tid : tid + 1]; }
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < 16; ++u) {
-        const int c = cq + 4 * u;
-        if (live && c <= r) M[(size_t)r * ld + c] = v[u];
-    }
-    if (tid < np - 1) { sh.F.rdf[tid] = rd; sh.P[tid] = pr; }
-    __syncthreads();
-}
-
-// Append the support atom at position a as the factor's last row: forward
-// substitution L l = G_Pa by warp 0, l_nn = sqrt(G_aa - l^T l).  Returns 0, or
-// -1 when the new pivot is not positive (the caller refactors).
-__device__ __noinline__ int fac_append(FinShared& sh, const float* Gi, int smax, int a, int np) {
-    float* M = sh.F.Mf;
-    const int ld = sh.F.ldf;
-    const int tid = threadIdx.x, lane = tid & 31;
-    if (tid < 32) {
-        const int r0 = lane, r1 = lane + 32;
-        float y0 = r0 < np ? Gi[(size_t)sh.P[r0] * smax + a] : 0.f;
-        float y1 = r1 < np ? Gi[(size_t)sh.P[r1] * smax + a] : 0.f;
-        for (int j = 0; j < np; ++j) {
-            const float yj = __shfl_sync(0xffffffffu, j < 32 ? y0 : y1, j & 31) * sh.F.rdf[j];
-            if (lane == (j & 31)) { if (j < 32) y0 = yj; else y1 = yj; }
-            if (r0 > j && r0 < np) y0 -= M[(size_t)r0 * ld + j] * yj;
-            if (r1 > j && r1 < np) y1 -= M[(size_t)r1 * ld + j] * yj;
-        }
-        float ss = (r0 < np ? y0 * y0 : 0.f) + (r1 < np ? y1 * y1 : 0.f);
-#pragma unroll
-        for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        const float dnn = Gi[(size_t)a * smax + a] - ss;
-        if (r0 < np) M[(size_t)np * ld + r0] = y0;
-        if (r1 < np) M[(size_t)np * ld + r1] = y1;
-        if (lane == 0) {
-            const bool ok = dnn > 0.f;
-            sh.ival[0] = ok ? 0 : 1;
-            if (ok) {
-                const float dg = sqrtf(dnn);
-                M[(size_t)np * ld + np] = dg;
-                sh.F.rdf[np] = 1.f / dg;
-                sh.P[np] = a;
-            }
-        }
-    }
-    __syncthreads();
-    return sh.ival[0] ? -1 : 0;
-}
-
-// Drop factor row/column k of a factor of any size (np <= 4 blockDim.x + 1), by the
-// CTA.  The trailing factor absorbs the dropped column by the same rank-one update as
-// fac_remove: thread t owns trailing rows k + 1 + t + q nt (q < 4) and keeps their
-// entries of the dropped column in registers.  Rotation j (row J = k + 1 + j) is
-// worked out by the owner of row J from its own entries, so one barrier per rotation
-// suffices (two slots alternate); the entries of column J + 1, which rotation j does
-// not touch, are loaded while it runs.  Then rows below k move up by one row and,
-// right of column k, one column left, a few rows at a time (every source read before
-// the barrier that precedes the writes of its chunk, and a destination is never a
-// source of a later chunk); P and the reciprocal diagonal follow.
-__device__ __noinline__ void fac_remove_cta(FinShared& sh, int k, int np) {
-    constexpr int RQ = 4;
-    float* M = sh.F.Mf;
-    const int ld = sh.F.ldf;
-    const int m = np - k - 1;
-    const int tid = threadIdx.x, nt = blockDim.x;
-    float x[RQ], nx[RQ];
-#pragma unroll
-    for (int q = 0; q < RQ; ++q) {
-        const int i = tid + q * nt;
-        x[q] = i < m ? M[(size_t)(k + 1 + i) * ld + k] : 0.f;
-        nx[q] = i < m ? M[(size_t)(k + 1 + i) * ld + k + 1] : 0.f;  // column J of rotation 0
-    }
-    for (int j = 0; j < m; ++j) {
-        const int J = k + 1 + j;
-        float cur[RQ];
-#pragma unroll
-        for (int q = 0; q < RQ; ++q) {
-            cur[q] = nx[q];
-            const int i = tid + q * nt;
-            nx[q] = (i > j && i < m) ? M[(size_t)(k + 1 + i) * ld + J + 1] : 0.f;  // i > j: j + 1 < m
-        }
-        if (tid == j % nt) {
-            const int qo = j / nt;
-            float ljj = 0.f, xj = 0.f;
-#pragma unroll
-            for (int q = 0; q < RQ; ++q)
-                if (q == qo) { ljj = cur[q]; xj = x[q]; }
-            const float r = sqrtf(ljj * ljj + xj * xj);
-            sh.rot[j & 1][0] = r / ljj;
-            sh.rot[j & 1][1] = xj / ljj;
-            M[(size_t)J * ld + J] = r;
-            sh.F.rdf[J] = 1.f / r;
-        }
-        __syncthreads();
-        const float c = sh.rot[j & 1][0], sn = sh.rot[j & 1][1];
-#pragma unroll
-        for (int q = 0; q < RQ; ++q) {
-            const int i = tid + q * nt;
-            if (i > j && i < m) {
-                const float ln = (cur[q] + sn * x[q]) / c;
-                M[(size_t)(k + 1 + i) * ld + J] = ln;
-                x[q] = c * x[q] - sn * ln;
-            }
-        }
-    }
-    __syncthreads();
-    // rows k + 1 .. np - 1 up by one; their columns right of k left by one
-    const int rows = max(1, (8 * nt) / np);
-    for (int r0 = k + 1; r0 < np; r0 += rows) {
-        const int r1 = min(np, r0 + rows);
-        const int tot = (r1 - r0) * np;
-        float v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int e = tid + u * nt;
-            v[u] = 0.f;
-            if (e < tot) {
-                const int r = r0 + e / np, c = e % np;  // destination column c of row r - 1
-                if (c < r) v[u] = M[(size_t)r * ld + (c < k ? c : c + 1)];
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int e = tid + u * nt;
-            if (e < tot) {
-                const int r = r0 + e / np, c = e % np;
-                if (c < r) M[(size_t)(r - 1) * ld + c] = v[u];
-            }
-        }
-        __syncthreads();
-    }
-    float rd[RQ];
-    int pr[RQ];
-#pragma unroll
-    for (int q = 0; q < RQ; ++q) {
-        const int i = k + tid + q * nt;
-        if (i < np - 1) { rd[q] = sh.F.rdf[i + 1]; pr[q] = sh.P[i + 1]; }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < RQ; ++q) {
-        const int i = k + tid + q * nt;
-        if (i < np - 1) { sh.F.rdf[i] = rd[q]; sh.P[i] = pr[q]; }
-    }
-    __syncthreads();
-}
-
-// Append the support atom at position a as row np of a factor of any size, by the
-// CTA: the forward sweep L y = G_Pa in the FP32 scratch vector, l_nn = sqrt(G_aa -
-// y^T y).  Returns 0, or -1 when the new pivot is not positive (the caller refactors).
-__device__ __noinline__ int fac_append_cta(FinShared& sh, const float* Gi, int smax, int a, int np) {
-    float* M = sh.F.Mf;
-    const int ld = sh.F.ldf;
-    float* v = sh.F.vf;
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-    for (int r = tid; r < np; r += nt) v[r] = Gi[(size_t)sh.P[r] * smax + a];
-    __syncthreads();
-    fwd_cta(M, ld, np, sh.F.rdf, v, sh.F.stage_n >= 32 * 33 ? sh.F.stage : nullptr);
-    double ss = 0.0;
-    for (int r = tid; r < np; r += nt) ss += (double)v[r] * (double)v[r];
-#pragma unroll
-    for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    if (lane == 0) sh.red[warp] = ss;
-    __syncthreads();
-    double tot = 0.0;
-    for (int q = 0; q < nw; ++q) tot += sh.red[q];
-    const float dnn = (float)((double)Gi[(size_t)a * smax + a] - tot);
-    const bool ok = dnn > 0.f;
-    if (ok) {
-        for (int r = tid; r < np; r += nt) M[(size_t)np * ld + r] = v[r];
-        if (tid == 0) {
-            const float dg = sqrtf(dnn);
-            M[(size_t)np * ld + np] = dg;
-            sh.F.rdf[np] = 1.f / dg;
-            sh.P[np] = a;
-        }
-    }
-    __syncthreads();
-    return ok ? 0 : -1;
-}
-
-// After atoms of P were zeroed (sign 0): drop them from the FP32 factor, last
-// first, or leave the factor to be rebuilt.
-__device__ void drop_zeroed(FinShared& sh, int np) {
-    if (sh.fac_np < 0 || sh.F.fp64) {
-        __syncthreads();
-        if (threadIdx.x == 0) sh.fac_np = -1;
-        __syncthreads();
-        return;
-    }
-    int cur = np;
-    for (int a = np - 1; a >= 0; --a) {
-        if (sh.sg[sh.P[a]] != 0) continue;
-        if (cur <= FAC_INC_MAX) fac_remove(sh, a, cur);
-        else fac_remove_cta(sh, a, cur);
-        --cur;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) sh.fac_np = cur;
-    __syncthreads();
-}
-
-// The atom at position a joins P: append it to the FP32 factor, or leave the
-// factor to be rebuilt.
-__device__ void join_support(FinShared& sh, const float* Gi, int smax, int a, int np) {
-    const bool ok = sh.fac_np >= 0 && !sh.F.fp64;
-    __syncthreads();
-    const int res = !ok ? -1 : (np < FAC_INC_MAX ? fac_append(sh, Gi, smax, a, np) : fac_append_cta(sh, Gi, smax, a, np));
-    if (threadIdx.x == 0) sh.fac_np = res == 0 ? np + 1 : -1;
-    __syncthreads();
 }
 
 // r = b - A_P x in double-FP32.  Each thread keeps 8 independent chains (8
@@ -1157,31 +906,33 @@ __device__ int exact_factor(FinShared& sh, const float* A, int n, int np) {
 
 // Copy the lower triangle of G_PP into the current factor storage and factor it.
 __device__ void gather_gram(FinShared& sh, const float* Gi, int smax, int np) {
-    // the np x np lower triangle as one flat range of independent loads (row r holds
-    // entries r(r+1)/2 .. r(r+1)/2 + r)
-    const int tot = np * (np + 1) / 2;
-    for (int e0 = threadIdx.x; e0 < tot; e0 += 4 * blockDim.x) {
-        // four loads in flight before the stores (the stores could alias them)
-        float v[4];
-        int rr[4], cc[4];
+    // a warp per four rows, 32 columns at a time: up to four independent loads per lane and chunk,
+    // all before the stores
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int r0 = 4 * warp; r0 < np; r0 += 4 * nw) {
+        const float* gr[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int e = e0 + u * blockDim.x;
-            rr[u] = -1;
-            if (e < tot) {
-                int r = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-                while ((r + 1) * (r + 2) / 2 <= e) ++r;
-                while (r * (r + 1) / 2 > e) --r;
-                rr[u] = r;
-                cc[u] = e - r * (r + 1) / 2;
-                v[u] = __ldg(Gi + (size_t)sh.P[r] * smax + sh.P[cc[u]]);
+        for (int u = 0; u < 4; ++u) gr[u] = Gi + (size_t)sh.P[min(r0 + u, np - 1)] * smax;
+        for (int c0 = 0; c0 <= min(r0 + 3, np - 1); c0 += 64) {
+            float v[4][2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = c0 + 32 * h + lane;
+                const int pc = c < np ? sh.P[c] : 0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u][h] = (c <= r0 + u && r0 + u < np) ? __ldg(gr[u] + pc) : 0.f;
             }
-        }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (rr[u] < 0) continue;
-            if (sh.F.fp64) sh.F.Md[(size_t)rr[u] * sh.F.ldd + cc[u]] = (double)v[u];
-            else sh.F.Mf[(size_t)rr[u] * sh.F.ldf + cc[u]] = v[u];
+            for (int h = 0; h < 2; ++h) {
+                const int c = c0 + 32 * h + lane;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int r = r0 + u;
+                    if (c > r || r >= np) continue;
+                    if (sh.F.fp64) sh.F.Md[(size_t)r * sh.F.ldd + c] = (double)v[u][h];
+                    else sh.F.Mf[(size_t)r * sh.F.ldf + c] = v[u][h];
+                }
+            }
         }
     }
     __syncthreads();
@@ -1530,8 +1281,8 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
         sh.w = p; p += scap;
         sh.F.rdd = p; p += scap;
         float* q = reinterpret_cast<float*>(p);
-        sh.F.rdf = q; q += scap;
-        sh.F.vf = q; q += scap;
+        sh.F.rdf = q; q += fac_vec(scap);  // (16-byte aligned)
+        sh.F.vf = q; q += fac_vec(scap);
         // the FP32 factor sits in shared memory when the signal's whole active set fits
         // the msm x msm area the launch reserved, else in the signal's global workspace;
         // an odd stride spreads a column over the banks
@@ -1542,11 +1293,12 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
         // the FIN_SLOTS list slots run concurrently, so each slot has its own part
         double* wk = C > 1 ? d.fin_pool + ((size_t)cur * d.fin_slots + blockIdx.x) * smax * smax
                            : d.chol + (size_t)i * smax * smax;
+        sh.F.in_sm = fsm ? 1 : 0;
         sh.F.Mf = fsm ? q : reinterpret_cast<float*>(wk);
         if (msm) q += (size_t)msm * ((msm + 1) | 1);
-        sh.F.stage = msm ? nullptr : q;  // panel staging for a factor in global memory
-        sh.F.stage_n = msm ? 0 : fac_stage_floats(scap);
-        if (!msm) q += (size_t)fac_stage_floats(scap);
+        sh.F.stage = q;
+        sh.F.stage_n = fac_stage_floats(scap);
+        q += (size_t)fac_stage_floats(scap);
         sh.P = reinterpret_cast<int*>(q);
         sh.sg = sh.P + scap;
         sh.Pi = sh.sg + scap;
@@ -1583,8 +1335,7 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
     ClusterSync cs{sh.cbar, C, 0u};
     // (the cluster's last block bounds every block's workspace slot: a uniform check)
     if (MPL_OOB(C > 1 && ((int)(blockIdx.x / C) * C + C > d.fin_slots || (int)rank >= C), 701)) return;
-    float* cgv = msm ? nullptr
-                     : reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(sh.F.stage) + 15) & ~(uintptr_t)15);
+    float* cgv = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(sh.F.stage) + 15) & ~(uintptr_t)15);
     const double lam = (double)d.lam[i];
     const double tol = d.tol;
     const bool vec4 = (n & 3) == 0;  // float4 rows: block-cooperative residual and correlations
@@ -1616,17 +1367,16 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
     double kkt_on = 0.0, cmax_s = 0.0;
     int np = 0;
     const int max_steps = s + 32;
-    if (tid == 0) { sh.ival[3] = 0; sh.fac_np = -1; }  // ival[3] = 1: the last step added an atom from the exact check
+    if (tid == 0) sh.ival[3] = 0;  // ival[3] = 1: the last step added an atom from the exact check
     for (int a = tid; a < s; a += nt) sh.adds[a] = 0;
     __syncthreads();
     int steps = 0;
     unsigned long long flops = 0;  // algorithmic work (thread 0 keeps the tally)
     unsigned long long bytes = 0;  // algorithmic bytes streamed: Gram rows, atom columns, b
     for (int step = 0; step < max_steps; ++step, ++steps) {
-        // the FP32 factor of the previous step, updated for the atoms that left or joined P,
-        // or a new support list and factor
-        const bool inc = sh.fac_np >= 0 && !sh.F.fp64;
-        np = inc ? sh.fac_np : build_support(s, sh);
+        // the support and its factor from scratch (an update of the last step's factor, a chain of
+        // rotations, took longer than the blocked factorisation does)
+        np = build_support(s, sh);
         // ---- solve on P
         if (np > 0) {
             for (int a = tid; a < np; a += nt) sh.z[a] = (double)hi[sh.P[a]] - lam * (double)sh.sg[sh.P[a]];
@@ -1649,31 +1399,25 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
                 flops += (unsigned long long)(it + 1) * 2ull * np * np;
                 bytes += (unsigned long long)(it + 1) * 4ull * np * s;  // rows of G_PS per product
             } else {
-                if (!inc) {
-                    flops += (unsigned long long)np * np * np / 3 + 2ull * np * np;
-                    bytes += 2ull * np * (np + 1);  // the lower triangle of G_PP gathered
-                    FT_SPLIT(8);
-                    gather_gram(sh, Gi, smax, np);
-                    FT_SPLIT(9);
-                    const int fres = factor(sh.F, np, &sh.ival[0]);
-                    FT_ADD(0);
-                    if (fres != 0) {
-                        if (sh.F.fp64) break;
-                        __syncthreads();
-                        if (tid == 0) sh.F.fp64 = 1;  // FP32 pivot breakdown: retry this step in FP64
-                        __syncthreads();
-                        --step;
-                        continue;
-                    }
-                } else {
-                    flops += 2ull * np * np;
+                flops += (unsigned long long)np * np * np / 3 + 2ull * np * np;
+                bytes += 2ull * np * (np + 1);  // the lower triangle of G_PP gathered
+                FT_SPLIT(8);
+                gather_gram(sh, Gi, smax, np);
+                FT_SPLIT(9);
+                const int fres = factor(sh.F, np, &sh.ival[0]);
+                FT_ADD(0);
+                if (fres != 0) {
+                    if (sh.F.fp64) break;
+                    __syncthreads();
+                    if (tid == 0) sh.F.fp64 = 1;  // FP32 pivot breakdown: retry this step in FP64
+                    __syncthreads();
+                    --step;
+                    continue;
                 }
                 fsolve(sh.F, np, sh.z);
                 FT_ADD(1);
             }
         }
-        if (tid == 0) sh.fac_np = (!sh.F.fp64 && !sh.cg) ? np : -1;
-        __syncthreads();
         // ---- first sign crossing on the segment x -> z.  Skipped right after the
         // exact check admitted an atom: its coefficient may be below the FP32
         // Gram block's resolution, so it goes straight to exact refinement.
@@ -1714,7 +1458,6 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
                 if (sh.x[pa] == 0.0) sh.sg[pa] = 0;
             }
             __syncthreads();
-            drop_zeroed(sh, np);
             continue;
         }
         // consistent: x <- z on P (zero elsewhere)
@@ -1753,7 +1496,6 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
             }
             __syncthreads();
             if (sh.ival[0]) break;
-            join_support(sh, Gi, smax, a, np);
             continue;
         }
         // ---- exact verification: r = b - A_P x, c = A^T r (double-FP32), Newton refinement on P
@@ -1768,8 +1510,7 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
             FT_CNT(11);
             if (vec4) {
                 if (C > 1) {
-                    if (!residual_cluster(d, cs, rank, d.A32, n, sh.Pi, xd, np, b, rh, rl, cgv,
-                                          msm ? 0 : sh.F.stage_n - 4))
+                    if (!residual_cluster(d, cs, rank, d.A32, n, sh.Pi, xd, np, b, rh, rl, cgv, sh.F.stage_n - 4))
                         return;
                 } else {
                     residual_df4(d.A32, n, sh.Pi, xd, np, b, rh, rl);
@@ -1870,7 +1611,6 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
         }
         __syncthreads();
         if (sh.ival[0]) {
-            drop_zeroed(sh, np);
             continue;
         }
         flops += 2ull * n * (unsigned long long)(s - np);
@@ -1944,7 +1684,6 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
             }
             __syncthreads();
             if (sh.ival[0]) break;
-            join_support(sh, Gi, smax, a, np);
             continue;
         }
         kkt_on = fmax(dmax / lsc, fmax(cmax_s - lam, 0.0) / lsc);
@@ -2066,7 +1805,7 @@ cudaError_t launch_finish(const Dev& d, int cur, int ub, int est, int scap, cuda
     // shared-memory factor area: the whole bound while two CTAs still fit on an SM
     auto dyn_of = [&](int mf, int rs) {
         return 4 * (size_t)scap * sizeof(double) +
-               (2 * (size_t)scap + (mf ? (size_t)mf * ((mf + 1) | 1) : (size_t)fac_stage_floats(scap))) * sizeof(float) +
+               (2 * (size_t)fac_vec(scap) + (mf ? (size_t)mf * ((mf + 1) | 1) : 0) + (size_t)fac_stage_floats(scap)) * sizeof(float) +
                4 * (size_t)scap * sizeof(int) + (rs ? 2 * (size_t)d.n * sizeof(float) + 16 : 0);
     };
     const int rsm = d.n <= 4096 ? 1 : 0;
