@@ -1367,7 +1367,7 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
     double kkt_on = 0.0, cmax_s = 0.0;
     int np = 0;
     const int max_steps = s + 32;
-    if (tid == 0) sh.ival[3] = 0;  // ival[3] = 1: the last step added an atom from the exact check
+    if (tid == 0) sh.ival[3] = 0;  // ival[3] != 0: the last step added an atom from the exact check
     for (int a = tid; a < s; a += nt) sh.adds[a] = 0;
     __syncthreads();
     int steps = 0;
@@ -1377,11 +1377,29 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
         // the support and its factor from scratch (an update of the last step's factor, a chain of
         // rotations, took longer than the blocked factorisation does)
         np = build_support(s, sh);
+        // the last step's exact check admitted an atom: x solves the rest of the support exactly,
+        // so the step starts at the Newton refinement with the correlations already known (z holds
+        // them by position).  An FP32 solve here would only perturb x by its own error, which took
+        // one more exact evaluation to find and to remove; and the new coefficient may be below
+        // the FP32 Gram block's resolution, so no crossing and no Gram check apply.  (4096 x 65536, the
+        // signals with most steps: 5.6 -> 4.4 exact evaluations; the batch of 1024 29.8 -> 28.9 ms,
+        // 2048 x 32768 x 512 6.3 -> 6.2 ms.  entry = 1: the refinement had ended short of its goal;
+        // solve again, without the crossing test.)
+        const int entry = sh.ival[3];
+        const bool exact_entry = entry == 2;
+        if (exact_entry) {
+            for (int a = tid; a < np; a += nt) sh.w[a] = sh.z[sh.P[a]];
+        }
+        __syncthreads();
+        if (tid == 0) sh.ival[3] = 0;
         // ---- solve on P
         if (np > 0) {
-            for (int a = tid; a < np; a += nt) sh.z[a] = (double)hi[sh.P[a]] - lam * (double)sh.sg[sh.P[a]];
+            if (!exact_entry)
+                for (int a = tid; a < np; a += nt) sh.z[a] = (double)hi[sh.P[a]] - lam * (double)sh.sg[sh.P[a]];
             FT_CNT(6);
-            if (sh.cg) {
+            if (sh.cg && exact_entry) {
+                // (the refinement's own solve is all this step needs)
+            } else if (sh.cg) {
                 // the sign-fixed system from the current point (the master problem's solution)
                 const int it = cg_solve(sh, Gi, smax, s, np, sh.z, sh.x, 1e-6f, FIN_CG_MAXIT, cgv, (scap + 3) & ~3,
                                         d, &cs, rank);
@@ -1391,7 +1409,7 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
                 if (it == -2) return;
                 if (it < 0) {  // not converging: factor this signal's blocks from now on
                     __syncthreads();
-                    if (tid == 0) sh.cg = 0;
+                    if (tid == 0) { sh.cg = 0; sh.ival[3] = entry; }
                     __syncthreads();
                     --step;
                     continue;
@@ -1409,23 +1427,21 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
                 if (fres != 0) {
                     if (sh.F.fp64) break;
                     __syncthreads();
-                    if (tid == 0) sh.F.fp64 = 1;  // FP32 pivot breakdown: retry this step in FP64
+                    // FP32 pivot breakdown: retry this step in FP64
+                    if (tid == 0) { sh.F.fp64 = 1; sh.ival[3] = entry; }
                     __syncthreads();
                     --step;
                     continue;
                 }
-                fsolve(sh.F, np, sh.z);
+                if (!exact_entry) fsolve(sh.F, np, sh.z);
                 FT_ADD(1);
             }
         }
-        // ---- first sign crossing on the segment x -> z.  Skipped right after the
-        // exact check admitted an atom: its coefficient may be below the FP32
-        // Gram block's resolution, so it goes straight to exact refinement.
-        const bool exact_entry = sh.ival[3] != 0;
+        // ---- first sign crossing on the segment x -> z
         __syncthreads();
-        if (tid == 0) { sh.dval[1] = 2.0; sh.ival[2] = -1; sh.ival[3] = 0; }
+        if (tid == 0) { sh.dval[1] = 2.0; sh.ival[2] = -1; }
         __syncthreads();
-        if (!exact_entry && !lam0) {
+        if (!entry && !lam0) {
           for (int a = tid; a < np; a += nt) {
             const int pa = sh.P[a];
             const double xa = sh.x[pa], za = sh.z[a];
@@ -1461,14 +1477,16 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
             continue;
         }
         // consistent: x <- z on P (zero elsewhere)
-        for (int a = tid; a < s; a += nt) if (sh.sg[a] == 0) sh.x[a] = 0.0;
-        __syncthreads();
-        for (int a = tid; a < np; a += nt) sh.x[sh.P[a]] = sh.z[a];
+        if (!exact_entry) {
+            for (int a = tid; a < s; a += nt) if (sh.sg[a] == 0) sh.x[a] = 0.0;
+            __syncthreads();
+            for (int a = tid; a < np; a += nt) sh.x[sh.P[a]] = sh.z[a];
+        }
         __syncthreads();
         // ---- zero entries of S through the Gram block: add the largest violator
         if (tid == 0) sh.dval[2] = 0.0;
         __syncthreads();
-        for (int a = warp; a < s; a += nw) {
+        for (int a = exact_entry ? s : warp; a < s; a += nw) {
             if (sh.sg[a] != 0) continue;
             double acc = 0.0;
             for (int c = lane; c < np; c += 32)
@@ -1504,6 +1522,10 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
         df* xd = reinterpret_cast<df*>(sh.z);  // z is free now: x_P split into FP32 pairs
         for (int a = tid; a < np; a += nt) sh.Pi[a] = Si[sh.P[a]];
         for (int ref = 0; ref < 24; ++ref) {
+            double lmax = 0.0;
+          if (ref == 0 && exact_entry) {  // (the residual and its correlations are the last step's)
+            for (int a = tid; a < np; a += nt) lmax = fmax(lmax, fabs(sh.w[a]));
+          } else {
             for (int a = tid; a < np; a += nt) xd[a] = to_df(sh.x[sh.P[a]]);
             __syncthreads();
             FX_BEGIN
@@ -1521,7 +1543,6 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
             __syncthreads();
             flops += 4ull * n * np;  // residual and on-support correlations
             bytes += 8ull * n * np + 4ull * n;  // the support's columns twice, and b
-            double lmax = 0.0;
             if (vec4) {
                 if (C > 1) {
                     if (!dots_cluster(d, cs, rank, d.A32, n, sh.Pi, np, rh, rl, sh.w)) return;
@@ -1541,10 +1562,11 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
                     lmax = fmax(lmax, fabs(dv));
                 }
             }
+            FX_END(10);
+          }
 #pragma unroll
             for (int o = 16; o; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
             __syncthreads();
-            FX_END(10);
             if (lane == 0) sh.red[warp] = lmax;
             __syncthreads();
             dmax = 0.0;
@@ -1673,12 +1695,15 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
         if (sh.dval[3] != 0.0) {
             const unsigned long long key = (unsigned long long)__double_as_longlong(sh.dval[3]);
             const int a = 0xFFF - (int)(key & 0xFFFull);
-            // sign of the exact correlation of the entering atom
+            // the support's c - lambda s by position, and the entering atom's, with the sign of its
+            // exact correlation
+            for (int k = tid; k < np; k += nt) sh.z[sh.P[k]] = sh.w[k];
             if (warp == 0) {
                 const double ca = dot_df(d.A32 + (size_t)Si[a] * n, rh, rl, n);
                 if (lane == 0) {
                     sh.sg[a] = ca > 0.0 ? 1 : -1;
-                    sh.ival[3] = 1;  // enters through exact refinement
+                    sh.z[a] = ca - lam * (double)sh.sg[a];
+                    sh.ival[3] = dmax <= 0.1 * tol * lsc ? 2 : 1;  // enters through exact refinement
                     sh.ival[0] = ++sh.adds[a] > 3;
                 }
             }
