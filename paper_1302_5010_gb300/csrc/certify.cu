@@ -963,9 +963,14 @@ __device__ __forceinline__ float bsumf(float v, double* red) {
 // critical path), a signal's finish runs on a cluster of C CTAs (C SMs).  Every CTA runs the
 // whole finish on identical data, so their control flow is identical; only the column sweeps
 // are divided: the exact residual by row blocks of n / C entries, the correlations by blocks
-// of the atom list, after which every CTA reads the other blocks from its peers' shared
-// memory (distributed shared memory).  Before such reads, and before a CTA overwrites what
-// its peers may still read, the cluster meets at a barrier built on two mbarriers per CTA used
+// of the atom list, the CG's products by blocks of rows.  Each CTA writes its block into every
+// peer's shared memory (distributed shared memory) and the cluster meets once; reading the
+// peers' blocks instead was one remote round trip per peer and a second meeting, so that nobody
+// overwrote what a peer still read.  With writes that is settled by what lies between: a block is
+// overwritten only after a meeting that follows its last read (the CG's product alternates
+// between two buffers, having none).  Measured with clusters of 8: a CG iteration of 240 atoms 24.8 -> 12.0
+// thousand cycles, an exact evaluation of 2048 x 240 77 -> 53; the 2048 x 32768 batch of 512 6.45 -> 5.83 ms.
+// The barrier is built on two mbarriers per CTA used
 // in turn (C arrivals, one remote arrive from each CTA), waited on with a bound: on expiry the
 // CTA records DERR_TIMEOUT and the finish returns without its result.
 constexpr uint64_t FIN_CLUSTER_WAIT_NS = 4000000000ull;
@@ -988,6 +993,7 @@ struct ClusterSync {
     uint64_t* bar;  // this CTA's two barriers (count C each)
     int C;
     unsigned phase;
+    unsigned products;  // CG products so far: the buffer the next one is written to
 };
 
 // All threads of all C CTAs: returns false (uniformly within the CTA) when the wait expired.
@@ -1000,20 +1006,19 @@ struct ClusterSync {
 __device__ bool csync(const Dev& d, ClusterSync& cs) {
     __syncthreads();
     uint64_t* bar = cs.bar + (cs.phase & 1u);
-    if (threadIdx.x == 0) {
-        asm volatile("fence.acq_rel.cluster;" ::: "memory");
+    // thread r arrives at CTA r, so that the releases wait side by side; each covers the writes of
+    // the whole CTA, ordered before it by the barrier above
+    if ((int)threadIdx.x < cs.C) {
         const uint32_t local = static_cast<uint32_t>(__cvta_generic_to_shared(bar));
-        for (int r = 0; r < cs.C; ++r) {
-            uint32_t remote;
-            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(r));
-            asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
-        }
+        uint32_t remote;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(threadIdx.x));
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
     }
     const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(bar));
     const uint32_t parity = (cs.phase >> 1) & 1u;
     bool ok = false;
     uint64_t t0 = 0;
-    for (uint32_t it = 0;; ++it) {
+    for (uint32_t it = 1;; ++it) {
         uint32_t done;
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
@@ -1023,10 +1028,10 @@ __device__ bool csync(const Dev& d, ClusterSync& cs) {
             : "r"(a), "r"(parity)
             : "memory");
         if (done) { ok = true; break; }
-        if ((it & 255u) == 0u) {
+        if ((it & 255u) == 0u) {  // (the timer is slow to read: not in the first, short waits)
             uint64_t now;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-            if (it == 0) t0 = now;
+            if (t0 == 0) t0 = now;
             else if (now - t0 > FIN_CLUSTER_WAIT_NS) break;
         }
     }
@@ -1046,9 +1051,20 @@ __device__ __forceinline__ void part_of(int len, int C, int b, int align, int* l
     *hi = min(len, *lo + per);
 }
 
+// Copies entries [lo, hi) of the float arrays a and b (multiples of 4, 16-byte aligned) to the
+// same place in every peer.
+__device__ __forceinline__ void push_block(const ClusterSync& cs, unsigned rank, float* a, float* b, int lo, int hi) {
+    const int nv = (hi - lo) >> 2, per = 2 * nv;
+    for (int t = threadIdx.x; t < per * (cs.C - 1); t += blockDim.x) {
+        const int q = t / per, e = t - q * per;
+        float* src = (e < nv ? a : b) + lo + 4 * (e < nv ? e : e - nv);
+        *reinterpret_cast<float4*>(peer_ptr(src, (rank + 1 + q) % cs.C)) = *reinterpret_cast<const float4*>(src);
+    }
+}
+
 // r = b - A_P x: this CTA's row block (with the atoms spread over thread groups when the block
 // has fewer float4 slots than the CTA has threads, given scratch of blockDim.x x 8 floats),
-// then the other blocks from the peers.
+// written to the peers.  The peers read the last residual in correlations that end with a meeting.
 __device__ bool residual_cluster(const Dev& d, ClusterSync& cs, unsigned rank, const float* A, int n,
                                  const int* Pi, const df* xd, int np, const float* b, float* rh, float* rl,
                                  float* scratch, int scratch_n) {
@@ -1065,22 +1081,13 @@ __device__ bool residual_cluster(const Dev& d, ClusterSync& cs, unsigned rank, c
         residual_df4_groups(A, n, Pi, xd, np, b, rh, rl, lo, hi, G, scratch);
     else
         residual_df4_range(A, n, Pi, xd, np, b, rh, rl, lo, hi);
-    if (!csync(d, cs)) return false;
-    for (int q = 1; q < cs.C; ++q) {
-        const unsigned pr = (rank + q) % cs.C;
-        int plo, phi;
-        part_of(n, cs.C, (int)pr, 4, &plo, &phi);
-        const float4* sh4 = reinterpret_cast<const float4*>(peer_ptr(rh, pr));
-        const float4* sl4 = reinterpret_cast<const float4*>(peer_ptr(rl, pr));
-        for (int k = plo + 4 * (int)threadIdx.x; k < phi; k += 4 * (int)blockDim.x) {
-            reinterpret_cast<float4*>(rh)[k >> 2] = sh4[k >> 2];
-            reinterpret_cast<float4*>(rl)[k >> 2] = sl4[k >> 2];
-        }
-    }
-    return csync(d, cs);  // no peer overwrites its block before every CTA has read it
+    __syncthreads();
+    push_block(cs, rank, rh, rl, lo, hi);
+    return csync(d, cs);
 }
 
-// out[a] = a_{idx[a]}^T r for a < cnt: this CTA's block of atoms, then the others' results.
+// out[a] = a_{idx[a]}^T r for a < cnt: this CTA's block of atoms, written to the peers (who read the
+// last correlations before they meet in the residual, or keep them in another part of out).
 __device__ bool dots_cluster(const Dev& d, ClusterSync& cs, unsigned rank, const float* A, int n, const int* idx,
                              int cnt, const float* rh, const float* rl, double* out) {
     int lo, hi;
@@ -1089,70 +1096,97 @@ __device__ bool dots_cluster(const Dev& d, ClusterSync& cs, unsigned rank, const
     for (int a = threadIdx.x; a < cnt; a += blockDim.x)
         MPL_OOB(idx[a] < 0 || idx[a] >= d.m, 704);
 #endif
-    if (hi > lo) dots_df_warp(A, n, idx + lo, hi - lo, rh, rl, out + lo);
-    if (!csync(d, cs)) return false;
-    for (int q = 1; q < cs.C; ++q) {
-        const unsigned pr = (rank + q) % cs.C;
-        int plo, phi;
-        part_of(cnt, cs.C, (int)pr, 2, &plo, &phi);
-        const double* po = peer_ptr(out, pr);
-        for (int a = plo + (int)threadIdx.x; a < phi; a += (int)blockDim.x) out[a] = po[a];
+    if (hi > lo) {
+        dots_df_warp(A, n, idx + lo, hi - lo, rh, rl, out + lo);
+        __syncthreads();
+        const int len = hi - lo;
+        for (int t = threadIdx.x; t < len * (cs.C - 1); t += blockDim.x) {
+            const int q = t / len;
+            double* src = out + lo + (t - q * len);
+            *peer_ptr(src, (rank + 1 + q) % cs.C) = *src;
+        }
     }
     return csync(d, cs);
 }
 
-// q_a = (G_SS v)_a for the support positions a = P[k] (v is zero outside P, so this is
-// G_PP v_P): a warp per pair of rows, the row's first s entries as float4 slices when the
-// block's leading dimension allows (else scalar), fixed butterfly per row.
+// q_a = (G_SS v)_a for the support positions a = P[k], k < np (v is zero outside P and from s up to
+// the next multiple of 4, so this is G_PP v_P): lane l sums the float4 slices c = 4 l + 128 u of a
+// row in order of u, then a fixed butterfly.  A warp takes four rows per round and four slices of
+// each at a time, all sixteen loads before the first product: a round costs a round trip to L2
+// whatever it carries, and a branch between the loads one each.
+// With C > 1 each product is written to the same place in the C CTAs of the cluster.
 __device__ __noinline__ void gram_rows_mv(const float* __restrict__ Gi, int smax, int s, const int* P, int np,
-                             const float* v, float* q) {
+                                          const float* v, float* q, int C) {
+    __builtin_assume(__isShared(P));
+    __builtin_assume(__isShared(v));
+    __builtin_assume(__isShared(q));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const bool vec = (smax & 3) == 0;
-    for (int k = 2 * warp; k < np; k += 2 * nw) {
-        const int ra = P[k], rb = k + 1 < np ? P[k + 1] : P[k];
-        const float* ga = Gi + (size_t)ra * smax;
-        const float* gb = Gi + (size_t)rb * smax;
-        float sa = 0.f, sb = 0.f;
-        for (int c0 = 4 * lane; c0 < s; c0 += 512) {
-            float4 a4[4], b4[4];
+    if ((smax & 3) != 0) {  // rows that are not 16-byte aligned: the same slices and order by scalar loads
+        for (int k = warp; k < np; k += nw) {
+            const float* g = Gi + (size_t)P[k] * smax;
+            float acc = 0.f;
+            for (int c = 4 * lane; c < s; c += 128) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int c = c0 + 128 * u;
-                if (c < s) {
-                    if (vec) {
-                        a4[u] = __ldg(reinterpret_cast<const float4*>(ga + c));
-                        b4[u] = __ldg(reinterpret_cast<const float4*>(gb + c));
-                    } else {
-                        a4[u] = make_float4(__ldg(ga + c), c + 1 < s ? __ldg(ga + c + 1) : 0.f,
-                                            c + 2 < s ? __ldg(ga + c + 2) : 0.f, c + 3 < s ? __ldg(ga + c + 3) : 0.f);
-                        b4[u] = make_float4(__ldg(gb + c), c + 1 < s ? __ldg(gb + c + 1) : 0.f,
-                                            c + 2 < s ? __ldg(gb + c + 2) : 0.f, c + 3 < s ? __ldg(gb + c + 3) : 0.f);
-                    }
-                } else {
-                    a4[u] = b4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                }
+                for (int e = 0; e < 4; ++e)
+                    if (c + e < s) acc = fmaf(__ldg(g + c + e), v[c + e], acc);
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane < C) *(C > 1 ? peer_ptr(q + P[k], (unsigned)lane) : q + P[k]) = acc;
+        }
+        return;
+    }
+    constexpr int RW = 4, U = 4;
+    const int c_max = ((s + 3) & ~3) - 4;  // the last slice
+#pragma unroll 1
+    for (int k = RW * warp; k < np; k += RW * nw) {
+        const float* g[RW];
+        float acc[RW];
+#pragma unroll
+        for (int w = 0; w < RW; ++w) {
+            g[w] = Gi + (size_t)P[min(k + w, np - 1)] * smax;
+            acc[w] = 0.f;
+        }
+#pragma unroll 1
+        for (int c0 = 4 * lane; c0 - 4 * lane < s; c0 += 128 * U) {
+            float4 y[RW][U];
+            // (past the row the last slice is read again, and multiplied by zero)
+#pragma unroll
+            for (int w = 0; w < RW; ++w)
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    y[w][u] = __ldg(reinterpret_cast<const float4*>(g[w] + min(c0 + 128 * u, c_max)));
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
                 const int c = c0 + 128 * u;
-                if (c < s) {
-                    // v has zeros from s up to the next multiple of 4 (and outside P)
-                    const float4 x = *reinterpret_cast<const float4*>(v + c);
-                    sa = fmaf(a4[u].x, x.x, sa); sa = fmaf(a4[u].y, x.y, sa);
-                    sa = fmaf(a4[u].z, x.z, sa); sa = fmaf(a4[u].w, x.w, sa);
-                    sb = fmaf(b4[u].x, x.x, sb); sb = fmaf(b4[u].y, x.y, sb);
-                    sb = fmaf(b4[u].z, x.z, sb); sb = fmaf(b4[u].w, x.w, sb);
+                float4 x = *reinterpret_cast<const float4*>(v + min(c, c_max));
+                const bool in = c <= c_max;
+                x.x = in ? x.x : 0.f;
+                x.y = in ? x.y : 0.f;
+                x.z = in ? x.z : 0.f;
+                x.w = in ? x.w : 0.f;
+#pragma unroll
+                for (int w = 0; w < RW; ++w) {
+                    acc[w] = fmaf(y[w][u].x, x.x, acc[w]);
+                    acc[w] = fmaf(y[w][u].y, x.y, acc[w]);
+                    acc[w] = fmaf(y[w][u].z, x.z, acc[w]);
+                    acc[w] = fmaf(y[w][u].w, x.w, acc[w]);
                 }
             }
         }
 #pragma unroll
         for (int o = 16; o; o >>= 1) {
-            sa += __shfl_xor_sync(0xffffffffu, sa, o);
-            sb += __shfl_xor_sync(0xffffffffu, sb, o);
+#pragma unroll
+            for (int w = 0; w < RW; ++w) acc[w] += __shfl_xor_sync(0xffffffffu, acc[w], o);
         }
-        if (lane == 0) {
-            q[ra] = sa;
-            if (k + 1 < np) q[rb] = sb;
+        // lane 4 r + w: row w to CTA r
+        static_assert(RW * FIN_CLUSTER_MAX <= 32, "a lane per row and CTA");
+        float mine = acc[0];
+#pragma unroll
+        for (int w = 1; w < RW; ++w) mine = lane % RW == w ? acc[w] : mine;
+        if (lane / RW < C && k + lane % RW < np) {
+            float* o = q + P[k + lane % RW];
+            *(C > 1 ? peer_ptr(o, (unsigned)(lane / RW)) : o) = mine;
         }
     }
 }
@@ -1161,36 +1195,34 @@ __device__ __noinline__ void gram_rows_mv(const float* __restrict__ Gi, int smax
 // shared memory; the Gram blocks of these workloads are well conditioned).  io holds the
 // right-hand side on entry and the solution on exit, both indexed by support slot k < np;
 // x0 (indexed by S position, may be null) is the warm start on P.  The four vectors are
-// kept by S position in `vec` (4 x ld floats, 16-byte aligned, ld >= s rounded up to 4):
-// z, r, p (zero outside P, the product's operand) and q = G p.  Stops when the recurred
+// kept by S position in `vec` (5 x ld floats, 16-byte aligned, ld >= s rounded up to 4):
+// z, r, p (zero outside P, the product's operand) and q = G p (two, in turn).  Stops when the recurred
 // residual is at most rtol ||rhs||; returns the iterations taken, or -1 when maxit is
 // reached or the curvature p^T G p is not positive (the caller falls back to a factor).
 // G_PP v for the CG: the whole block by this CTA, or in a clustered finish this CTA's block
-// of rows followed by the other rows' products from the peers (each row by one CTA, with
-// the same arithmetic, so the product does not depend on the cluster size).  false: a
-// cluster barrier timed out.
-__device__ bool cg_product(const Dev& d, ClusterSync* cs, unsigned rank, const float* Gi, int smax, int s,
-                           const int* P, int np, const float* v, float* q) {
-    if (!cs || cs->C <= 1) {
-        gram_rows_mv(Gi, smax, s, P, np, v, q);
-        return true;
+// of rows, written to all its peers (each row by one CTA, with the same arithmetic, so the
+// product does not depend on the cluster size).  q: the two buffers, ld apart; the product's
+// place is returned.  Null: a cluster barrier timed out.
+__device__ __forceinline__ const float* cg_product(const Dev& d, ClusterSync* cs, unsigned rank, const float* Gi,
+                                                   int smax, int s, const int* P, int np, const float* v, float* q,
+                                                   int ld) {
+    const bool cluster = cs && cs->C > 1;
+    int lo = 0, hi = np;
+    if (cluster) {
+        part_of(np, cs->C, (int)rank, 2, &lo, &hi);
+        q += (cs->products++ & 1u) ? ld : 0;
     }
-    int lo, hi;
-    part_of(np, cs->C, (int)rank, 2, &lo, &hi);
 #ifdef MPL_BOUNDS
     for (int k = threadIdx.x; k < np; k += blockDim.x)
         MPL_OOB(P[k] < 0 || P[k] >= s, 705);
 #endif
-    if (hi > lo) gram_rows_mv(Gi, smax, s, P + lo, hi - lo, v, q);
-    if (!csync(d, *cs)) return false;
-    for (int r = 1; r < cs->C; ++r) {
-        const unsigned pr = (rank + r) % cs->C;
-        int plo, phi;
-        part_of(np, cs->C, (int)pr, 2, &plo, &phi);
-        const float* pq = peer_ptr(q, pr);
-        for (int k = plo + (int)threadIdx.x; k < phi; k += (int)blockDim.x) q[P[k]] = pq[P[k]];
+    if (hi > lo) gram_rows_mv(Gi, smax, s, P + lo, hi - lo, v, q, cluster ? cs->C : 1);
+    if (cluster) {
+        if (!csync(d, *cs)) return nullptr;
+    } else {
+        __syncthreads();
     }
-    return csync(d, *cs);
+    return q;
 }
 
 // Returns the iterations taken, -1 when it does not converge, -2 when a cluster barrier
@@ -1201,7 +1233,7 @@ __device__ __noinline__ int cg_solve(FinShared& sh, const float* Gi, int smax, i
     float* z = vec;
     float* r = vec + ld;
     float* p = vec + 2 * ld;
-    float* q = vec + 3 * ld;
+    float* qb = vec + 3 * ld;
     const int sp = (s + 3) & ~3;
     for (int a = tid; a < sp; a += nt) { p[a] = 0.f; z[a] = 0.f; }
     __syncthreads();
@@ -1215,8 +1247,8 @@ __device__ __noinline__ int cg_solve(FinShared& sh, const float* Gi, int smax, i
     }
     bb = bsumf(bb, sh.red);
     if (x0) {  // r = rhs - G z0
-        if (!cg_product(d, cs, rank, Gi, smax, s, sh.P, np, p, q)) return -2;
-        __syncthreads();
+        const float* q = cg_product(d, cs, rank, Gi, smax, s, sh.P, np, p, qb, ld);
+        if (!q) return -2;
         for (int k = tid; k < np; k += nt) { const int a = sh.P[k]; r[a] -= q[a]; }
         __syncthreads();
     }
@@ -1229,8 +1261,8 @@ __device__ __noinline__ int cg_solve(FinShared& sh, const float* Gi, int smax, i
     for (;;) {
         if (rr <= stop2) { ok = 1; break; }
         if (it >= maxit) break;
-        if (!cg_product(d, cs, rank, Gi, smax, s, sh.P, np, p, q)) return -2;
-        __syncthreads();
+        const float* q = cg_product(d, cs, rank, Gi, smax, s, sh.P, np, p, qb, ld);
+        if (!q) return -2;
         float pq = 0.f;
         for (int k = tid; k < np; k += nt) { const int a = sh.P[k]; pq = fmaf(p[a], q[a], pq); }
         pq = bsumf(pq, sh.red);
@@ -1332,7 +1364,7 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
     const unsigned rank = C > 1 ? cluster_rank() : 0u;
-    ClusterSync cs{sh.cbar, C, 0u};
+    ClusterSync cs{sh.cbar, C, 0u, 0u};
     // (the cluster's last block bounds every block's workspace slot: a uniform check)
     if (MPL_OOB(C > 1 && ((int)(blockIdx.x / C) * C + C > d.fin_slots || (int)rank >= C), 701)) return;
     float* cgv = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(sh.F.stage) + 15) & ~(uintptr_t)15);
@@ -1708,6 +1740,7 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
                 }
             }
             __syncthreads();
+            if (C > 1 && !csync(d, cs)) return;  // the residual has been read
             if (sh.ival[0]) break;
             continue;
         }
