@@ -107,19 +107,57 @@ __device__ __forceinline__ df warp_df_sum(df v) {
 }
 
 // ---------------------------------------------------------------- block helpers
-__device__ __forceinline__ double bsum(double v, double* red) {
+// The FP64 pipe takes two lanes a cycle on an SM: one FP64 instruction of a 512-thread CTA is 256
+// cycles.  So the CTA's reductions do as little as they can in it (a CG iteration's two sums and vector
+// updates at 512 threads: 10.4 thousand cycles with the warps' totals kept as doubles; with the screened
+// check of the zeros the 4096 x 65536 batch of 1024 28.2 -> 26.0 ms, 2048 x 32768 x 512 5.40 -> 5.02 ms,
+// 1024 x 8192 x 256 0.599 -> 0.581 ms).
+
+// Largest v >= 0 (not NaN) over the CTA, in every thread, by integer comparisons of the bits.
+__device__ __forceinline__ double bmax(double v, double* red) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    unsigned long long u = (unsigned long long)__double_as_longlong(v);
 #pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = 16; o; o >>= 1) u = max(u, __shfl_xor_sync(0xffffffffu, u, o));
     __syncthreads();
-    if (lane == 0) red[warp] = v;
+    if (lane == 0) red[warp] = __longlong_as_double((long long)u);
     __syncthreads();
-    double t = 0.0;
-    for (int w = 0; w < nw; ++w) t += red[w];
-    return t;
+    u = lane < nw ? (unsigned long long)__double_as_longlong(red[lane]) : 0ull;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) u = max(u, __shfl_xor_sync(0xffffffffu, u, o));
+    return __longlong_as_double((long long)u);
 }
 
-
+// Sums of eight values over the CTA (at most 32 warps) into part[0..8): each level of the warps'
+// butterfly halves the values a lane carries (9 additions instead of 40), then one warp adds
+// the warps' totals.  part: 8 doubles per warp.  Fixed order; all threads call, and may read part
+// after a barrier of their own.
+__device__ __forceinline__ void bsum8(double (&v)[8], double* part) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int h = 4, o = 16; h; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+            const double send = up ? v[q] : v[q + h];
+            v[q] = (up ? v[q + h] : v[q]) + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    // lane 4 q holds the warp's total of value q (bits 16, 8, 4 of the lane: 4, 2, 1 of q)
+    __syncthreads();
+    if ((lane & 3) == 0) part[warp * 8 + (lane >> 2)] = v[0];
+    __syncthreads();
+    if (warp == 0) {
+        double t = 0.0;
+        for (int w = lane >> 3; w < nw; w += 4) t += part[w * 8 + (lane & 7)];
+        t += __shfl_xor_sync(0xffffffffu, t, 8);
+        t += __shfl_xor_sync(0xffffffffu, t, 16);
+        __syncwarp();
+        if (lane < 8) part[lane] = t;
+    }
+}
 
 // Right-looking Cholesky by the whole CTA, panels of W columns (the FP64 fallback, in global
 // memory): one thread factors the W x W diagonal block, the threads take the panel's rows
@@ -618,6 +656,92 @@ __device__ int build_support(int s, FinShared& sh) {
     return sh.ival[1];
 }
 
+// Positions of S outside the support, in order, into zl (one warp; count in ival[2]).
+__device__ int list_zeros(int s, FinShared& sh, int* zl) {
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        int base = 0;
+        for (int a0 = 0; a0 < s; a0 += 32) {
+            const int a = a0 + threadIdx.x;
+            const bool z = a < s && sh.sg[a] == 0;
+            const unsigned b = __ballot_sync(0xffffffffu, z);
+            if (z) zl[base + __popc(b & ((1u << threadIdx.x) - 1u))] = a;
+            base += __popc(b);
+        }
+        if (threadIdx.x == 0) sh.ival[2] = base;
+    }
+    __syncthreads();
+    return sh.ival[2];
+}
+
+// The correlations h_a - (G_SS x)_a of the nz positions a in zl (rows of 16-byte alignment) in FP32,
+// with a bound on their error: flag[k] = 0 where the correlation is surely within thr.  v: x in FP32
+// by position, zeros from s up to the next multiple of 4.  A lane's sum has at most ceil(s / 128) * 4
+// products, the butterfly five additions, x one rounding, and so has the sum of their sizes.
+__device__ __noinline__ void screen_zeros(const float* __restrict__ Gi, int smax, int s, const int* zl, int nz,
+                                          const float* v, const float* __restrict__ hi, float thr, int* flag) {
+    __builtin_assume(__isShared(zl));
+    __builtin_assume(__isShared(v));
+    __builtin_assume(__isShared(flag));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    constexpr int RW = 4, U = 2;
+    const int c_max = ((s + 3) & ~3) - 4;
+    const float gam = (float)(((s + 127) >> 7) * 4 + 10) * 6.1e-8f;
+#pragma unroll 1
+    for (int k = RW * warp; k < nz; k += RW * nw) {
+        const float* g[RW];
+        float acc[RW], mag[RW];
+#pragma unroll
+        for (int w = 0; w < RW; ++w) {
+            g[w] = Gi + (size_t)zl[min(k + w, nz - 1)] * smax;
+            acc[w] = mag[w] = 0.f;
+        }
+        const float ha = __ldg(hi + zl[min(k + lane % RW, nz - 1)]);
+#pragma unroll 1
+        for (int c0 = 4 * lane; c0 - 4 * lane < s; c0 += 128 * U) {
+            float4 y[RW][U];
+#pragma unroll
+            for (int w = 0; w < RW; ++w)
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    y[w][u] = __ldg(reinterpret_cast<const float4*>(g[w] + min(c0 + 128 * u, c_max)));
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int c = c0 + 128 * u;
+                const float4 t = *reinterpret_cast<const float4*>(v + min(c, c_max));
+                const bool in = c <= c_max;
+                const float x[4] = {in ? t.x : 0.f, in ? t.y : 0.f, in ? t.z : 0.f, in ? t.w : 0.f};
+#pragma unroll
+                for (int w = 0; w < RW; ++w) {
+                    const float z[4] = {y[w][u].x, y[w][u].y, y[w][u].z, y[w][u].w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        acc[w] = fmaf(z[e], x[e], acc[w]);
+                        mag[w] = fmaf(fabsf(z[e]), fabsf(x[e]), mag[w]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+#pragma unroll
+            for (int w = 0; w < RW; ++w) {
+                acc[w] += __shfl_xor_sync(0xffffffffu, acc[w], o);
+                mag[w] += __shfl_xor_sync(0xffffffffu, mag[w], o);
+            }
+        }
+        float a = acc[0], m = mag[0];
+#pragma unroll
+        for (int w = 1; w < RW; ++w) {
+            a = lane == w ? acc[w] : a;
+            m = lane == w ? mag[w] : m;
+        }
+        // (the last terms: the subtraction's rounding, products below the normal range)
+        const float c = fabsf(ha - a) + (gam * m + 1.3e-7f * (fabsf(ha) + fabsf(a)) + 1e-35f);
+        if (lane < RW && k + lane < nz) flag[k + lane] = c <= thr ? 0 : 1;  // (NaN: 1)
+    }
+}
+
 // r = b - A_P x in double-FP32.  Each thread keeps 8 independent chains (8
 // entries of r), so the loads of one atom column overlap the arithmetic.
 __device__ void residual_df(const float* __restrict__ A, int n, const int* Pi, const df* xd, int np,
@@ -726,6 +850,27 @@ __device__ double dot_ff(const float* __restrict__ a, const float* __restrict__ 
     return to_d(warp_df_sum(df_add(c0, c1)));
 }
 
+// The last columns a, a + step, ... < np (one to seven) of the sweeps below, subtracted from entries
+// k .. k + 3 in that order: all loaded before the first product (one by one, each was a round trip).
+__device__ __forceinline__ void columns_rest(const float* __restrict__ A, int n, const int* Pi, const df* xd, int np,
+                                             int a, int step, int k, df& c0, df& c1, df& c2, df& c3) {
+    float4 v[7];
+#pragma unroll
+    for (int u = 0; u < 7; ++u) {  // (past the end the first one again)
+        const int q = a + u * step < np ? a + u * step : a;
+        v[u] = __ldg(reinterpret_cast<const float4*>(A + (size_t)Pi[q] * n + k));
+    }
+#pragma unroll
+    for (int u = 0; u < 7; ++u) {
+        if (a + u * step >= np) break;
+        const df x = xd[a + u * step];
+        c0 = df_fma(c0, -v[u].x, x);
+        c1 = df_fma(c1, -v[u].y, x);
+        c2 = df_fma(c2, -v[u].z, x);
+        c3 = df_fma(c3, -v[u].w, x);
+    }
+}
+
 // r = b - A_P x in double-FP32 for n % 4 == 0: thread t owns the four entries
 // 4t + 4 nt c; the atom columns are read as float4, eight atoms per round so
 // that eight loads are in flight.  Each entry sums the atoms in order of P, as
@@ -750,14 +895,7 @@ __device__ void residual_df4_range(const float* __restrict__ A, int n, const int
                 c3 = df_fma(c3, -v[u].w, x);
             }
         }
-        for (; a < np; ++a) {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(A + (size_t)Pi[a] * n + k));
-            const df x = xd[a];
-            c0 = df_fma(c0, -v.x, x);
-            c1 = df_fma(c1, -v.y, x);
-            c2 = df_fma(c2, -v.z, x);
-            c3 = df_fma(c3, -v.w, x);
-        }
+        if (a < np) columns_rest(A, n, Pi, xd, np, a, 1, k, c0, c1, c2, c3);
         *reinterpret_cast<float4*>(rh + k) = make_float4(c0.hi, c1.hi, c2.hi, c3.hi);
         *reinterpret_cast<float4*>(rl + k) = make_float4(c0.lo, c1.lo, c2.lo, c3.lo);
     }
@@ -800,14 +938,7 @@ __device__ void residual_df4_groups(const float* __restrict__ A, int n, const in
                 c3 = df_fma(c3, -w[u].w, x);
             }
         }
-        for (; a < np; a += G) {
-            const float4 w = __ldg(reinterpret_cast<const float4*>(A + (size_t)Pi[a] * n + k));
-            const df x = xd[a];
-            c0 = df_fma(c0, -w.x, x);
-            c1 = df_fma(c1, -w.y, x);
-            c2 = df_fma(c2, -w.z, x);
-            c3 = df_fma(c3, -w.w, x);
-        }
+        if (a < np) columns_rest(A, n, Pi, xd, np, a, G, k, c0, c1, c2, c3);
         float4* sp = reinterpret_cast<float4*>(scratch + (size_t)tid * 8);
         sp[0] = make_float4(c0.hi, c0.lo, c1.hi, c1.lo);
         sp[1] = make_float4(c2.hi, c2.lo, c3.hi, c3.lo);
@@ -836,7 +967,7 @@ __device__ void residual_df4_groups(const float* __restrict__ A, int n, const in
 // memory; one butterfly per pair (the first level splits the two atoms over the
 // half-warps).  Fixed summation order.
 __device__ void dots_df_warp(const float* __restrict__ A, int n, const int* idx, int cnt, const float* rh,
-                             const float* rl, double* out) {
+                             const float* rl, df* out) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int a0 = 2 * warp; a0 < cnt; a0 += 2 * nw) {
         const bool two = a0 + 1 < cnt;
@@ -883,8 +1014,8 @@ __device__ void dots_df_warp(const float* __restrict__ A, int n, const int* idx,
             w.lo = __shfl_xor_sync(0xffffffffu, keep.lo, o);
             keep = df_add(keep, w);
         }
-        if (lane == 0) out[a0] = to_d(keep);
-        if (lane == 16 && two) out[a0 + 1] = to_d(keep);
+        if (lane == 0) out[a0] = keep;
+        if (lane == 16 && two) out[a0 + 1] = keep;
     }
 }
 
@@ -951,10 +1082,11 @@ __device__ __forceinline__ float bsumf(float v, double* red) {
 #pragma unroll
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     __syncthreads();
-    if (lane == 0) red[warp] = (double)v;
+    float* rf = reinterpret_cast<float*>(red);  // (doubles here cost 16 conversions a thread: 4000 cycles)
+    if (lane == 0) rf[warp] = v;
     __syncthreads();
     float t = 0.f;
-    for (int w = 0; w < nw; ++w) t += (float)red[w];
+    for (int w = 0; w < nw; ++w) t += rf[w];
     return t;
 }
 
@@ -1089,7 +1221,7 @@ __device__ bool residual_cluster(const Dev& d, ClusterSync& cs, unsigned rank, c
 // out[a] = a_{idx[a]}^T r for a < cnt: this CTA's block of atoms, written to the peers (who read the
 // last correlations before they meet in the residual, or keep them in another part of out).
 __device__ bool dots_cluster(const Dev& d, ClusterSync& cs, unsigned rank, const float* A, int n, const int* idx,
-                             int cnt, const float* rh, const float* rl, double* out) {
+                             int cnt, const float* rh, const float* rl, df* out) {
     int lo, hi;
     part_of(cnt, cs.C, (int)rank, 2, &lo, &hi);
 #ifdef MPL_BOUNDS
@@ -1102,7 +1234,7 @@ __device__ bool dots_cluster(const Dev& d, ClusterSync& cs, unsigned rank, const
         const int len = hi - lo;
         for (int t = threadIdx.x; t < len * (cs.C - 1); t += blockDim.x) {
             const int q = t / len;
-            double* src = out + lo + (t - q * len);
+            double* src = reinterpret_cast<double*>(out + lo) + (t - q * len);  // (a pair at once)
             *peer_ptr(src, (rank + 1 + q) % cs.C) = *src;
         }
     }
@@ -1518,19 +1650,38 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
         // ---- zero entries of S through the Gram block: add the largest violator
         if (tid == 0) sh.dval[2] = 0.0;
         __syncthreads();
-        for (int a = exact_entry ? s : warp; a < s; a += nw) {
-            if (sh.sg[a] != 0) continue;
-            double acc = 0.0;
-            for (int c = lane; c < np; c += 32)
-                acc += (double)Gi[(size_t)a * smax + sh.P[c]] * sh.x[sh.P[c]];
+        if (!exact_entry) {
+            // the zeros' positions in z (free until the verification) behind flags for the FP64 sums: at two FP64
+            // lanes a cycle an SM these took most of the check, and few correlations are near enough to need them
+            // (4096 x 65536, 113 zeros of 352 atoms: 62 thousand cycles, now 20)
+            int* zl = reinterpret_cast<int*>(sh.z);
+            int* zf = zl + scap;
+            const int nzl = list_zeros(s, sh, zl);
+            if ((smax & 3) == 0 && nzl > 0) {
+                const int sp = (s + 3) & ~3;
+                for (int a = tid; a < sp; a += nt) cgv[a] = a < s ? (float)sh.x[a] : 0.f;
+                __syncthreads();
+                // (thr is below the FP64 test's threshold by more than its own rounding)
+                screen_zeros(Gi, smax, s, zl, nzl, cgv, hi, (float)(lam * (1.0 + 1e-3 - 1e-6)), zf);
+            } else {
+                for (int k = tid; k < nzl; k += nt) zf[k] = 1;
+            }
+            __syncthreads();
+            for (int k = warp; k < nzl; k += nw) {
+                if (!zf[k]) continue;
+                const int a = zl[k];
+                double acc = 0.0;
+                for (int c = lane; c < np; c += 32)
+                    acc += (double)Gi[(size_t)a * smax + sh.P[c]] * sh.x[sh.P[c]];
 #pragma unroll
-            for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            const double ca = (double)hi[a] - acc;
-            if (lane == 0 && fabs(ca) > lam * (1.0 + 1e-3)) {  // well beyond the Gram block's resolution
-                // largest |c|, ties to the lowest position
-                unsigned long long key = ((unsigned long long)__double_as_longlong(fabs(ca)) & ~0xFFFull) |
-                                         (unsigned long long)(0xFFF - a);
-                atomicMax(reinterpret_cast<unsigned long long*>(&sh.dval[2]), key);
+                for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                const double ca = (double)hi[a] - acc;
+                if (lane == 0 && fabs(ca) > lam * (1.0 + 1e-3)) {  // well beyond the Gram block's resolution
+                    // largest |c|, ties to the lowest position
+                    unsigned long long key = ((unsigned long long)__double_as_longlong(fabs(ca)) & ~0xFFFull) |
+                                             (unsigned long long)(0xFFF - a);
+                    atomicMax(reinterpret_cast<unsigned long long*>(&sh.dval[2]), key);
+                }
             }
         }
         __syncthreads();
@@ -1538,11 +1689,15 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
         if (sh.dval[2] != 0.0) {
             const unsigned long long key = (unsigned long long)__double_as_longlong(sh.dval[2]);
             const int a = 0xFFF - (int)(key & 0xFFFull);
-            if (tid == 0) {
+            if (warp == 0) {
                 double acc = 0.0;
-                for (int c = 0; c < np; ++c) acc += (double)Gi[(size_t)a * smax + sh.P[c]] * sh.x[sh.P[c]];
-                sh.sg[a] = ((double)hi[a] - acc) > 0.0 ? 1 : -1;
-                sh.ival[0] = ++sh.adds[a] > 3;  // an atom that keeps re-entering: give up
+                for (int c = lane; c < np; c += 32) acc += (double)Gi[(size_t)a * smax + sh.P[c]] * sh.x[sh.P[c]];
+#pragma unroll
+                for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if (lane == 0) {
+                    sh.sg[a] = ((double)hi[a] - acc) > 0.0 ? 1 : -1;
+                    sh.ival[0] = ++sh.adds[a] > 3;  // an atom that keeps re-entering: give up
+                }
             }
             __syncthreads();
             if (sh.ival[0]) break;
@@ -1577,13 +1732,13 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
             bytes += 8ull * n * np + 4ull * n;  // the support's columns twice, and b
             if (vec4) {
                 if (C > 1) {
-                    if (!dots_cluster(d, cs, rank, d.A32, n, sh.Pi, np, rh, rl, sh.w)) return;
+                    if (!dots_cluster(d, cs, rank, d.A32, n, sh.Pi, np, rh, rl, reinterpret_cast<df*>(sh.w))) return;
                 } else {
-                    dots_df_warp(d.A32, n, sh.Pi, np, rh, rl, sh.w);
+                    dots_df_warp(d.A32, n, sh.Pi, np, rh, rl, reinterpret_cast<df*>(sh.w));
                 }
                 __syncthreads();
                 for (int a = tid; a < np; a += nt) {
-                    const double dv = sh.w[a] - lam * (double)sh.sg[sh.P[a]];
+                    const double dv = to_d(reinterpret_cast<const df*>(sh.w)[a]) - lam * (double)sh.sg[sh.P[a]];
                     sh.w[a] = dv;
                     lmax = fmax(lmax, fabs(dv));
                 }
@@ -1596,13 +1751,7 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
             }
             FX_END(10);
           }
-#pragma unroll
-            for (int o = 16; o; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-            __syncthreads();
-            if (lane == 0) sh.red[warp] = lmax;
-            __syncthreads();
-            dmax = 0.0;
-            for (int q = 0; q < nw; ++q) dmax = fmax(dmax, sh.red[q]);
+            dmax = bmax(lmax, sh.red);
             if (np == 0 || dmax <= 0.1 * tol * lsc) break;
             if (ref > 0 && dmax > 0.25 * dprev) {
                 // slow contraction: CG's FP32 block limits it (factor it), or the FP32 factor
@@ -1675,31 +1824,17 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
         if (vec4) {
             // zero entries of S: atom indices after those of P in Pi, positions in z (free now)
             int* zpos = reinterpret_cast<int*>(sh.z);
-            if (warp == 0) {
-                int base = 0;
-                for (int a0 = 0; a0 < s; a0 += 32) {
-                    const int a = a0 + lane;
-                    const bool z0 = a < s && sh.sg[a] == 0;
-                    const unsigned bal = __ballot_sync(0xffffffffu, z0);
-                    if (z0) {
-                        const int k = base + __popc(bal & ((1u << lane) - 1u));
-                        zpos[k] = a;
-                        sh.Pi[np + k] = Si[a];
-                    }
-                    base += __popc(bal);
-                }
-                if (lane == 0) sh.ival[2] = base;
-            }
+            const int nz = list_zeros(s, sh, zpos);
+            for (int k = tid; k < nz; k += nt) sh.Pi[np + k] = Si[zpos[k]];
             __syncthreads();
-            const int nz = sh.ival[2];
             if (C > 1) {
-                if (!dots_cluster(d, cs, rank, d.A32, n, sh.Pi + np, nz, rh, rl, sh.w + np)) return;
+                if (!dots_cluster(d, cs, rank, d.A32, n, sh.Pi + np, nz, rh, rl, reinterpret_cast<df*>(sh.w) + np)) return;
             } else {
-                dots_df_warp(d.A32, n, sh.Pi + np, nz, rh, rl, sh.w + np);
+                dots_df_warp(d.A32, n, sh.Pi + np, nz, rh, rl, reinterpret_cast<df*>(sh.w) + np);
             }
             __syncthreads();
             for (int k = tid; k < nz; k += nt) {
-                const double ca = sh.w[np + k];
+                const double ca = to_d(reinterpret_cast<const df*>(sh.w)[np + k]);
                 if (fabs(ca) > cmax) { cmax = fabs(ca); worst = zpos[k]; }
             }
         } else {
@@ -1716,13 +1851,7 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
                                      (unsigned long long)(0xFFF - worst);
             atomicMax(reinterpret_cast<unsigned long long*>(&sh.dval[3]), key);
         }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) cmax = fmax(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
-        __syncthreads();
-        if (lane == 0) sh.red[warp] = cmax;
-        __syncthreads();
-        cmax_s = 0.0;
-        for (int q = 0; q < nw; ++q) cmax_s = fmax(cmax_s, sh.red[q]);
+        cmax_s = bmax(cmax, sh.red);  // (its barriers also separate dval[3] from its reading below)
         FT_ADD(5);
         if (sh.dval[3] != 0.0) {
             const unsigned long long key = (unsigned long long)__double_as_longlong(sh.dval[3]);
@@ -1783,26 +1912,19 @@ __global__ void __launch_bounds__(NT, 2 * FIN_THREADS / NT) k_finish(Dev d, int 
             es += e * e;
             ts += fq * fq;
         }
-        const double L1 = bsum(l1, sh.red);
-        const double RR = bsum(rr, sh.red);
-        const double RB = bsum(rb, sh.red);
-        const double RS = bsum(rs, sh.red);
-        const double ES = bsum(es, sh.red);
-        const double TS = bsum(ts, sh.red);
-#pragma unroll
-        for (int o = 16; o; o >>= 1) cm = fmax(cm, __shfl_xor_sync(0xffffffffu, cm, o));
-        __syncthreads();
-        if (lane == 0) sh.red[warp] = cm;
-        __syncthreads();
+        double sums[8] = {l1, rr, rb, rs, es, ts, 0.0, 0.0};
+        double* part = reinterpret_cast<double*>(cgv);  // (the staging area is free now)
+        bsum8(sums, part);
+        const double CM = bmax(cm, sh.red);
+        if (tid < 3) {  // ||r||, ||r - bf(r)||, ||bf(r)||: a square root each, side by side
+            const float v = (float)(sqrt(part[3 + tid]) * (1.0 + 1e-5));
+            (tid == 0 ? d.rnorm : tid == 1 ? d.r16e : d.r16t)[i] = v;
+        }
         if (tid == 0) {
-            double CM = 0.0;
-            for (int q = 0; q < nw; ++q) CM = fmax(CM, sh.red[q]);
+            const double L1 = part[0], RR = part[1], RB = part[2];
             d.obj[i] = lam * L1 + 0.5 * RR;
             d.rr[i] = RR;
             d.rb[i] = RB;
-            d.rnorm[i] = (float)(sqrt(RS) * (1.0 + 1e-5));
-            d.r16e[i] = (float)(sqrt(ES) * (1.0 + 1e-5));
-            d.r16t[i] = (float)(sqrt(TS) * (1.0 + 1e-5));
             if (d.xl1) d.xl1[i] = __double2float_ru(L1 * (1.0 + 1e-6));
             d.kkt_in[i] = kkt_on;
             d.ginf[i] = fmax(CM, cmax_s);

@@ -39,3 +39,17 @@ def test_entries_below_the_gram_block(n, k, p, smax):
     assert np.linalg.norm(X64 - Xo, axis=1).max() <= 1.8e-7
     assert np.abs(X64 - Xo)[tiny].max() <= 2e-8
     assert np.count_nonzero(X64[tiny]) == np.count_nonzero(Xo[tiny])
+
+
+@pytest.mark.parametrize("smax", [511, 512])
+def test_zero_entries_screened_or_not(smax):
+    """Active sets with many zero entries, whose Gram correlations are screened in FP32 when the rows are
+    16-byte aligned (512) and summed in FP64 otherwise (511): both end at the oracle's solution.
+    Correlations on the support are within 1e-7 lambda, so an entry is off by at most that times the
+    inverse block's norm (below 10 for Gaussian blocks of 240 of 1024 rows) in both solvers: relative to
+    ||x||, with lambda 0.005 of the largest correlation, below 2e-9 sqrt(240) 10 / sqrt(60) < 1e-7."""
+    P = synth.small_problem(1024, 3000, 12, 60, 200, rho=40, lam_frac=0.005, seed=1500)
+    _, X64, res = solve_gpu(P, precision=0, smax=smax)
+    assert_certified(res)
+    Xo = oracle_solve(P)
+    assert np.linalg.norm(X64 - Xo) <= 1e-7 * np.linalg.norm(Xo)
