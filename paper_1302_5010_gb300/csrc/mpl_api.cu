@@ -733,7 +733,7 @@ static cudaError_t launch_iteration(mpl_ctx* h, const Dev& d, int t, int act_ub,
     const int qmax = (t == 0 && warm_active(h, d)) ? d.rho + warm_additions(h, d) : d.omega * d.rho;
     if (h->qgram) {
         if ((e = launch_gram_gather(d, act_ub, run, nl)) != cudaSuccess) return e;
-    } else if ((e = launch_gram(d, act_ub, qmax, run, nl)) != cudaSuccess) {
+    } else if ((e = launch_gram(d, act_ub, qmax, scap, h->sms, run, nl)) != cudaSuccess) {
         return e;
     }
     if (pt) pt->end(3, e0, run);

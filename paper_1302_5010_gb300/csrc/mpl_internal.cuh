@@ -247,7 +247,8 @@ cudaError_t launch_compact(const Dev& d, int cur, int slot, cudaStream_t s, int6
 // The new rows and columns of each growing signal's Gram block (h of the new atoms was
 // written by the selection that appended them).
 // qmax: most atoms a signal can take this iteration (picks the tile width).
-cudaError_t launch_gram(const Dev& d, int ub, int qmax, cudaStream_t s, int64_t* nl);
+// qmax, scap: bounds on the atoms a signal gained and on its |S|.
+cudaError_t launch_gram(const Dev& d, int ub, int qmax, int scap, int sms, cudaStream_t s, int64_t* nl);
 // Gram growth gathered from Q (MPL_OPT_QGRAM): same outputs, bit for bit, as launch_gram.
 cudaError_t launch_gram_gather(const Dev& d, int ub, cudaStream_t s, int64_t* nl);
 // The exact finish of the signals the selection of an iteration sent to list slot `slot`

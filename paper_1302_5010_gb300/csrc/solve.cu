@@ -174,163 +174,103 @@ __global__ void __launch_bounds__(256) k_init(Dev d) {
 }
 
 // ------------------------------------------------------------------ gram
-// G[a][b] for a in [0, s), b in [s0, s) (mirrored), tile 64 (a) x 32 (b).
-constexpr int GBM = 64, GBN = 32, GBK = 32;
-
-template <bool VEC>
-__device__ __forceinline__ float4 gram_load(const float* row, int k, int n) {
-    if (row == nullptr || k >= n) return make_float4(0.f, 0.f, 0.f, 0.f);
-    if (VEC) return __ldg(reinterpret_cast<const float4*>(row + k));
-    float t[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) t[e] = (k + e < n) ? __ldg(row + k + e) : 0.f;
-    return make_float4(t[0], t[1], t[2], t[3]);
-}
-
-template <bool VEC>
-__global__ void __launch_bounds__(256) k_gram(Dev d) {
-    pdl_enter();
-    const int g = blockIdx.x;
-    if (g >= d.cnt->grow_n) return;
-    const int i = d.list_grow[g];
-    const int s = d.ssize[i], q = d.snew[i], s0 = s - q;
-    const int a0 = blockIdx.y * GBM;
-    if (a0 >= s || q == 0) return;  // q == 0: a refine pass, the block is complete
-    const int n = d.n, smax = d.smax;
-    const int* Si = d.S + (size_t)i * smax;
-    float* Gi = d.G + (size_t)i * smax * smax;
-    // two K-slices: the next slice's loads are in flight while this one is used
-    __shared__ __align__(16) float As[2][GBK][GBM + 4];
-    __shared__ __align__(16) float Bs[2][GBK][GBN + 4];
-    const int tid = threadIdx.x;
-    const int ty = tid >> 3, tx = tid & 7;
-    const int lr = tid >> 3, lk = (tid & 7) * 4;
-
-    // columns 0..q-1 are the new atoms (their h = a^T b comes with the selection's re-score)
-    for (int b0 = 0; b0 < q; b0 += GBN) {
-        float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-        const int ra0 = a0 + lr, ra1 = a0 + lr + 32;
-        const float* pa0 = (ra0 < s) ? d.A32 + (size_t)Si[ra0] * n : nullptr;
-        const float* pa1 = (ra1 < s) ? d.A32 + (size_t)Si[ra1] * n : nullptr;
-        const int rb = b0 + lr;
-        const float* pb = (rb < q) ? d.A32 + (size_t)Si[s0 + rb] * n : nullptr;
-        float4 v0 = gram_load<VEC>(pa0, lk, n), v1 = gram_load<VEC>(pa1, lk, n), vb = gram_load<VEC>(pb, lk, n);
-        const int nsl = (n + GBK - 1) / GBK;
-        for (int sl = 0; sl < nsl; ++sl) {
-            const int buf = sl & 1;
-            As[buf][lk + 0][lr] = v0.x; As[buf][lk + 1][lr] = v0.y; As[buf][lk + 2][lr] = v0.z; As[buf][lk + 3][lr] = v0.w;
-            As[buf][lk + 0][lr + 32] = v1.x; As[buf][lk + 1][lr + 32] = v1.y;
-            As[buf][lk + 2][lr + 32] = v1.z; As[buf][lk + 3][lr + 32] = v1.w;
-            Bs[buf][lk + 0][lr] = vb.x; Bs[buf][lk + 1][lr] = vb.y; Bs[buf][lk + 2][lr] = vb.z; Bs[buf][lk + 3][lr] = vb.w;
-            __syncthreads();
-            if (sl + 1 < nsl) {
-                const int kk = (sl + 1) * GBK + lk;
-                v0 = gram_load<VEC>(pa0, kk, n);
-                v1 = gram_load<VEC>(pa1, kk, n);
-                vb = gram_load<VEC>(pb, kk, n);
-            }
-#pragma unroll 8
-            for (int k = 0; k < GBK; ++k) {
-                const float x0 = As[buf][k][ty * 2], x1 = As[buf][k][ty * 2 + 1];
-                const float4 y = *reinterpret_cast<const float4*>(&Bs[buf][k][tx * 4]);
-                acc[0][0] = fmaf(x0, y.x, acc[0][0]); acc[0][1] = fmaf(x0, y.y, acc[0][1]);
-                acc[0][2] = fmaf(x0, y.z, acc[0][2]); acc[0][3] = fmaf(x0, y.w, acc[0][3]);
-                acc[1][0] = fmaf(x1, y.x, acc[1][0]); acc[1][1] = fmaf(x1, y.y, acc[1][1]);
-                acc[1][2] = fmaf(x1, y.z, acc[1][2]); acc[1][3] = fmaf(x1, y.w, acc[1][3]);
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int a = a0 + ty * 2 + u;
-            if (a >= s) continue;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const int bb = b0 + tx * 4 + v;
-                if (bb >= q) continue;
-                const int col = s0 + bb;
-                Gi[(size_t)a * smax + col] = acc[u][v];
-                Gi[(size_t)col * smax + a] = acc[u][v];
-            }
-        }
-    }
-}
-
-// Same per-output summation order (k ascending, one FMA chain) as k_gram, with
-// the K slices staged by cp.async in a GS-deep ring so that GS - 1 slices are in
-// flight while one is consumed.  Tile BM rows (atoms of S) x BN columns (new
-// atoms); each thread computes TR rows x TC columns.  The host takes the
-// narrow 32 x 16 tile when at most 16 atoms arrive per signal (the columns of a
-// wider tile would mostly be empty).  Needs n % 4 == 0 (16-byte rows).
-constexpr int GS = 4, GPAD = GBK + 4;
-
+// G[a][b] for a in [0, s), b in [s0, s) (mirrored): every entry one FMA chain over k ascending, the order
+// of the FP32 GEMM that builds Q, so that the Gram block gathered from Q is the same bits.
+// Tile BM rows (atoms of S) x BN columns (new atoms; their h = a^T b comes with the selection's
+// re-score), TR x TC entries per thread; K slices of BK staged by cp.async in a ring of ST, so that
+// ST - 1 slices are in flight while one is consumed.  A thread's columns are NX apart, so a narrow
+// pass (q - b0 columns) runs with as many of them as it fills; a warp whose rows are all past s
+// only loads.  VEC: rows are 16-byte aligned (n % 4 == 0), else copied word by word.
 __device__ __forceinline__ void cp_async16(float* dst, const float* src, int bytes) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(float* dst, const float* src, int bytes) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(sa), "l"(src), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-template <int BM, int BN, int TR, int TC>
-__global__ void __launch_bounds__(256) k_gram_async(Dev d) {
+// One slice's products for the first NV of a thread's columns.
+template <int NV, int NX, int TR, int TC, int BK>
+__device__ __forceinline__ void gram_slice(const float* Ar, const float* Bt, float (&acc)[TR][TC]) {
+    constexpr int PAD = BK + 4;
+#pragma unroll
+    for (int k = 0; k < BK; k += 4) {
+        float4 x[TR];
+#pragma unroll
+        for (int u = 0; u < TR; ++u) x[u] = *reinterpret_cast<const float4*>(Ar + u * PAD + k);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const float4 y = *reinterpret_cast<const float4*>(Bt + v * NX * PAD + k);
+#pragma unroll
+            for (int u = 0; u < TR; ++u) {
+                acc[u][v] = fmaf(x[u].x, y.x, acc[u][v]);
+                acc[u][v] = fmaf(x[u].y, y.y, acc[u][v]);
+                acc[u][v] = fmaf(x[u].z, y.z, acc[u][v]);
+                acc[u][v] = fmaf(x[u].w, y.w, acc[u][v]);
+            }
+        }
+    }
+}
+
+template <int BM, int BN, int TR, int TC, int BK, int ST, bool VEC>
+__global__ void __launch_bounds__((BM / TR) * (BN / TC)) k_gram(Dev d) {
     pdl_enter();
-    static_assert((BM / TR) * (BN / TC) == 256, "one output block per thread");
+    constexpr int NT = (BM / TR) * (BN / TC);
     constexpr int NX = BN / TC;                  // threads along the columns
-    constexpr int CHUNKS = (BM + BN) * (GBK / 4);  // 16-byte chunks per slice
+    constexpr int PAD = BK + 4;
+    constexpr int CHUNKS = (BM + BN) * (BK / 4);  // 4-entry chunks per slice
+    constexpr int PER = CHUNKS / NT;
+    static_assert(CHUNKS % NT == 0 && 32 % NX == 0 && TC <= 4, "whole chunks per thread, whole rows per warp");
     const int g = blockIdx.x;
     if (g >= d.cnt->grow_n) return;
     const int i = d.list_grow[g];
     const int s = d.ssize[i], q = d.snew[i], s0 = s - q;
     const int a0 = blockIdx.y * BM;
-    if (a0 >= s || q == 0) return;
+    if (a0 >= s || q == 0) return;  // q == 0: a refine pass, the block is complete
     const int n = d.n, smax = d.smax;
     if (blockIdx.y == 0 && threadIdx.x == 0)  // s atom columns read, 2 s q of G written
         atomicAdd(&d.cnt->gram_bytes, 4ull * n * s + 8ull * s * q);
     const int* Si = d.S + (size_t)i * smax;
     float* Gi = d.G + (size_t)i * smax * smax;
-    extern __shared__ __align__(16) float gsm[];
-    float* As = gsm;                            // [GS][BM][GPAD]
-    float* Bs = gsm + (size_t)GS * BM * GPAD;   // [GS][BN][GPAD]
+    extern __shared__ __align__(16) float gsm[];  // [ST][BM + BN][PAD]
     const int tid = threadIdx.x;
     const int ty = tid / NX, tx = tid % NX;
-    const int nsl = (n + GBK - 1) / GBK;
+    const bool rows = a0 + ((tid & ~31) / NX) * TR < s;  // (the same in the whole warp)
+    const int nsl = (n + BK - 1) / BK;
     for (int b0 = 0; b0 < q; b0 += BN) {
-        // source rows of this thread's chunks (c = tid + 256 e), fixed for the column chunk
-        constexpr int PER = (CHUNKS + 255) / 256;
+        // source rows of this thread's chunks (c = tid + NT e), fixed for the column chunk
         const float* src[PER];
-        float* dst0[PER];
 #pragma unroll
         for (int e = 0; e < PER; ++e) {
-            const int c = tid + 256 * e;
-            const int rr = c / (GBK / 4), kc = (c % (GBK / 4)) * 4;
-            const float* p = nullptr;
-            if (c < CHUNKS) {
-                if (rr < BM) {
-                    const int ra = a0 + rr;
-                    p = ra < s ? d.A32 + (size_t)Si[ra] * n : nullptr;
-                } else {
-                    const int rb = b0 + rr - BM;
-                    p = rb < q ? d.A32 + (size_t)Si[s0 + rb] * n : nullptr;
-                }
-            }
-            src[e] = p;
-            dst0[e] = c >= CHUNKS ? nullptr : (rr < BM ? As + (size_t)rr * GPAD + kc : Bs + (size_t)(rr - BM) * GPAD + kc);
+            const int rr = (tid + NT * e) / (BK / 4);
+            const int r = rr < BM ? a0 + rr : s0 + b0 + rr - BM;  // position in S
+            src[e] = r < s ? d.A32 + (size_t)Si[r] * n : nullptr;
         }
         auto issue = [&](int sl) {
-            const int st = sl % GS;
+            float* st = gsm + (size_t)(sl % ST) * (BM + BN) * PAD;
 #pragma unroll
             for (int e = 0; e < PER; ++e) {
-                if (dst0[e] == nullptr) continue;
-                const int c = tid + 256 * e;
-                const int rr = c / (GBK / 4), kc = (c % (GBK / 4)) * 4, k = sl * GBK + kc;
-                float* dst = dst0[e] + (size_t)st * (rr < BM ? BM : BN) * GPAD;
-                const bool ok = src[e] != nullptr && k < n;
-                cp_async16(dst, ok ? src[e] + k : d.A32, ok ? 16 : 0);
+                const int c = tid + NT * e;
+                const int kc = (c % (BK / 4)) * 4, k = sl * BK + kc;
+                float* dst = st + (c / (BK / 4)) * PAD + kc;
+                if (VEC) {
+                    const bool ok = src[e] != nullptr && k < n;
+                    cp_async16(dst, ok ? src[e] + k : d.A32, ok ? 16 : 0);
+                } else {
+#pragma unroll
+                    for (int w = 0; w < 4; ++w) {
+                        const bool ok = src[e] != nullptr && k + w < n;
+                        cp_async4(dst + w, ok ? src[e] + k + w : d.A32, ok ? 4 : 0);
+                    }
+                }
             }
         };
 #pragma unroll
-        for (int sl = 0; sl < GS - 1; ++sl) {
+        for (int sl = 0; sl < ST - 1; ++sl) {
             if (sl < nsl) issue(sl);
             cp_async_commit();
         }
@@ -339,30 +279,21 @@ __global__ void __launch_bounds__(256) k_gram_async(Dev d) {
         for (int u = 0; u < TR; ++u)
 #pragma unroll
             for (int v = 0; v < TC; ++v) acc[u][v] = 0.f;
+        const int nv = rows ? min(TC, (q - b0 + NX - 1) / NX) : 0;
         for (int sl = 0; sl < nsl; ++sl) {
-            cp_async_wait<GS - 2>();
+            cp_async_wait<ST - 2>();
             __syncthreads();
-            if (sl + GS - 1 < nsl) issue(sl + GS - 1);
+            if (sl + ST - 1 < nsl) issue(sl + ST - 1);
             cp_async_commit();
-            const int st = sl % GS;
-            const float* Ar = As + ((size_t)st * BM + ty * TR) * GPAD;
-            const float* Bt = Bs + ((size_t)st * BN + tx) * GPAD;
-#pragma unroll
-            for (int k = 0; k < GBK; k += 4) {
-                float4 x[TR];
-#pragma unroll
-                for (int u = 0; u < TR; ++u) x[u] = *reinterpret_cast<const float4*>(Ar + (size_t)u * GPAD + k);
-#pragma unroll
-                for (int v = 0; v < TC; ++v) {
-                    const float4 y = *reinterpret_cast<const float4*>(Bt + (size_t)v * NX * GPAD + k);
-#pragma unroll
-                    for (int u = 0; u < TR; ++u) {
-                        acc[u][v] = fmaf(x[u].x, y.x, acc[u][v]);
-                        acc[u][v] = fmaf(x[u].y, y.y, acc[u][v]);
-                        acc[u][v] = fmaf(x[u].z, y.z, acc[u][v]);
-                        acc[u][v] = fmaf(x[u].w, y.w, acc[u][v]);
-                    }
-                }
+            const float* st = gsm + (size_t)(sl % ST) * (BM + BN) * PAD;
+            const float* Ar = st + ty * TR * PAD;
+            const float* Bt = st + (BM + tx) * PAD;
+            switch (nv) {
+                case 0: break;
+                case 1: gram_slice<1, NX, TR, TC, BK>(Ar, Bt, acc); break;
+                case 2: gram_slice<2, NX, TR, TC, BK>(Ar, Bt, acc); break;
+                case 3: gram_slice<TC < 3 ? TC : 3, NX, TR, TC, BK>(Ar, Bt, acc); break;
+                default: gram_slice<TC, NX, TR, TC, BK>(Ar, Bt, acc); break;
             }
         }
         cp_async_wait<0>();
@@ -382,9 +313,6 @@ __global__ void __launch_bounds__(256) k_gram_async(Dev d) {
         }
     }
 }
-
-template <int BM, int BN>
-constexpr size_t gram_smem() { return (size_t)GS * (BM + BN) * GPAD * sizeof(float); }
 
 // ------------------------------------------------------------------ APG
 // Blocks of more than APG_REG_S atoms: in shared memory when s <= gcap (<= APG_SMEM_S), else streamed
@@ -1396,39 +1324,49 @@ cudaError_t launch_init(const Dev& d, cudaStream_t s, int64_t* nl) {
     return cudaGetLastError();
 }
 
+// The two tiles: GRAM_L for batches that fill the chip, GRAM_S for the others.
+template <int BM, int BN, int TR, int TC, int BK, int ST>
+static cudaError_t gram_launch(const Dev& d, int ub, int scap, cudaStream_t s, bool prepare) {
+    constexpr size_t sm = (size_t)ST * (BM + BN) * (BK + 4) * sizeof(float);
+    if (prepare) {
+        cudaError_t e = cudaFuncSetAttribute(k_gram<BM, BN, TR, TC, BK, ST, true>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_gram<BM, BN, TR, TC, BK, ST, false>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        return e;
+    }
+    const dim3 grid(ub, (scap + BM - 1) / BM), block((BM / TR) * (BN / TC));
+    return (d.n & 3) == 0 ? launch_chain(k_gram<BM, BN, TR, TC, BK, ST, true>, grid, block, sm, s, d)
+                          : launch_chain(k_gram<BM, BN, TR, TC, BK, ST, false>, grid, block, sm, s, d);
+}
+static cudaError_t gram_large(const Dev& d, int ub, int scap, cudaStream_t s, bool prepare = false) {
+    return gram_launch<64, 64, 4, 4, 32, 4>(d, ub, scap, s, prepare);
+}
+static cudaError_t gram_small(const Dev& d, int ub, int scap, cudaStream_t s, bool prepare = false) {
+    return gram_launch<32, 32, 2, 4, 32, 6>(d, ub, scap, s, prepare);
+}
+
 cudaError_t prepare_gram() {
     static bool attr = false;
     if (attr) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_gram_async<64, 32, 2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)gram_smem<64, 32>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_gram_async<64, 64, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)gram_smem<64, 64>());
+    cudaError_t e = gram_large(Dev{}, 0, 0, nullptr, true);
+    if (e == cudaSuccess) e = gram_small(Dev{}, 0, 0, nullptr, true);
     if (e == cudaSuccess) attr = true;
     return e;
 }
 
-cudaError_t launch_gram(const Dev& d, int ub, int qmax, cudaStream_t s, int64_t* nl) {
+cudaError_t launch_gram(const Dev& d, int ub, int qmax, int scap, int sms, cudaStream_t s, int64_t* nl) {
     if (ub <= 0) return cudaSuccess;
-    if ((d.n & 3) == 0) {
-        cudaError_t ep = prepare_gram();
-        if (ep != cudaSuccess) return ep;
-        if (qmax <= 16) {  // the new atoms fit one 16-column tile
-            dim3 grid(ub, (d.smax + 31) / 32);
-            ep = launch_chain(k_gram_async<32, 16, 1, 2>, grid, dim3(256), gram_smem<32, 16>(), s, d);
-        } else if (qmax <= 64) {  // one 64-column pass (e.g. a warm start's first iteration)
-            dim3 grid(ub, (d.smax + 63) / 64);
-            ep = launch_chain(k_gram_async<64, 64, 4, 4>, grid, dim3(256), gram_smem<64, 64>(), s, d);
-        } else {
-            dim3 grid(ub, (d.smax + 63) / 64);
-            ep = launch_chain(k_gram_async<64, 32, 2, 4>, grid, dim3(256), gram_smem<64, 32>(), s, d);
-        }
-        if (ep != cudaSuccess) return ep;
-    } else {
-        dim3 grid(ub, (d.smax + GBM - 1) / GBM);
-        const cudaError_t eg = launch_chain(k_gram<false>, grid, dim3(256), 0, s, d);
-        if (eg != cudaSuccess) return eg;
-    }
+    cudaError_t e = prepare_gram();
+    if (e != cudaSuccess) return e;
+    // The large tile reads each atom column half as often, and pays where its blocks fill the chip twice
+    // over and its columns are mostly used: 512 signals of 2048 x 32768 gaining 50 atoms each, 2.6 ms a
+    // solve against 3.0 with the small one; 300 gaining 100, 4.5 against 5.9.  Below, the small one:
+    // 1024 x 8192, 512 signals gaining 24, 0.31 ms; 75 signals of 1496 x 20011 gaining 30, 0.23.
+    const bool large = qmax > 32 && (long long)ub * ((scap + 63) / 64) >= 2ll * sms;
+    e = large ? gram_large(d, ub, scap, s) : gram_small(d, ub, scap, s);
+    if (e != cudaSuccess) return e;
     ++*nl;
     return cudaGetLastError();
 }
