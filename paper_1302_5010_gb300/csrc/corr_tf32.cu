@@ -13,7 +13,7 @@
 // A persistent CTA walks output tiles of 128 atoms x w signals.  Roles (five warpgroups):
 //   warps 0-7   loaders: rows of atoms and of the active signals' residuals (gathered through the
 //               active list) are copied asynchronously, as FP32, to where their hi part goes in
-//               one of two stages (128-byte-swizzled tiles); each lane then splits the 16 bytes it
+//               one of two stages (three, a stage ahead, up to 128 signals; 128-byte-swizzled tiles); each lane then splits the 16 bytes it
 //               copied, so that no thread waits for another's copies.
 //   warp 8      allocates TMEM; one thread issues the 12 tcgen05.mma of a stage (kind::tf32,
 //               M = 128, N = w, K = 8) into the stage's accumulator and commits.
@@ -21,7 +21,9 @@
 //               (each warp its 32 atoms and half of the tile's signals); scores stored at the end.
 // setmaxnreg moves registers from the loaders to the accumulating warps.
 //
-// What bounds it: the loaders' instructions.  A stage of a 128 x 256 tile takes 3500 cycles, of
+// What bounds it: the loaders' instructions, and with few signals the latency of their copies and
+// splits, which the third stage overlaps (2048 x 32768: 16 signals 181 -> 124 us, 64 193 -> 141, 128 198 -> 155;
+// 777 x 6001 x 99 55 -> 49 us).  A stage of a 128 x 256 tile takes 3500 cycles, of
 // which the tensor core works 2100 and shared memory (three reads of every operand by
 // the MMAs, the copies and the split: 340 KB) at least 2650.  2044 x 32771 x 500: 480 us
 // (140 TFLOP/s), 4096 x 65536 x 1024: 3.13 ms, 1024 x 8192 x 256: 51 us; the FP32 chain on the SIMT
@@ -46,7 +48,7 @@ namespace {
 constexpr int TF_BM = 128;           // atoms per tile
 constexpr int TF_BN = 256;           // most signals per tile
 constexpr int TF_BK = 32;            // columns of n per stage: one 128-byte swizzle row
-constexpr int TF_STAGES = 2;         // stages, each with its TMEM accumulator
+constexpr int TF_STAGES = 3;         // most stages, each with its TMEM accumulator (see TfTile)
 constexpr int TF_THREADS = 640;
 constexpr int TF_LOADERS = 8;        // loader warps
 constexpr int TF_MMA_WARP = 8;
@@ -58,8 +60,8 @@ constexpr int TF_SLOTS = 8;          // flag slots by tile (the loaders run at m
 constexpr int TF_ROWS = TF_BM + TF_BN;
 
 constexpr int TF_A_BYTES = TF_BM * 128;
-constexpr int TF_HALF_BYTES = TF_ROWS * 128;          // the hi (or lo) tiles: atoms, then signals
-constexpr int TF_STAGE_BYTES = 2 * TF_HALF_BYTES;
+constexpr int TF_RING_BYTES = 4 * TF_ROWS * 128;      // two stages of the widest tile
+constexpr int TF_TMEM = 512;                          // columns: the whole TMEM of the SM
 
 struct TfShared {
     uint64_t full[TF_STAGES];    // the loaders have filled the stage
@@ -73,8 +75,8 @@ struct TfShared {
     unsigned char nan[TF_SLOTS][TF_ROWS];        // ... a NaN
     unsigned char any[TF_SLOTS][8];              // any such row, by loader warp
 };
-constexpr size_t TF_SMEM = (size_t)TF_STAGES * TF_STAGE_BYTES + 1024 + sizeof(TfShared);
-static_assert(TF_SMEM <= 227 * 1024, "two stages and the barriers fit one CTA's shared memory");
+constexpr size_t TF_SMEM = (size_t)TF_RING_BYTES + 1024 + sizeof(TfShared);
+static_assert(TF_SMEM <= 227 * 1024, "the stages and the barriers fit one CTA's shared memory");
 static_assert(TF_ITEMS * TF_STEP == TF_ROWS && TF_STEP % 8 == 0, "every row has one loader");
 
 // Instruction descriptor, kind::tf32: D f32, A/B tf32, both K-major, M x N.
@@ -115,18 +117,36 @@ __device__ __forceinline__ void st_shared4(uint32_t dst, const uint32_t (&v)[4])
                  : "memory");
 }
 
-// Signals per tile (a multiple of 16, at most TF_BN): the count of active signals shrinks from one
-// outer iteration to the next, and a narrower tile costs less.  A stage takes about 576 + w units
-// (2700 cycles measured at w = 64, 3000 at 128, 3500 at 256), and ceil(tiles / grid) tiles run
-// in turn on a CTA.
+// A kernel for at most TF_NARROW signals per tile has three stages in the same ring, and its loaders copy a
+// stage ahead of the one they split.  With two that would make them wait for the MMAs of the stage
+// before, which take about as long as a wide tile's split.
+constexpr int TF_NARROW = 128;
+template <bool NARROW>
+struct TfTile {
+    static constexpr int STAGES = NARROW ? 3 : 2;
+    static constexpr int BN = NARROW ? TF_NARROW : TF_BN;        // most signals
+    static constexpr int ROWS = TF_BM + BN;
+    static constexpr int GROUPS = ROWS / (4 * TF_STEP);          // of four items, per loader warp
+    static constexpr int HALF_BYTES = ROWS * 128;                // the hi (or lo) tiles: atoms, then signals
+    static constexpr int STAGE_BYTES = 2 * HALF_BYTES;
+    static_assert(STAGES * STAGE_BYTES <= TF_RING_BYTES && STAGES * BN <= TF_TMEM && ROWS % (4 * TF_STEP) == 0 &&
+                  STAGES <= TF_STAGES, "the stages fit, in whole groups");
+};
+
+// Signals per tile (a multiple of 16): the count of active signals shrinks from one outer iteration
+// to the next, and a narrower tile costs less.  A stage takes about 576 + w units (2700 cycles
+// measured at w = 64, 3000 at 128, 3500 at 256), 420 + w in the narrow kernel (1900 at 16, 2400 at 128),
+// and ceil(tiles / grid) tiles run in turn on a CTA.
+template <bool NARROW>
 __device__ __forceinline__ int pick_width(int act_n, int tiles_m, int grid) {
-    const int t0 = (act_n + TF_BN - 1) / TF_BN;
-    int best = TF_BN;
+    constexpr int BN = TfTile<NARROW>::BN;
+    const int t0 = (act_n + BN - 1) / BN;
+    int best = BN;
     float cost = 3e38f;
     for (int t = t0; t < t0 + 8; ++t) {
         const int w = (((act_n + t - 1) / t) + 15) / 16 * 16;
         const float tiles = (float)tiles_m * (float)((act_n + w - 1) / w);
-        const float c = ceilf(tiles / (float)grid) * (float)(576 + w);
+        const float c = ceilf(tiles / (float)grid) * (float)((NARROW ? 420 : 576) + w);
         if (c < cost) { cost = c; best = w; }
     }
     return best;
@@ -138,7 +158,7 @@ __device__ __forceinline__ uint32_t tf32_hi(uint32_t x) { return (x + 0x1000u) &
 
 // Four entries of which some may have no split: those keep their upper bits (a NaN stays one) and
 // flag the row.
-__device__ __noinline__ void store_nosplit(float4 v, uint32_t dst, unsigned char* inf, unsigned char* nan) {
+__device__ __noinline__ void store_nosplit(float4 v, uint32_t dst, uint32_t half, unsigned char* inf, unsigned char* nan) {
     const float f[4] = {v.x, v.y, v.z, v.w};
     uint32_t hi[4], lo[4];
 #pragma unroll
@@ -151,29 +171,134 @@ __device__ __noinline__ void store_nosplit(float4 v, uint32_t dst, unsigned char
         if (a > 0x7f800000u) { hi[e] = 0x7fc00000u; *nan = 1; }
     }
     st_shared4(dst, hi);
-    st_shared4(dst + TF_HALF_BYTES, lo);
+    st_shared4(dst + half, lo);
 }
 
-template <bool VEC>
+// A loader warp's part of a tile: the slices' copies, their splits, the stages handed on.  Returns false
+// when a wait expired.  NARROW: at most TF_NARROW signals, three stages, copies a stage ahead.
+template <bool VEC, bool NARROW>
+__device__ __forceinline__ bool load_tile(const Dev& d, TfShared& sh, uint32_t base, const volatile int* abort_flag,
+                                          int warp, int lane, int rows, int slot, int nk, int n, int& stage,
+                                          uint32_t& ph) {
+    constexpr int NST = TfTile<NARROW>::STAGES, GROUPS = TfTile<NARROW>::GROUPS;
+    constexpr uint32_t HALF = TfTile<NARROW>::HALF_BYTES;
+    const int r0 = warp * 4 + (lane >> 3), kc = (lane & 7) * 4;
+    const uint32_t dst0 = base + (uint32_t)(r0 * 128 + (((lane & 7) ^ (r0 & 7)) << 4));
+    // copied as FP32 to where hi goes: each lane splits the 16 bytes it copied, so its own copies are all
+    // it waits for
+    auto copy_group = [&](uint32_t dst, int k, int g) {
+        if (4 * warp + 4 * g * TF_STEP < rows) {  // (the same in all lanes)
+            const float* row[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) row[i] = sh.row[r0 + (4 * g + i) * TF_STEP];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t q = dst + (uint32_t)((4 * g + i) * TF_STEP * 128);
+                // (zeros past the end: a row repeated there instead would be one hot line for every CTA)
+                const bool in = row[i] != nullptr && k < n;
+                if (VEC) copy4_16(q, in ? row[i] + k : d.A32, in ? n - k : 0);
+                else copy4_4(q, in ? row[i] + k : d.A32, in ? n - k : 0);
+            }
+        }
+        copy_commit();
+    };
+    auto split_group = [&](uint32_t dst, int g) {
+        if (4 * warp + 4 * g * TF_STEP >= rows) return;
+        float4 v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = ld_shared4(dst + (uint32_t)((4 * g + i) * TF_STEP * 128));
+        float chk = 0.f;  // NaN once some lo is not finite
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float x[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+            uint32_t hi[4], lo[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                hi[e] = tf32_hi(__float_as_uint(x[e]));
+                const float l = x[e] - __uint_as_float(hi[e]);
+                chk = fmaf(l, 0.f, chk);
+                lo[e] = __float_as_uint(l) + 0x1000u;  // (the tensor core reads the upper bits)
+            }
+            st_shared4(dst + (uint32_t)((4 * g + i) * TF_STEP * 128), hi);
+            st_shared4(dst + (uint32_t)((4 * g + i) * TF_STEP * 128) + HALF, lo);
+        }
+        if (chk != chk) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = r0 + (4 * g + i) * TF_STEP;
+                store_nosplit(v[i], dst + (uint32_t)((4 * g + i) * TF_STEP * 128), HALF, &sh.inf[slot][r],
+                              &sh.nan[slot][r]);
+            }
+            sh.any[slot][warp] = 1;
+        }
+    };
+    // waits for a stage to be free and copies slice kb to it
+    auto copy_stage = [&](int st, uint32_t parity, int kb) {
+        bool free = mbar_wait(&sh.done[st], parity ^ 1u, abort_flag);
+        free = __all_sync(0xffffffffu, free);
+        if (!free) {
+            if (lane == 0) { sh.abort_flag = 1; atomicCAS(&d.cnt->err, 0, (int)DERR_TIMEOUT); }
+            copy_wait<0>();
+            return false;
+        }
+        const uint32_t dst = dst0 + (uint32_t)st * (2u * HALF);
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) copy_group(dst, kb * TF_BK + kc, g);
+        return true;
+    };
+    if (NARROW && !copy_stage(stage, ph, 0)) return false;
+#pragma unroll 1
+    for (int kb = 0; kb < nk; ++kb) {
+        if (NARROW) {
+            if (kb + 1 < nk) {
+                const int nx = stage + 1 == NST ? 0 : stage + 1;
+                if (!copy_stage(nx, nx ? ph : ph ^ 1u, kb + 1)) return false;
+                copy_wait<GROUPS>();
+            } else {
+                copy_wait<0>();
+            }
+        } else if (!copy_stage(stage, ph, kb)) {
+            return false;
+        }
+        const uint32_t dst = dst0 + (uint32_t)stage * (2u * HALF);
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) {
+            if (!NARROW) {
+                if (g == 0) copy_wait<2>();
+                else if (g == 1) copy_wait<1>();
+                else copy_wait<0>();
+            }
+            split_group(dst, g);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sh.full[stage]);
+        if (++stage == NST) { stage = 0; ph ^= 1u; }
+    }
+    return true;
+}
+
+template <bool VEC, bool NARROW>
 __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
     pdl_enter();
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    TfShared& sh = *reinterpret_cast<TfShared*>(base + TF_STAGES * TF_STAGE_BYTES);
+    TfShared& sh = *reinterpret_cast<TfShared*>(base + TF_RING_BYTES);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int act_n = d.cnt->act_n[cur];
     const int m = d.m, n = d.n;
     const int tiles_m = (m + TF_BM - 1) / TF_BM;
     if (act_n <= 0) return;
-    const int w = pick_width(act_n, tiles_m, (int)gridDim.x);
+    const int w = pick_width<NARROW>(act_n, tiles_m, (int)gridDim.x);
     const int tiles_n = (act_n + w - 1) / w;
     const long long ntiles = (long long)tiles_m * tiles_n;
     if ((long long)blockIdx.x >= ntiles) return;  // (the whole CTA, before it holds anything)
     const int nk = (n + TF_BK - 1) / TF_BK;
+    using T = TfTile<NARROW>;
+    constexpr int nst = T::STAGES;
     volatile int* abort_flag = &sh.abort_flag;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < TF_STAGES; ++s) {
+        for (int s = 0; s < nst; ++s) {
             mbar_init(&sh.full[s], TF_LOADERS);
             mbar_init(&sh.done[s], 1);
             mbar_init(&sh.tempty[s], TF_ACC_WARPS);
@@ -184,7 +309,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
     }
     if (warp == TF_MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem)),
-                     "r"(TF_STAGES * TF_BN));
+                     "r"(TF_TMEM));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     fence_before();
@@ -202,9 +327,9 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
         if (warp < TF_LOADERS) {
             // item i of this warp: rows 4 warp + TF_STEP i .. + 3 of [atoms | signals], eight lanes
             // (16 bytes each) per row; in groups of four items, of which a narrow tile takes fewer
-            const int r0 = warp * 4 + (lane >> 3), kc = (lane & 7) * 4;
+            const int r0 = warp * 4 + (lane >> 3);
             const int rows = TF_BM + w;
-            const uint32_t dst0 = smem_u32(base) + (uint32_t)(r0 * 128 + (((lane & 7) ^ (r0 & 7)) << 4));
+            const uint32_t base_u = smem_u32(base);
             int stage = 0;
             uint32_t ph = 0;
             unsigned tcount = 0;
@@ -230,70 +355,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
                 }
                 if (lane == 0) sh.any[slot][warp] = 0;
                 __syncwarp();
-                for (int kb = 0; kb < nk; ++kb) {
-                    ok = mbar_wait(&sh.done[stage], ph ^ 1u, abort_flag);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) { if (lane == 0) give_up(); break; }
-                    // copied as FP32 to where hi goes: each lane splits the 16 bytes it copied, so
-                    // its own copies are all it waits for
-                    const uint32_t dst = dst0 + (uint32_t)(stage * TF_STAGE_BYTES);
-                    const int k = kb * TF_BK + kc;
-#pragma unroll
-                    for (int g = 0; g < TF_ITEMS / 4; ++g) {
-                        if (4 * warp + 4 * g * TF_STEP < rows) {  // (the same in all lanes)
-                            const float* row[4];
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) row[i] = sh.row[r0 + (4 * g + i) * TF_STEP];
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const uint32_t q = dst + (uint32_t)((4 * g + i) * TF_STEP * 128);
-                                // (zeros past the end: a row repeated there instead would be one
-                                // hot line for every CTA)
-                                const bool in = row[i] != nullptr && k < n;
-                                if (VEC) copy4_16(q, in ? row[i] + k : d.A32, in ? n - k : 0);
-                                else copy4_4(q, in ? row[i] + k : d.A32, in ? n - k : 0);
-                            }
-                        }
-                        copy_commit();
-                    }
-#pragma unroll
-                    for (int g = 0; g < TF_ITEMS / 4; ++g) {
-                        if (g == 0) copy_wait<2>();
-                        else if (g == 1) copy_wait<1>();
-                        else copy_wait<0>();
-                        if (4 * warp + 4 * g * TF_STEP >= rows) continue;
-                        float4 v[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) v[i] = ld_shared4(dst + (uint32_t)((4 * g + i) * TF_STEP * 128));
-                        float chk = 0.f;  // NaN once some lo is not finite
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const float x[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
-                            uint32_t hi[4], lo[4];
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                hi[e] = tf32_hi(__float_as_uint(x[e]));
-                                const float l = x[e] - __uint_as_float(hi[e]);
-                                chk = fmaf(l, 0.f, chk);
-                                lo[e] = __float_as_uint(l) + 0x1000u;  // (the tensor core reads the upper bits)
-                            }
-                            st_shared4(dst + (uint32_t)((4 * g + i) * TF_STEP * 128), hi);
-                            st_shared4(dst + (uint32_t)((4 * g + i) * TF_STEP * 128 + TF_HALF_BYTES), lo);
-                        }
-                        if (chk != chk) {
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const int r = r0 + (4 * g + i) * TF_STEP;
-                                store_nosplit(v[i], dst + (uint32_t)((4 * g + i) * TF_STEP * 128), &sh.inf[slot][r],
-                                              &sh.nan[slot][r]);
-                            }
-                            sh.any[slot][warp] = 1;
-                        }
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sh.full[stage]);
-                    if (++stage == TF_STAGES) { stage = 0; ph ^= 1u; }
-                }
+                ok = load_tile<VEC, NARROW>(d, sh, base_u, abort_flag, warp, lane, rows, slot, nk, n, stage, ph);
             }
         } else if (warp == TF_MMA_WARP && lane == 0) {
             const uint32_t idesc = idesc_tf32(TF_BM, w);
@@ -312,11 +374,11 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
                     // tensor core here
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     fence_after();
-                    const uint8_t* sb = base + stage * TF_STAGE_BYTES;
+                    const uint8_t* sb = base + stage * T::STAGE_BYTES;
                     const uint64_t ah = sdesc_sw128(sb), bh = sdesc_sw128(sb + TF_A_BYTES);
-                    const uint64_t al = sdesc_sw128(sb + TF_HALF_BYTES);
-                    const uint64_t bl = sdesc_sw128(sb + TF_HALF_BYTES + TF_A_BYTES);
-                    const uint32_t dt = tmem + (uint32_t)(stage * TF_BN);
+                    const uint64_t al = sdesc_sw128(sb + T::HALF_BYTES);
+                    const uint64_t bl = sdesc_sw128(sb + T::HALF_BYTES + TF_A_BYTES);
+                    const uint32_t dt = tmem + (uint32_t)(stage * T::BN);
 #pragma unroll
                     for (int k = 0; k < TF_BK / 8; ++k) {  // 8 columns of n: 32 bytes along the swizzle row
                         const uint64_t off = (uint64_t)((k * 32) >> 4);
@@ -329,7 +391,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
                         mma_tf32(dt, ah + off, bh + off, idesc, 1u);
                     }
                     mma_commit(&sh.done[stage]);
-                    if (++stage == TF_STAGES) { stage = 0; ph ^= 1u; }
+                    if (++stage == nst) { stage = 0; ph ^= 1u; }
                 }
             }
             if (*abort_flag) {
@@ -350,9 +412,9 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
         bool ok = true;
         for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tcount) {
             const int tm = (int)(t / tiles_n), tn = (int)(t - (long long)tm * tiles_n);
-            float acc[TF_BN / 32][16];
+            float acc[T::BN / 32][16];
 #pragma unroll
-            for (int i = 0; i < TF_BN / 32; ++i)
+            for (int i = 0; i < T::BN / 32; ++i)
 #pragma unroll
                 for (int e = 0; e < 16; ++e) acc[i][e] = 0.f;
             for (int kb = 0; kb < nk; ++kb) {
@@ -361,9 +423,9 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
                 ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
                 if (!ok) { if (lane == 0) give_up(); break; }
                 fence_after();
-                const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(stage * TF_BN);
+                const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(stage * T::BN);
 #pragma unroll
-                for (int i = 0; i < TF_BN / 32; ++i) {
+                for (int i = 0; i < T::BN / 32; ++i) {
                     if (2 * i + grp < nblk) {
                         float v[16];
                         tmem_ld16(tb + (uint32_t)((2 * i + grp) * 16), v);
@@ -374,7 +436,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
                 fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sh.tempty[stage]);
-                if (++stage == TF_STAGES) { stage = 0; ph ^= 1u; }
+                if (++stage == nst) { stage = 0; ph ^= 1u; }
             }
             if (!ok) break;
             const int slot = tcount & (TF_SLOTS - 1);
@@ -384,7 +446,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
 #pragma unroll
             for (int l = 0; l < TF_LOADERS; ++l) flagged |= sh.any[slot][l] != 0;
 #pragma unroll
-            for (int i = 0; i < TF_BN / 32; ++i) {
+            for (int i = 0; i < T::BN / 32; ++i) {
                 if (2 * i + grp < nblk) {
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
@@ -417,21 +479,21 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
     __syncthreads();
     fence_after();
     if (warp == TF_MMA_WARP) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TF_STAGES * TF_BN));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TF_TMEM));
     }
 }
 
 // The registers that setmaxnreg hands out come from the launch's own: 5 x 128 threads at numRegs.
 bool regs_cover(const cudaFuncAttributes& a) { return 5 * a.numRegs >= 2 * TF_REGS_ACC + 3 * TF_REGS_LOAD; }
 
-template <bool VEC>
+template <bool VEC, bool NARROW>
 cudaError_t launch_t(const Dev& d, int cur, int act_n_ub, cudaStream_t s) {
     // (per launch: the attribute belongs to the current context; about a microsecond of host time)
     cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, k_corr_tf32<VEC>);
+    cudaError_t e = cudaFuncGetAttributes(&fa, k_corr_tf32<VEC, NARROW>);
     if (e != cudaSuccess) return e;
     if (!regs_cover(fa)) return cudaErrorNotSupported;
-    e = cudaFuncSetAttribute(k_corr_tf32<VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TF_SMEM);
+    e = cudaFuncSetAttribute(k_corr_tf32<VEC, NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TF_SMEM);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -439,13 +501,16 @@ cudaError_t launch_t(const Dev& d, int cur, int act_n_ub, cudaStream_t s) {
     // one CTA per SM; tiles of 16 signals are the narrowest
     const long long tiles = (long long)((d.m + TF_BM - 1) / TF_BM) * ((act_n_ub + 15) / 16);
     const int grid = (int)(tiles < sms ? tiles : sms);
-    return launch_chain(k_corr_tf32<VEC>, dim3(grid), dim3(TF_THREADS), TF_SMEM, s, d, cur);
+    return launch_chain(k_corr_tf32<VEC, NARROW>, dim3(grid), dim3(TF_THREADS), TF_SMEM, s, d, cur);
 }
 
 }  // namespace
 
 cudaError_t launch_corr_tf32(const Dev& d, int cur, int act_n_ub, cudaStream_t s, int64_t* nl) {
-    const cudaError_t e = (d.n & 3) == 0 ? launch_t<true>(d, cur, act_n_ub, s) : launch_t<false>(d, cur, act_n_ub, s);
+    // (one wide tile beats two narrow ones: 2048 x 32768 x 256 245 us against 320)
+    const bool narrow = act_n_ub <= TF_NARROW, vec = (d.n & 3) == 0;
+    const cudaError_t e = narrow ? (vec ? launch_t<true, true>(d, cur, act_n_ub, s) : launch_t<false, true>(d, cur, act_n_ub, s))
+                                 : (vec ? launch_t<true, false>(d, cur, act_n_ub, s) : launch_t<false, false>(d, cur, act_n_ub, s));
     if (e != cudaSuccess) return e;
     ++*nl;
     return cudaSuccess;

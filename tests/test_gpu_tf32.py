@@ -82,3 +82,16 @@ def test_non_finite_values(n, m, p):
     At2, R2 = _data(n, m, p, n)
     clean = np.ix_([i for i in range(p) if i not in (3, 7, 8, 9, 17)], [j for j in range(m) if j not in (10, 11, 12, 13)])
     np.testing.assert_array_equal(C[clean], _noalloc(At2, R2)[clean])
+
+
+@pytest.mark.parametrize("n,m,p", [(130, 20000, 128), (192, 20001, 65), (225, 39000, 16), (256, 20100, 129)])
+def test_several_tiles_per_block(n, m, p):
+    """Up to 128 signals take three stages: slices that are 2, 0 and 2 modulo 3, so that consecutive
+    tiles of a block start in different stages; 129 signals take the wide kernel's two.  Bound as above."""
+    At, R = _data(n, m, p, n + m + p)
+    C = _noalloc(At, R).astype(np.float64)
+    exact = R.astype(np.float64) @ At.astype(np.float64).T
+    absdot = np.abs(R.astype(np.float64)) @ np.abs(At.astype(np.float64)).T
+    tf = 98.0 * 2.0 ** -22 + (n / 32.0 + 2.0) * 2.0 ** -24
+    assert np.all(np.abs(C - exact) <= tf * absdot)
+    assert np.linalg.norm(C - exact) <= 2.0 ** -19 * np.linalg.norm(exact)
