@@ -67,7 +67,8 @@ typedef enum {
     MPL_OPT_PROFILE = 8,    /* 1: record per-phase device times (mpl_get_phase_times) with
                                timing events, inside the captured graphs too. default 0 */
     MPL_OPT_GRAPH = 9,      /* 1: each outer iteration is replayed from a captured CUDA graph
-                               (captured on first use per batch size and iteration). default 1 */
+                               (captured on first use per batch size and iteration), until at
+                               most a quarter of the signals is active. default 1 */
     MPL_OPT_WARM_CANDIDATES = 10, /* W: atoms per signal scored by the proposal network (the W
                                      largest |a_j^T b| of the first correlation; the rho largest
                                      violators join S anyway, the network picks among the

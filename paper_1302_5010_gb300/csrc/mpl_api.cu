@@ -916,6 +916,7 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
     // have not come back yet); grids are sized by it outside graph mode (captured graphs are
     // sized for p)
     int live = p;
+    int act = p;  // an upper bound on the signals active in the next iteration
     // every finish hands its work back through reent[] of its list slot; an iteration merges
     // the finishes that are done by its start and waits only for the one whose slot it reuses
     // (FIN_SLOTS iterations on), so a retry takes at least two iterations
@@ -969,10 +970,11 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
         }
         drain = false;
         if (mask) CK(launch_merge(d, t & 1, mask, back, st, &nl));
+        act = std::min(act + back, p);
 #ifdef MPL_TIMELINE
         mark(0, st);
 #endif
-        if (graph) {
+        if (graph && 4 * (long long)act > p) {
             size_t gi = 0;
             CK(iteration_graph(h, d, t, p, tol, st, &gi));
             CK(cudaGraphLaunch(h->graphs[gi].exec, st));
@@ -986,7 +988,13 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
                 }
             }
         } else {
-            CK(launch_iteration(h, d, t, live, st, &pt, &nl));
+            // Few signals left: grids and kernels for them, launched one by one, instead of the graph's
+            // for all p.  A quarter is where the kernels for fewer signals begin to differ (an FP32
+            // correlation of 2048 x 32768: 470 us for 512 signals' tiles, 155 for 128, 45 by
+            // matrix-vector products up to 8); a launch is 2 us of the host, which is ahead.  512 such signals in
+            // FP32 10.57 -> 10.04 ms, 1024 x 8192 x 256 1.147 -> 1.095; BF16 batches the same.
+            // (At least one: the host waits for the lists of every iteration.)
+            CK(launch_iteration(h, d, t, std::max(act, 1), st, graph && !h->profile ? nullptr : &pt, &nl));
         }
 #ifdef MPL_TIMELINE
         mark(2, st);
@@ -1025,7 +1033,8 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
         // active next iteration, plus the signals of the finishes not merged yet
         int in_fin = 0;
         for (int q = 0; q < FIN_SLOTS; ++q) in_fin += pend[q] ? pend_n[q] : 0;
-        live = v.act_next + in_fin;
+        act = v.act_next;
+        live = act + in_fin;
         if (v.act_next == 0 && in_fin > 0) {
             // nothing left to iterate on but finishes in flight.  Their signals come back for the
             // worst-case analysis, so the next iteration is queued behind them; under an
