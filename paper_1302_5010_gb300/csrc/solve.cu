@@ -60,16 +60,42 @@ __device__ __forceinline__ float block_sum_after_barrier(float v, float* red) {
     return t;
 }
 
-__device__ __forceinline__ double block_sum_d(double v, double* red) {
+// Sums of four values over the CTA, in part[0..4) for the threads of warp 0.  FP64 instructions take two
+// lanes a cycle on an SM: each level of the butterfly halves the values a lane carries, and one
+// warp adds the warps' totals (part: 4 per warp).  Fixed order.
+__device__ __forceinline__ void block_sum4_d(double (&v)[4], double* part) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int h = 2, o = 16; h; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+            const double send = up ? v[q] : v[q + h];
+            v[q] = (up ? v[q + h] : v[q]) + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+#pragma unroll
+    for (int o = 4; o; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    // lane 8 q holds the warp's total of value q (bits 16, 8 of the lane: 2, 1 of q)
+    if ((lane & 7) == 0) part[warp * 4 + (lane >> 3)] = v[0];
     __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    double t = 0.0;
-    for (int w = 0; w < nw; ++w) t += red[w];
-    return t;
+    if (warp == 0) {
+        double t = 0.0;
+        for (int w = lane >> 2; w < nw; w += 8) t += part[w * 4 + (lane & 3)];
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        __syncwarp();
+        if (lane < 4) part[lane] = t;
+        __syncwarp();
+    }
+}
+
+// s += x x in double-FP32 (the product exact, the sum to 2^-46).
+__device__ __forceinline__ void add_square(float x, float& hi, float& lo) {
+    const float p = x * x, e = fmaf(x, x, -p);
+    const float t = hi + p, z = t - hi;
+    lo += ((hi - (t - z)) + (p - z)) + e;
+    hi = t;
 }
 
 __device__ __forceinline__ float softf(float v, float t) {
@@ -86,7 +112,10 @@ __global__ void __launch_bounds__(256) k_init(Dev d) {
     const float* b = d.B + (size_t)i * n;
     float* r32 = d.R32 + (size_t)i * n;
     double* r64 = d.R64 + (size_t)i * n;
-    double ss = 0.0, es = 0.0, ts = 0.0;
+    // ||b||^2 in FP64; the rounding terms, which feed bounds with a margin of 1e-6, in pairs of floats (a third
+    // of the FP64 work; with the sums below 2048 signals of 1024 entries 73 -> 31 us, 256 of them 14.5 -> 8.4)
+    double ss = 0.0;
+    float eh = 0.f, el = 0.f, th = 0.f, tl = 0.f;
     int nf = 0;
     // entries k = tid + j nt in order of j; four loads in flight before their stores
     for (int k0 = threadIdx.x; k0 < n; k0 += 4 * blockDim.x) {
@@ -109,17 +138,32 @@ __global__ void __launch_bounds__(256) k_init(Dev d) {
             if (d.R16) d.R16[(size_t)i * n + k] = q;
             if (d.pos) d.R16c[(size_t)i * n + k] = q;  // active list = identity
             ss += (double)v * (double)v;
-            const double fq = (double)__bfloat162float(q), e = (double)v - fq;
-            es += e * e;
-            ts += fq * fq;
+            const float fq = __bfloat162float(q);
+            add_square(v - fq, eh, el);  // (the difference is exact)
+            add_square(fq, th, tl);
         }
     }
     uint32_t* mw = d.mask + (size_t)i * d.mw;
     for (int w = threadIdx.x; w < d.mw; w += blockDim.x) mw[w] = 0u;
     nf = __syncthreads_or(nf);
-    const double bb = block_sum_d(ss, red);
-    const double ee = block_sum_d(es, red);
-    const double tt = block_sum_d(ts, red);
+    double sums[4] = {ss, (double)eh + (double)el, (double)th + (double)tl, 0.0};
+    __shared__ double part[32];
+    block_sum4_d(sums, part);
+    __syncthreads();
+    const double bb = part[0];
+    double ee = part[1], tt = part[2];
+    if (!(bb >= 1e-20 && bb <= 1e30)) {
+        // squares outside FP32's range (or no number at all): the same sums in FP64
+        double s2[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int k = threadIdx.x; k < n; k += blockDim.x) {
+            const double fq = (double)__bfloat162float(__float2bfloat16_rn(b[k])), e = (double)b[k] - fq;
+            s2[0] += e * e;
+            s2[1] += fq * fq;
+        }
+        block_sum4_d(s2, red);
+        ee = red[0];  // (used by thread 0)
+        tt = red[1];
+    }
     if (threadIdx.x == 0) {
         d.r16e[i] = __double2float_ru(sqrt(ee) * (1.0 + 1e-6));
         d.r16t[i] = __double2float_ru(sqrt(tt) * (1.0 + 1e-6));
