@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
 bool regs_cover(const cudaFuncAttributes& a) { return 5 * a.numRegs >= 2 * TF_REGS_ACC + 3 * TF_REGS_LOAD; }
 
 template <bool VEC, bool NARROW>
-cudaError_t launch_t(const Dev& d, int cur, int act_n_ub, cudaStream_t s) {
+cudaError_t launch_t(const Dev& d, int cur, int act_n_ub, int sms, cudaStream_t s) {
     // (per launch: the attribute belongs to the current context; about a microsecond of host time)
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, k_corr_tf32<VEC, NARROW>);
@@ -495,9 +495,6 @@ cudaError_t launch_t(const Dev& d, int cur, int act_n_ub, cudaStream_t s) {
     if (!regs_cover(fa)) return cudaErrorNotSupported;
     e = cudaFuncSetAttribute(k_corr_tf32<VEC, NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TF_SMEM);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     // one CTA per SM; tiles of 16 signals are the narrowest
     const long long tiles = (long long)((d.m + TF_BM - 1) / TF_BM) * ((act_n_ub + 15) / 16);
     const int grid = (int)(tiles < sms ? tiles : sms);
@@ -507,10 +504,16 @@ cudaError_t launch_t(const Dev& d, int cur, int act_n_ub, cudaStream_t s) {
 }  // namespace
 
 cudaError_t launch_corr_tf32(const Dev& d, int cur, int act_n_ub, cudaStream_t s, int64_t* nl) {
-    // (one wide tile beats two narrow ones: 2048 x 32768 x 256 245 us against 320)
-    const bool narrow = act_n_ub <= TF_NARROW, vec = (d.n & 3) == 0;
-    const cudaError_t e = narrow ? (vec ? launch_t<true, true>(d, cur, act_n_ub, s) : launch_t<false, true>(d, cur, act_n_ub, s))
-                                 : (vec ? launch_t<true, false>(d, cur, act_n_ub, s) : launch_t<false, false>(d, cur, act_n_ub, s));
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    // The narrow kernel where its tiles run side by side (1024 x 8192 x 256: 50 -> 46 us, the solve 1.084 -> 1.052 ms); else one wide tile
+    // beats two narrow ones in turn (2048 x 32768 x 256: 245 us against 320).
+    const long long tiles_m = (d.m + TF_BM - 1) / TF_BM;
+    const bool narrow = act_n_ub <= TF_NARROW || tiles_m * ((act_n_ub + TF_NARROW - 1) / TF_NARROW) <= sms;
+    if ((d.n & 3) == 0) e = narrow ? launch_t<true, true>(d, cur, act_n_ub, sms, s) : launch_t<true, false>(d, cur, act_n_ub, sms, s);
+    else e = narrow ? launch_t<false, true>(d, cur, act_n_ub, sms, s) : launch_t<false, false>(d, cur, act_n_ub, sms, s);
     if (e != cudaSuccess) return e;
     ++*nl;
     return cudaSuccess;

@@ -84,10 +84,12 @@ def test_non_finite_values(n, m, p):
     np.testing.assert_array_equal(C[clean], _noalloc(At2, R2)[clean])
 
 
-@pytest.mark.parametrize("n,m,p", [(130, 20000, 128), (192, 20001, 65), (225, 39000, 16), (256, 20100, 129)])
+@pytest.mark.parametrize("n,m,p", [(130, 20000, 128), (192, 20001, 65), (225, 39000, 16), (256, 20100, 129),
+                                   (161, 20000, 257), (300, 19999, 512)])
 def test_several_tiles_per_block(n, m, p):
-    """Up to 128 signals take three stages: slices that are 2, 0 and 2 modulo 3, so that consecutive
-    tiles of a block start in different stages; 129 signals take the wide kernel's two.  Bound as above."""
+    """Up to 128 signals, and more where their tiles run side by side, take three stages: slices that are
+    2, 0 and 2 modulo 3, so that consecutive
+    tiles of a block start in different stages; the others take the wide kernel's two.  Bound as above."""
     At, R = _data(n, m, p, n + m + p)
     C = _noalloc(At, R).astype(np.float64)
     exact = R.astype(np.float64) @ At.astype(np.float64).T
