@@ -317,8 +317,10 @@ def kernel_rooflines(P, precision: int, phase: dict, work: dict, pk: dict, sms: 
     cols = work["gemm_columns"]
     flops = 2.0 * P.n * P.m * cols
     if precision == 0:
-        out["correlation"] = entry("k_corr_f32", "alu", flops, phase["correlation"], fp32_peak, "TFLOP/s",
-                                   fp32_note, "flop_per_step")
+        # every FP32 product is three TF32 ones, at half the BF16 rate each
+        out["correlation"] = entry("k_corr_tf32", "tensor", flops, phase["correlation"], pk["bf16_tflops"] / 6.0,
+                                   "TFLOP/s", f"dense bf16 burst / 6 (split TF32), of {pk['source']}",
+                                   "flop_per_step")
     else:
         out["correlation"] = entry("k_corr_bf16", "tensor", flops, phase["correlation"], pk["bf16_tflops"],
                                    "TFLOP/s", f"dense bf16 burst, of {pk['source']}", "flop_per_step")
@@ -335,13 +337,13 @@ def kernel_rooflines(P, precision: int, phase: dict, work: dict, pk: dict, sms: 
                               "bytes_per_step")
     else:
         out["master"] = entry("k_apg", "alu", 2.0 * work["apg_elems"], phase["master"], fp32_peak, "TFLOP/s",
-                              fp32_note + "; Gram blocks resident in shared memory", "flop_per_step")
+                              fp32_note + "; Gram blocks resident in registers or shared memory", "flop_per_step")
     out["selection"] = entry("k_select", "hbm", 4.0 * P.m * cols, phase["selection"], hbm, "GB/s",
                              hbm_note + "; one read of the score rows (the re-score band and any second "
                                         "pass come on top)", "bytes_per_step")
     out["residual"] = entry("k_residual", "hbm", work["residual_bytes"], phase["residual"], hbm, "GB/s",
                             hbm_note, "bytes_per_step")
-    out["gram"] = entry("k_gram_gather" if work["qgram"] else "k_gram_async", "hbm", work["gram_bytes"],
+    out["gram"] = entry("k_gram_gather" if work["qgram"] else "k_gram", "hbm", work["gram_bytes"],
                         phase["gram"], hbm, "GB/s", hbm_note, "bytes_per_step")
     return out
 

@@ -1,5 +1,7 @@
 // Worst-case analysis of Algorithm 1 for all active signals at once:
-// the correlation scores C = A^T R, computed in plain FP32 on the SIMT cores.
+// the correlation scores C = A^T R, computed in plain FP32 on the SIMT cores: the chain that builds Q
+// (whose bits the computed Gram block shares) and correlates signals of fewer than TF32_MIN_N entries;
+// longer ones go to the tensor cores in split TF32, a few signals to the matrix-vector route.
 //
 // C row k holds the m scores of signal act[k]: C[k*m + j] = a_j^T r_{act[k]}.
 // Both operands are K-major in HBM (atoms and residuals are n-contiguous), so a

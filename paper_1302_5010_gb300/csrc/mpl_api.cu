@@ -2,7 +2,7 @@
 // workspace and the outer loop of Algorithm 1 over all signals (Sec. 3).
 //
 // One outer iteration, for the signals still active:
-//   correlation  C = A^T R                       (FP32 SIMT or BF16 tcgen05)
+//   correlation  C = A^T R                       (split TF32 or BF16 tcgen05, or matrix-vector)
 //   selection    top-rho violators, stop test     (k_select, k_compact)
 //   growth       Gram rows A_S^T A_J, h_J         (k_gram)
 //   finish       FP64 exact finish / certificate  (k_finish, signals w/o violators)
