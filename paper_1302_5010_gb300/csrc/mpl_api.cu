@@ -1177,7 +1177,9 @@ static mpl_status_t ensure_rownorms(mpl_ctx* h, cudaStream_t st) {
     d.A32 = h->A32;
     CK(launch_sketch_rownorm(h->A32, h->n, h->m, T, d.R32, st, &nl));
     CK(launch_prep_correlate(d, d.R32, st, &nl));  // identity column list (R32 copies onto itself)
-    CK(launch_corr_f32(d, 0, T, st, &nl));
+    // (one FMA chain per entry, not the split TF32 that scores signals: training amplifies a change of the
+    // feature's last bits to 1e-2 of the weights, and the sketch runs once per dictionary)
+    CK(launch_corr_chain(d, 0, T, st, &nl));
     CK(launch_rownorm(d.Cs, h->m, T, h->rn, st, &nl));
     CK(cudaStreamSynchronize(st));
     h->rn_ready = true;
