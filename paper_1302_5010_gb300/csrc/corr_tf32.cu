@@ -26,7 +26,7 @@
 // 777 x 6001 x 99 55 -> 49 us).  A stage of a 128 x 256 tile takes 3500 cycles, of
 // which the tensor core works 2100 and shared memory (three reads of every operand by
 // the MMAs, the copies and the split: 340 KB) at least 2650.  2044 x 32771 x 500: 480 us
-// (140 TFLOP/s), 4096 x 65536 x 1024: 3.13 ms, 1024 x 8192 x 256: 51 us; the FP32 chain on the SIMT
+// (140 TFLOP/s), 4096 x 65536 x 1024: 3.13 ms, 1024 x 8192 x 256: 46 us (three stages); the FP32 chain on the SIMT
 // cores takes 1596 us, 12.2 ms and 162 us.  Loads staged in registers (592 us), six loader warps
 // (507 us) and more, shorter stages with the copies issued ahead (557 to 650 us) were slower.
 // Error against FP64 (2-norm, Gaussian data): 1.3e-7 at n = 128, 2.4e-7 at n = 4096, the chain's
