@@ -376,8 +376,8 @@ __device__ unsigned radix_kth(K key, int m, int kth, SelSmem& sh) {
     return prefix;
 }
 
-// Key of the kth largest cached key without a histogram, for kth <= 512 (one
-// thread per key of the short list below).  Each thread's largest key is known
+// Key of the kth largest cached key without a histogram, for kth of at most 32 per
+// warp that owns keys.  Each thread's largest key is known
 // from fill_cache.  Let jw = ceil(kth / warps); every warp has jw threads whose
 // largest key is at least the warp's jw-th largest thread maximum, so at least
 // kth distinct keys are >= T = the minimum of those over the warps: T is a lower
@@ -385,13 +385,15 @@ __device__ unsigned radix_kth(K key, int m, int kth, SelSmem& sh) {
 // count.)  The keys >= T (with their atoms) go to a list
 // in sh.key as (key << 32 | j); the kth largest is the entry with exactly
 // kth - 1 entries above it.  Returns false (the caller takes the radix passes)
-// when T is 0 or the list has more than blockDim.x entries.  On success *tlo = T
+// when a warp would have to name more than its 32 thread maxima, when T is 0, or when
+// the list has fewer than kth or more than blockDim.x entries.  On success *tlo = T
 // and *below = the largest key < T (for the bound on the atoms left out).
 __device__ bool fast_kth(const unsigned* keys, int m, int kth, unsigned tmax, SelSmem& sh, unsigned* kkey,
                          unsigned* tlo, unsigned* below) {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
     const int nw = min(nt >> 5, (m + 127) >> 7);  // warps that own keys (four per thread and round)
     const int jw = (kth + nw - 1) / nw;
+    if (jw > 32) return false;
     unsigned v = tmax;
     if (jw == 1) {
 #pragma unroll
@@ -438,7 +440,7 @@ __device__ bool fast_kth(const unsigned* keys, int m, int kth, unsigned tmax, Se
     if (lane == 0 && omax) atomicMax(&sh.outmax, omax);
     __syncthreads();
     const unsigned c = sh.lcnt;
-    if (c > (unsigned)nt) return false;  // uniform
+    if (c > (unsigned)nt || c < (unsigned)kth) return false;  // uniform
     if (tid < (int)c) {
         const unsigned long long e = sh.key[tid];
         unsigned above = 0;
@@ -532,7 +534,7 @@ __device__ bool fast_kth_row(K key, const float* row, const uint32_t* msk, int m
     if (lane == 0 && omax) atomicMax(&sh.outmax, omax);
     __syncthreads();
     const unsigned c = sh.lcnt;
-    if (c > (unsigned)nt) return false;
+    if (c > (unsigned)nt || c < (unsigned)kth) return false;
     if (tid < (int)c) {
         const unsigned long long e = sh.key[tid];
         unsigned above = 0;
@@ -556,8 +558,8 @@ __device__ bool fast_kth_row(K key, const float* row, const uint32_t* msk, int m
 // can hold a key the band takes, and those chunks' keys at or above TL form the list: the
 // keys >= T at the front of sh.key (their rank gives the kth largest), those in [TL, T)
 // behind them.
-// Returns false (the row path) when more than SEL_KCAP chunks qualify, more than blockDim.x
-// keys are >= T, or the list overflows.  On success as fast_kth_row.
+// Returns false (the row path) when more than SEL_KCAP chunks qualify, fewer than kth or more than
+// blockDim.x keys are >= T, or the list overflows.  On success as fast_kth_row.
 #ifdef MPL_SEL_TRACE
 #define CK_TRACE(sig, w, a, b, c) do { if (threadIdx.x == 0 && (sig) < 8192) { g_sel_trace[sig][16] = (w); g_sel_trace[sig][17] = (a); g_sel_trace[sig][18] = (b); g_sel_trace[sig][19] = (c); } } while (0)
 #else
@@ -665,7 +667,7 @@ __device__ bool fast_kth_chunks(const float* row, const uint32_t* msk, int m, co
     if (lane == 0 && omax) atomicMax(&sh.outmax, omax);
     __syncthreads();
     const unsigned c = sh.lcnt, cl = sh.vc;
-    if (c > (unsigned)nt || cl > (unsigned)(SEL_KCAP - nt)) { CK_TRACE(sig, 4, c, cl, cc); return false; }  // uniform
+    if (c > (unsigned)nt || c < (unsigned)kth || cl > (unsigned)(SEL_KCAP - nt)) { CK_TRACE(sig, 4, c, cl, cc); return false; }  // uniform
     CK_TRACE(sig, 0, c, cl, cc);
     if (tid < (int)c) {
         const unsigned long long e = sh.key[tid];
