@@ -34,7 +34,9 @@
 //
 // Inputs at or near overflow (infinities, NaN, |x| >= 2^128 (1 - 2^-12)) have no split: their rows
 // are flagged and the affected scores recomputed with one FP32 FMA chain over n, so that a
-// score is infinite or NaN where the FP32 product is.
+// score is infinite or NaN where the FP32 product is.  2044 x 32771 x 500: 1.64 ms with one infinite
+// atom, 1.40 with one infinite signal, 6.6 with all of them (0.48 without; the SIMT kernel always 1.60;
+// one chain at a time 18, 2.3 and 197).
 //
 // Every wait is bounded; on expiry the CTA records DERR_TIMEOUT, the MMA thread waits (bounded) for
 // the MMAs it issued, and the CTA frees its TMEM and returns.
@@ -74,6 +76,7 @@ struct TfShared {
     unsigned char inf[TF_SLOTS][TF_ROWS];        // the row holds a value without a split
     unsigned char nan[TF_SLOTS][TF_ROWS];        // ... a NaN
     unsigned char any[TF_SLOTS][8];              // any such row, by loader warp
+    alignas(16) float chain[TF_ACC_WARPS][16 * 32];  // 32 columns of 16 signals (chain_block)
 };
 constexpr size_t TF_SMEM = (size_t)TF_RING_BYTES + 1024 + sizeof(TfShared);
 static_assert(TF_SMEM <= 227 * 1024, "the stages and the barriers fit one CTA's shared memory");
@@ -277,6 +280,64 @@ __device__ __forceinline__ bool load_tile(const Dev& d, TfShared& sh, uint32_t b
     return true;
 }
 
+// Scores of a warp's 32 atoms (one a lane) and 16 signals from k0 on that involve a value without a split,
+// and no NaN (whose products are NaN already): one FP32 FMA chain over n each.  a_inf, a_nan: the lane's
+// atom; inf, nan: the signals; rs: 16 x 32 floats of shared memory, the warp's own.  What bounds it is the
+// round trip to memory, so 32 columns of everything are read at once: a cache line of its atom
+// per lane, and the signals' rows through rs.  All 16 chains of a lane run together, whichever are wanted.
+template <bool VEC>
+__device__ __noinline__ void chain_block(const float* __restrict__ A, const float* __restrict__ R, const int* act,
+                                         float* C, int n, int m, int atom, bool a_inf, bool a_nan,
+                                         const unsigned char* inf, const unsigned char* nan, int k0, int act_n,
+                                         float* rs) {
+    const int lane = threadIdx.x & 31;
+    const bool mine = atom < m && !a_nan;
+    const unsigned snan = __ballot_sync(0xffffffffu, lane < 16 && nan[lane & 15] != 0);
+    const unsigned sinf = __ballot_sync(0xffffffffu, lane < 16 && inf[lane & 15] != 0) & ~snan;
+    if (!__any_sync(0xffffffffu, mine && (a_inf || sinf != 0u))) return;
+    const float* a = A + (size_t)min(atom, m - 1) * n;
+    const int sig = act[min(k0 + (lane & 15), act_n - 1)];
+    float s[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) s[e] = 0.f;
+#pragma unroll 1
+    for (int x0 = 0; x0 < n; x0 += 32) {
+        float av[32];
+        if (VEC) {
+#pragma unroll
+            for (int q = 0; q < 32; q += 4) {
+                const float4 v = x0 + q < n ? __ldg(reinterpret_cast<const float4*>(a + x0 + q))
+                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+                av[q] = v.x; av[q + 1] = v.y; av[q + 2] = v.z; av[q + 3] = v.w;
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 32; ++q) av[q] = x0 + q < n ? __ldg(a + x0 + q) : 0.f;
+        }
+        float rv[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const int i = __shfl_sync(0xffffffffu, sig, e);
+            rv[e] = x0 + lane < n ? __ldg(R + (size_t)i * n + x0 + lane) : 0.f;
+        }
+        __syncwarp();  // (the last columns have been read)
+#pragma unroll
+        for (int e = 0; e < 16; ++e) rs[e * 32 + lane] = rv[e];
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 32; q += 4)
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                const float4 r = *reinterpret_cast<const float4*>(rs + e * 32 + q);
+                s[e] = fmaf(av[q + 3], r.w, fmaf(av[q + 2], r.z, fmaf(av[q + 1], r.y, fmaf(av[q], r.x, s[e]))));
+            }
+    }
+#pragma unroll
+    for (int e = 0; e < 16; ++e)
+        if (mine && k0 + e < act_n && !((snan >> e) & 1u) && (a_inf || ((sinf >> e) & 1u)))
+            C[(size_t)(k0 + e) * m + atom] = s[e];
+}
+
 template <bool VEC, bool NARROW>
 __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
     pdl_enter();
@@ -456,22 +517,13 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
                     }
                 }
             }
-            if (flagged && atom < m) {
-                // scores with a value that has no split (and no NaN, whose products are NaN):
-                // one FP32 FMA chain over n
+            if (flagged) {
 #pragma unroll 1
-                for (int col = 0; col < w; ++col) {
-                    if (((col >> 4) & 1) != grp) continue;
-                    const int k = tn * w + col;
-                    if (k >= act_n || sh.nan[slot][ar] || sh.nan[slot][TF_BM + col]) continue;
-                    if (!sh.inf[slot][ar] && !sh.inf[slot][TF_BM + col]) continue;
-                    const float* a = d.A32 + (size_t)atom * n;
-                    const float* r = d.R32 + (size_t)d.act[cur][k] * n;
-                    float s = 0.f;
-#pragma unroll 1
-                    for (int x = 0; x < n; ++x) s = fmaf(__ldg(a + x), __ldg(r + x), s);
-                    d.Cs[(size_t)k * m + atom] = s;
-                }
+                for (int c0 = grp * 16; c0 < w; c0 += 32)
+                    if (tn * w + c0 < act_n)
+                        chain_block<VEC>(d.A32, d.R32, d.act[cur], d.Cs, n, m, atom, sh.inf[slot][ar] != 0,
+                                         sh.nan[slot][ar] != 0, sh.inf[slot] + TF_BM + c0, sh.nan[slot] + TF_BM + c0,
+                                         tn * w + c0, act_n, &sh.chain[warp - 12][0]);
             }
         }
     }
