@@ -39,7 +39,8 @@
 // one chain at a time 18, 2.3 and 197).
 //
 // Every wait is bounded; on expiry the CTA records DERR_TIMEOUT, the MMA thread waits (bounded) for
-// the MMAs it issued, and the CTA frees its TMEM and returns.
+// the MMAs it issued, the scores of the tiles the CTA did not finish are set to NaN, and the CTA
+// frees its TMEM and returns.
 #include "mpl_internal.cuh"
 #include "tc_ptx.cuh"
 
@@ -471,7 +472,8 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
         uint32_t ph = 0;
         unsigned tcount = 0;
         bool ok = true;
-        for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tcount) {
+        long long t = blockIdx.x;
+        for (; t < ntiles; t += gridDim.x, ++tcount) {
             const int tm = (int)(t / tiles_n), tn = (int)(t - (long long)tm * tiles_n);
             float acc[T::BN / 32][16];
 #pragma unroll
@@ -525,6 +527,15 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
                                          sh.nan[slot][ar] != 0, sh.inf[slot] + TF_BM + c0, sh.nan[slot] + TF_BM + c0,
                                          tn * w + c0, act_n, &sh.chain[warp - 12][0]);
             }
+        }
+        // a wait expired: this warp's scores of the tiles it did not finish are no numbers, so that a
+        // caller who cannot see the error code sees them
+        for (; t < ntiles; t += gridDim.x) {
+            const int tm = (int)(t / tiles_n), tn = (int)(t - (long long)tm * tiles_n);
+            const int atom = tm * TF_BM + q * 32 + lane;
+            for (int c0 = grp * 16; c0 < w; c0 += 32)
+                for (int k = tn * w + c0; k < min(act_n, tn * w + c0 + 16); ++k)
+                    if (atom < m) d.Cs[(size_t)k * m + atom] = __int_as_float(0x7fffffff);
         }
     }
     fence_before();

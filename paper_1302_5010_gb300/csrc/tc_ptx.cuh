@@ -8,7 +8,10 @@
 namespace mpl {
 namespace {
 
-constexpr uint64_t WAIT_LIMIT_NS = 4000000000ull;  // a wait gives up after 4 s
+#ifndef MPL_WAIT_LIMIT_NS
+#define MPL_WAIT_LIMIT_NS 4000000000ull
+#endif
+constexpr uint64_t WAIT_LIMIT_NS = MPL_WAIT_LIMIT_NS;  // a wait gives up after 4 s
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
