@@ -59,7 +59,6 @@ struct mpl_ctx {
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     cudaEvent_t ev_fork2 = nullptr, ev_join[2] = {};
     HostView* view = nullptr;                     // mapped pinned memory, written by the compaction
-    bool in_solve = false;                        // a solve began and did not end (it returned an error)
     cudaEvent_t ev_fin[FIN_SLOTS] = {};           // the exact finish of the last iteration of each slot
     int use_graph = 1;
     struct GraphEntry {
@@ -884,10 +883,12 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
     d.B = h->Bint;
     d.lam = h->lamint;
     d.view = h->view;
-    // no kernel of an earlier solve may write the view after this: one that ended has waited for
-    // them, one that returned an error has not
-    if (h->in_solve) CK(cudaDeviceSynchronize());
-    h->in_solve = true;
+    // whatever makes this solve return early, its kernels are done by then: they use the workspace
+    // of the handle's next call and write the view
+    struct Drain {
+        bool armed = true;
+        ~Drain() { if (armed) (void)cudaDeviceSynchronize(); }
+    } in_flight;
     std::memset(h->view, 0, sizeof(HostView));
     set_bounds(h, d);
     // a second, FP32 selection pass for bands that overflow the candidate buffer: only
@@ -1075,7 +1076,7 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
     CK(cudaEventRecord(h->ev_out, st));
     CK(cudaStreamWaitEvent(caller, h->ev_out, 0));
     CK(cudaStreamSynchronize(st));
-    h->in_solve = false;
+    in_flight.armed = false;
     if (h->cnt_h->err != 0) return h->cnt_h->err == DERR_TIMEOUT ? MPL_ERR_TIMEOUT : MPL_ERR_CUDA;
     pt.collect();
 #ifdef MPL_TIMELINE

@@ -1,0 +1,87 @@
+"""The library's host code on a machine without a GPU: its objects are linked with a stand-in for the
+CUDA runtime (fake_cudart.cpp) that keeps "device" memory on the host and records launches instead
+of running them, so that failures can be made to happen (an allocation that does not succeed, a
+device that stops answering) and the host's own decisions can be read off."""
+import ctypes
+import glob
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_1302_5010_gb300 import build as libbuild
+from paper_1302_5010_gb300 import mpl
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+REGS = 96  # registers a thread of the split TF32 kernel is compiled to
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    libbuild.build()
+    tmp = tmp_path_factory.mktemp("fake")
+    obj, out = str(tmp / "fake.o"), str(tmp / "libmpl_host.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(libbuild.nvcc()))), "include")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-w", "-I", libbuild.INCLUDE, "-I", cuda, "-c",
+                    os.path.join(HERE, "fake_cudart.cpp"), "-o", obj], check=True, capture_output=True)
+    objs = [os.path.join(libbuild.BUILD, os.path.basename(s)[:-3] + ".o") for s in libbuild._sources()]
+    subprocess.run(["g++", "-shared", "-o", out, obj, *objs, "-Wl,-Bsymbolic", "-Wl,-z,defs", "-lpthread"], check=True,
+                   capture_output=True)
+    h = ctypes.CDLL(out)
+    h.mpl_set_option.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_double]
+    for f in ("mpl_create", "bmpl_solve", "mpl_correlate", "mpl_correlate_noalloc", "mpl_proposal_set_weights",
+              "mpl_proposal_loss_grad", "mpl_autotune"):
+        getattr(h, f).restype = ctypes.c_int
+    h.fake_set.argtypes = [ctypes.c_int] * 5 + [ctypes.c_uint]
+    return h
+
+
+def fake(lib, regs=REGS, fail_malloc=0, iterations=1, delay_us=0, view_on=1, flags=0):
+    lib.fake_set(regs, fail_malloc, iterations, delay_us, view_on, flags)
+
+
+def _f32(a):
+    return a.ctypes.data_as(ctypes.c_void_p)
+
+
+class Handle:
+    def __init__(self, lib, n, m, **opts):
+        self.lib, self.n, self.m = lib, n, m
+        self.h = ctypes.c_void_p()
+        A = np.zeros((m, n), dtype=np.float32)
+        assert lib.mpl_create(_f32(A), n, m, ctypes.byref(self.h)) == mpl.MPL_OK
+        for k, v in opts.items():
+            assert lib.mpl_set_option(self.h, getattr(mpl, "MPL_OPT_" + k), float(v)) == mpl.MPL_OK
+
+    def solve(self, p):
+        B, lam = np.ones((p, self.n), dtype=np.float32), np.ones(p, dtype=np.float32)
+        X = np.zeros((p, self.m), dtype=np.float32)
+        return self.lib.bmpl_solve(self.h, _f32(B), p, _f32(lam), _f32(X), ctypes.c_double(1e-6), None)
+
+    def close(self):
+        self.lib.mpl_destroy(self.h)
+
+
+def test_the_stand_in_runs_a_solve(lib):
+    fake(lib, iterations=3)
+    s = Handle(lib, 128, 300, RHO=2)
+    assert s.solve(5) == mpl.MPL_OK
+    assert lib.fake_count(b"cudaGraphLaunch") == 3
+    s.close()
+    assert lib.fake_live() == 0
+
+
+@pytest.mark.parametrize("graph", [0, 1])
+def test_a_solve_that_fails_leaves_nothing_running(lib, graph):
+    """A solve that returns an error half way has waited for what it launched: its kernels use the
+    handle's workspace, which the next call on the handle (any of them) uses as well."""
+    s = Handle(lib, 128, 300, RHO=2, GRAPH=graph)
+    fake(lib, view_on=0)  # the stream runs dry without the selection's results
+    assert s.solve(5) == mpl.MPL_ERR_CUDA
+    last = max(lib.fake_last(b"k_"), lib.fake_last(b"cudaGraphLaunch"))
+    assert 0 <= last < lib.fake_last(b"cudaDeviceSynchronize")
+    fake(lib)
+    assert s.solve(5) == mpl.MPL_OK
+    assert lib.fake_count(b"cudaDeviceSynchronize") == 0  # (and a sound one waits for its own stream only)
+    s.close()
