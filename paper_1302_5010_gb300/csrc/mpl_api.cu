@@ -1150,19 +1150,23 @@ mpl_status_t mpl_correlate(mpl_handle_t h, const float* R, int p, float* C, void
 }
 
 // ---------------------------------------------------------------- proposal network
+// The buffers of the proposal network: all of them, or none.
 static cudaError_t prop_alloc(mpl_ctx* h) {
     if (h->pw) return cudaSuccess;
-    float** bufs[] = {&h->pw, &h->pwb, &h->pm1, &h->pm2, &h->pgrad};
-    for (float** q : bufs) {
-        cudaError_t e = cudaMalloc(q, PROP_NPARAM * sizeof(float));
-        if (e != cudaSuccess) return e;
-        cudaMemset(*q, 0, PROP_NPARAM * sizeof(float));
+    const struct { float** p; size_t floats; } bufs[] = {
+        {&h->pwb, PROP_NPARAM}, {&h->pm1, PROP_NPARAM}, {&h->pm2, PROP_NPARAM}, {&h->pgrad, PROP_NPARAM},
+        {&h->pacc, 4}, {&h->ppart, (size_t)TRAIN_MAX_ROWS * PROP_NPARAM}, {&h->rn, (size_t)h->m}, {&h->pw, PROP_NPARAM}};
+    cudaError_t e = cudaSuccess;
+    for (const auto& b : bufs) {
+        if (e == cudaSuccess) e = cudaMalloc(b.p, b.floats * sizeof(float));
+        if (e == cudaSuccess && b.floats == PROP_NPARAM) e = cudaMemset(*b.p, 0, PROP_NPARAM * sizeof(float));
     }
-    cudaError_t e = cudaMalloc(&h->pacc, 4 * sizeof(float));
-    if (e != cudaSuccess) return e;
-    e = cudaMalloc(&h->ppart, (size_t)TRAIN_MAX_ROWS * PROP_NPARAM * sizeof(float));
-    if (e != cudaSuccess) return e;
-    return cudaMalloc(&h->rn, (size_t)h->m * sizeof(float));
+    if (e != cudaSuccess)
+        for (const auto& b : bufs) {
+            cudaFree(*b.p);
+            *b.p = nullptr;
+        }
+    return e;
 }
 
 // ||A^T a_j|| by a 256-vector Rademacher sketch through the FP32 correlation kernel.

@@ -85,3 +85,25 @@ def test_a_solve_that_fails_leaves_nothing_running(lib, graph):
     assert s.solve(5) == mpl.MPL_OK
     assert lib.fake_count(b"cudaDeviceSynchronize") == 0  # (and a sound one waits for its own stream only)
     s.close()
+
+
+@pytest.mark.parametrize("k", range(1, 9))
+def test_proposal_buffers_all_or_none(lib, k):
+    """An allocation of the proposal network's buffers that fails leaves none of them behind: the next
+    call makes them all, and the training pass has the rows it writes its sums to."""
+    s = Handle(lib, 128, 300, RHO=2)
+    w = np.zeros(mpl.MPL_PROPOSAL_NPARAM, dtype=np.float32)
+    before = lib.fake_live()
+    fake(lib, fail_malloc=k)
+    assert lib.mpl_proposal_set_weights(s.h, _f32(w), w.size) == mpl.MPL_ERR_OOM
+    assert lib.fake_live() == before
+    assert lib.fake_count(b"k_sketch") == 0
+    fake(lib)
+    assert lib.mpl_proposal_set_weights(s.h, _f32(w), w.size) == mpl.MPL_OK
+    B, lam = np.ones((3, 128), dtype=np.float32), np.ones(3, dtype=np.float32)
+    X = np.zeros((3, 300), dtype=np.float32)
+    loss, g = ctypes.c_double(), np.zeros_like(w)
+    assert lib.mpl_proposal_loss_grad(s.h, _f32(B), 3, _f32(lam), _f32(X), ctypes.byref(loss), _f32(g)) == mpl.MPL_OK
+    assert lib.fake_count(b"k_train_fwd_bwd") == 1 and not lib.fake_train_part_null()
+    s.close()
+    assert lib.fake_live() == 0
