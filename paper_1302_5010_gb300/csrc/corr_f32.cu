@@ -138,7 +138,11 @@ __global__ void __launch_bounds__(256) k_corr_f32(Dev d, int cur, int jtile0) {
 cudaError_t launch_corr_f32(const Dev& d, int cur, int act_n_ub, cudaStream_t s, int64_t* nl) {
     if (act_n_ub <= 0) return cudaSuccess;
     if (gemv_route(d, act_n_ub)) return launch_corr_gemv(d, cur, act_n_ub, false, s, nl);
-    if (d.n >= TF32_MIN_N) return launch_corr_tf32(d, cur, act_n_ub, s, nl);
+    if (d.n >= TF32_MIN_N) {
+        // (not supported: compiled to fewer registers than it hands out; the chain is within its bound)
+        const cudaError_t e = launch_corr_tf32(d, cur, act_n_ub, s, nl);
+        if (e != cudaErrorNotSupported) return e;
+    }
     return launch_corr_chain(d, cur, act_n_ub, s, nl);
 }
 

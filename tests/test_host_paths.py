@@ -107,3 +107,21 @@ def test_proposal_buffers_all_or_none(lib, k):
     assert lib.fake_count(b"k_train_fwd_bwd") == 1 and not lib.fake_train_part_null()
     s.close()
     assert lib.fake_live() == 0
+
+
+@pytest.mark.parametrize("p", [9, 300])
+def test_correlation_without_the_registers_it_hands_out(lib, p):
+    """The split TF32 kernel hands its loaders' registers to the warps that accumulate; compiled to too few it
+    is not launched, and the FP32 chain, which computes the same product, takes the call."""
+    n, m = 256, 300
+    A, R, C = (np.zeros(s, dtype=np.float32) for s in ((m, n), (p, n), (p, m)))
+
+    def aligned(a):
+        b = np.zeros(a.size + 4, dtype=np.float32)
+        return b[(-b.ctypes.data // 4) % 4:][:a.size]
+
+    A, R, C = aligned(A), aligned(R), aligned(C)
+    for regs, kernel in ((REGS, b"k_corr_tf32"), (94, b"k_corr_f32")):
+        fake(lib, regs=regs)
+        assert lib.mpl_correlate_noalloc(_f32(A), n, m, _f32(R), p, _f32(C), None) == mpl.MPL_OK
+        assert lib.fake_count(b"k_corr_") == lib.fake_count(kernel) == 1
