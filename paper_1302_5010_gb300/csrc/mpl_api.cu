@@ -288,7 +288,7 @@ cudaError_t ensure_staging(float** buf, size_t* cap, size_t bytes) {
     return e;
 }
 
-// Rounding-error constants of the bounds used by the selection (unit roundoff u = 2^-24).
+// Rounding-error constants of the bounds used by the selection (unit roundoff u = 2^-24) for a batch of d.p.
 void set_bounds(mpl_ctx* h, Dev& d) {
     const double u = std::ldexp(1.0, -24);
     const double nu = (double)h->n * u;
@@ -298,8 +298,11 @@ void set_bounds(mpl_ctx* h, Dev& d) {
     // the split TF32 correlation (corr_tf32.cu): the operands' splits (2^-23 each) and the dropped
     // product of their low parts (2^-22), the tensor core's accumulation of 32 x 3 products
     // (assumed to lose at most 2^-22 of the running magnitude per product, as for BF16), and
-    // the FP32 sum of the n / 32 groups; the wider of the two FP32 forms covers both kernels
-    const double tf = 1.25 * (98.0 * std::ldexp(1.0, -22) + ((double)h->n / 32.0 + 2.0) * u);
+    // the FP32 sum of the n / 32 groups.  Where a batch can take it, the wider of the two FP32
+    // forms covers it and the chain or the matrix-vector products beside it; short signals and batches of a
+    // few keep the chain's (at n = 64 a quarter of the other)
+    const bool split = h->n >= TF32_MIN_N && !gemv_route(d, d.p);
+    const double tf = split ? 1.25 * (98.0 * std::ldexp(1.0, -22) + ((double)h->n / 32.0 + 2.0) * u) : 0.0;
     const double cf = std::max(c32, tf);
     d.bound_f32 = (float)(cf * 1.01);
     // identity route: FP32 beta and Q entries (gamma_n each, relative to colmax ||b|| and
@@ -308,7 +311,7 @@ void set_bounds(mpl_ctx* h, Dev& d) {
     const int smax = h->smax > 0 ? h->smax : default_smax(h);
     const double su = (double)(smax + 1) * u;
     const double gs = su / (1.0 - su);
-    const double gb = std::max(gam, tf);  // beta comes from either FP32 kernel
+    const double gb = std::max(gam, tf);  // beta comes from the same FP32 kernels
     d.bound_q = (float)((gb + 2.0 * gs * (1.0 + gb) + u) * 1.01);
     if (h->precision == 1) {
         // BF16 operands (relative 2^-8 each) with an FP32 accumulator assumed to

@@ -125,3 +125,29 @@ def test_correlation_without_the_registers_it_hands_out(lib, p):
         fake(lib, regs=regs)
         assert lib.mpl_correlate_noalloc(_f32(A), n, m, _f32(R), p, _f32(C), None) == mpl.MPL_OK
         assert lib.fake_count(b"k_corr_") == lib.fake_count(kernel) == 1
+
+
+@pytest.mark.parametrize("n,p,tf32", [(64, 5, False), (64, 20, False), (127, 20, False), (128, 20, True), (128, 5, True),
+                                      (200, 300, True), (256, 8, False), (256, 9, True), (1024, 5, False),
+                                      (1024, 20, True)])
+def test_band_of_the_kernels_that_run(lib, n, p, tf32):
+    """The selection's error bound is that of the correlation kernels the batch can take: gamma_n for the
+    chain (n < 128) and the matrix-vector products (at most 8 signals, n >= 256), the wider of
+    that and the split TF32 form for the others.  (u = 2^-24; 2 gamma_n + rounding of the residual.)"""
+    fake(lib)
+    s = Handle(lib, n, 300, RHO=2)
+    assert s.solve(p) == mpl.MPL_OK
+    got = (ctypes.c_float * 4)()
+    assert lib.fake_bounds(b"k_select", got) == 1
+    s.close()
+    u = 2.0 ** -24
+    gam = n * u / (1 - n * u)
+    chain = 2 * (gam + u)
+    split = 1.25 * (98 * 2.0 ** -22 + (n / 32 + 2) * u)
+    want = max(chain, split) if tf32 else chain
+    np.testing.assert_allclose(got[:2], [want * 1.01] * 2, rtol=1e-6)
+    assert got[3] == pytest.approx(chain * 1.01, rel=1e-6)
+    smax = min(n, 256)
+    gs = (smax + 1) * u / (1 - (smax + 1) * u)
+    gb = max(gam, split) if tf32 else gam
+    assert got[2] == pytest.approx((gb + 2 * gs * (1 + gb) + u) * 1.01, rel=1e-6)
