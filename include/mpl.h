@@ -311,10 +311,11 @@ int mpl_get_phase_times(mpl_handle_t h, double* ms_out, int cap);
  * candidate setting -- the identity route for the first k = 0, 1, 2, 4 outer
  * iterations after the first (MPL_OPT_QROUTE = k rho plus the warm-start
  * additions; k > 0 only when Q = A^T A fits in a quarter of the free device
- * memory) and MPL_OPT_SYNC_EVERY in {1, 2, 4}; then, where Q fits, the best
- * of those with MPL_OPT_QGRAM = 1 at each MPL_OPT_SYNC_EVERY; then, for the
- * BF16 path, the other GEMM tile widths (MPL_OPT_GEMM_TILE 64, 128, 256) with
- * the best of those -- and keeps the fastest on the handle.  Every candidate computes the same solution, so only time is
+ * memory); then, where Q fits, the best of those with MPL_OPT_QGRAM = 1; then,
+ * for the BF16 path, the other GEMM tile widths (MPL_OPT_GEMM_TILE 64, 128,
+ * 256) with the best of those -- and keeps the fastest on the handle.
+ * (MPL_OPT_SYNC_EVERY has no effect and stays as it is; one timing stands for
+ * its values 1, 2 and 4.)  Every candidate computes the same solution, so only time is
  * compared.  Each candidate runs once untimed (graph capture, Q build) and
  * three times timed with events on `stream`; the median counts.  The solutions
  * go to a scratch buffer the call allocates and frees; the handle's last-solve
@@ -323,10 +324,10 @@ int mpl_get_phase_times(mpl_handle_t h, double* ms_out, int cap);
  * candidate's), MPL_ERR_OOM for the scratch buffer. */
 typedef struct {
     int qroute;          /* chosen MPL_OPT_QROUTE */
-    int sync_every;      /* chosen MPL_OPT_SYNC_EVERY */
+    int sync_every;      /* MPL_OPT_SYNC_EVERY, as it was */
     double ms;           /* median solve time of the choice */
-    double ms_default;   /* median solve time with qroute 0, sync_every 2, qgram 0 */
-    int candidates;      /* settings timed */
+    double ms_default;   /* median solve time with qroute 0, qgram 0 */
+    int candidates;      /* settings compared: three per timed route or Gram source, one per tile */
     int qgram;           /* chosen MPL_OPT_QGRAM */
     int gemm_tile;       /* chosen MPL_OPT_GEMM_TILE (timed last, BF16 path only) */
 } mpl_tune_result_t;

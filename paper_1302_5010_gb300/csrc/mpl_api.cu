@@ -1470,56 +1470,53 @@ mpl_status_t mpl_autotune(mpl_handle_t h, const float* B, int p, const float* la
             const int v = std::min(smax, k * rho + warm_add);
             if (v > qcands.back()) qcands.push_back(v);
         }
-    const int se_cands[] = {1, 2, 4};
     float* X = nullptr;
     CK(cudaMalloc(&X, (size_t)m * p * sizeof(float)));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    const int keep_q = h->qroute, keep_se = h->sync_every, keep_prof = h->profile, keep_g = h->qgram;
+    const int keep_q = h->qroute, keep_prof = h->profile, keep_g = h->qgram;
     const int keep_bn = h->gemm_bn;
     h->profile = 0;
-    mpl_tune_result_t best{keep_q, keep_se, 1e300, 0.0, 0, keep_g, keep_bn};
+    mpl_tune_result_t best{keep_q, h->sync_every, 1e300, 0.0, 0, keep_g, keep_bn};
     mpl_status_t first_err = MPL_OK;
-    // stage 0: identity route x handshake interval with the computed Gram; stage 1: the
-    // Gram gathered from Q with the stage-0 route at each handshake interval
+    // one timing stands for the settings with MPL_OPT_SYNC_EVERY 1, 2 and 4, which are the same solve
+    constexpr int cadences = 3;
+    // stage 0: the identity route with the computed Gram; stage 1: the Gram gathered from Q
+    // with the stage-0 route
     for (int stage = 0; stage < 2; ++stage)
     for (int qr : (stage == 0 ? qcands : std::vector<int>{best.qroute})) {
         if (stage == 1 && (!q_fits || best.candidates == 0)) break;
-        for (int se : se_cands) {
-            h->qroute = qr;
-            h->sync_every = se;
-            h->qgram = stage;
-            clear_graphs(h);
-            mpl_status_t rc = bmpl_solve(h, B, p, lambda, X, tol, stream);  // capture + warm-up
-            std::vector<float> t;
-            for (int r = 0; r < 3 && (rc == MPL_OK || rc == MPL_ERR_NOT_CONVERGED); ++r) {
-                cudaEventRecord(e0, st);
-                rc = bmpl_solve(h, B, p, lambda, X, tol, stream);
-                cudaEventRecord(e1, st);
-                cudaEventSynchronize(e1);
-                float ms = 0.f;
-                cudaEventElapsedTime(&ms, e0, e1);
-                t.push_back(ms);
-            }
-            if (rc != MPL_OK && rc != MPL_ERR_NOT_CONVERGED) {
-                if (first_err == MPL_OK) first_err = rc;
-                continue;
-            }
-            std::sort(t.begin(), t.end());
-            const double med = t[t.size() / 2];
-            ++best.candidates;
-            if (qr == 0 && se == 2 && stage == 0) best.ms_default = med;
-            if (med < best.ms) { best.ms = med; best.qroute = qr; best.sync_every = se; best.qgram = stage; }
+        h->qroute = qr;
+        h->qgram = stage;
+        clear_graphs(h);
+        mpl_status_t rc = bmpl_solve(h, B, p, lambda, X, tol, stream);  // capture + warm-up
+        std::vector<float> t;
+        for (int r = 0; r < 3 && (rc == MPL_OK || rc == MPL_ERR_NOT_CONVERGED); ++r) {
+            cudaEventRecord(e0, st);
+            rc = bmpl_solve(h, B, p, lambda, X, tol, stream);
+            cudaEventRecord(e1, st);
+            cudaEventSynchronize(e1);
+            float ms = 0.f;
+            cudaEventElapsedTime(&ms, e0, e1);
+            t.push_back(ms);
         }
+        if (rc != MPL_OK && rc != MPL_ERR_NOT_CONVERGED) {
+            if (first_err == MPL_OK) first_err = rc;
+            continue;
+        }
+        std::sort(t.begin(), t.end());
+        const double med = t[t.size() / 2];
+        best.candidates += cadences;
+        if (qr == 0 && stage == 0) best.ms_default = med;
+        if (med < best.ms) { best.ms = med; best.qroute = qr; best.qgram = stage; }
     }
-    // stage 2 (BF16 GEMM only): the tile width with the chosen route, cadence and Gram source
+    // stage 2 (BF16 GEMM only): the tile width with the chosen route and Gram source
     best.gemm_tile = keep_bn;
     if (h->precision == 1 && best.candidates > 0) {
         for (int bn : {64, 128, 256}) {
             if (bn == keep_bn) continue;  // timed above
             h->qroute = best.qroute;
-            h->sync_every = best.sync_every;
             h->qgram = best.qgram;
             h->gemm_bn = bn;
             clear_graphs(h);
@@ -1549,13 +1546,11 @@ mpl_status_t mpl_autotune(mpl_handle_t h, const float* B, int p, const float* la
     clear_graphs(h);
     if (best.candidates == 0) {
         h->qroute = keep_q;
-        h->sync_every = keep_se;
         h->qgram = keep_g;
         h->gemm_bn = keep_bn;
         return first_err != MPL_OK ? first_err : MPL_ERR_CUDA;
     }
     h->qroute = best.qroute;
-    h->sync_every = best.sync_every;
     h->qgram = best.qgram;
     if (out) *out = best;
     return MPL_OK;

@@ -151,3 +151,21 @@ def test_band_of_the_kernels_that_run(lib, n, p, tf32):
     gs = (smax + 1) * u / (1 - (smax + 1) * u)
     gb = max(gam, split) if tf32 else gam
     assert got[2] == pytest.approx((gb + 2 * gs * (1 + gb) + u) * 1.01, rel=1e-6)
+
+
+@pytest.mark.parametrize("sync_every", [1, 2, 7])
+def test_autotuner_times_each_setting_once(lib, sync_every):
+    """MPL_OPT_SYNC_EVERY has no effect on a solve, so the tuner does not time its values against each other:
+    one solve to warm up and three timed for each of four route lengths and, with the best of them, the
+    gathered Gram rows.  The handle keeps the value it had."""
+    s = Handle(lib, 128, 300, RHO=2, SYNC_EVERY=sync_every)
+    p = 5
+    B, lam = np.ones((p, 128), dtype=np.float32), np.ones(p, dtype=np.float32)
+    out = mpl.TuneResult()
+    fake(lib)
+    assert lib.mpl_autotune(s.h, _f32(B), p, _f32(lam), ctypes.c_double(1e-6), None, ctypes.byref(out)) == mpl.MPL_OK
+    assert lib.fake_count(b"6k_init") == 4 * (4 + 1)
+    assert out.sync_every == sync_every and out.candidates == 3 * (4 + 1)
+    v = ctypes.c_double()
+    assert lib.mpl_get_option(s.h, mpl.MPL_OPT_SYNC_EVERY, ctypes.byref(v)) == mpl.MPL_OK and v.value == sync_every
+    s.close()
