@@ -181,6 +181,11 @@ mpl_status_t mpl_create(const float* A, int n, int m, mpl_handle_t* out);
  * Device buffers are read and written in stream order; the call returns after
  * the solve has completed on the stream (the outer loop is host-driven), so X
  * and the statistics are ready on return.
+ * While it runs, the host looks at mapped memory for each iteration's work
+ * lists: a core is polled at full rate for the whole solve, unless the device's
+ * scheduling flag (cudaSetDeviceFlags) is cudaDeviceScheduleYield or
+ * cudaDeviceScheduleBlockingSync; then the wait yields, or sleeps 20
+ * microseconds at a time.
  * Returns MPL_OK when every signal is certified, MPL_ERR_NOT_CONVERGED when
  * some signal is not (its best iterate is still written to X), or an error.
  */

@@ -14,9 +14,11 @@
 
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <cmath>
 #include <numeric>
 #include <random>
+#include <thread>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -814,11 +816,21 @@ static mpl_status_t ensure_streams(mpl_ctx* h) {
 
 // Until the compaction of the solve's `want`-th selection has written the view.  The stream is
 // asked now and then whether it failed, or ran dry without writing it (every kernel of the
-// chain is bounded, so one or the other happens).
-static mpl_status_t wait_view(mpl_ctx* h, cudaStream_t st, unsigned want) {
+// chain is bounded, so one or the other happens).  sched: the device's scheduling flag, kept as a
+// stream's synchronisation would keep it: yield the core between looks, or (blocking) sleep, after
+// a first look of some microseconds; by default, and where spinning is asked for, the host polls.
+static mpl_status_t wait_view(mpl_ctx* h, cudaStream_t st, unsigned want, unsigned sched) {
     const volatile unsigned* seq = &h->view->seq;
+    unsigned ask = 0xffffu;  // looks between two questions to the stream, less one
     for (unsigned spin = 1; *seq != want; ++spin) {
-        if ((spin & 0xffffu) != 0u) continue;
+        if (sched == cudaDeviceScheduleYield) {
+            ask = 0xffu;
+            std::this_thread::yield();
+        } else if (sched == cudaDeviceScheduleBlockingSync && spin >= 4096u) {
+            ask = 0x3fu;
+            std::this_thread::sleep_for(std::chrono::microseconds(20));
+        }
+        if ((spin & ask) != 0u) continue;
         const cudaError_t q = cudaStreamQuery(st);
         if (q == cudaErrorNotReady) {
             (void)cudaGetLastError();  // (not an error: still running)
@@ -943,6 +955,9 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
     mark(-1, st);
 #endif
     const bool early = h->stop_rinf >= 0.0 || h->stop_r2 >= 0.0 || h->stop_eps >= 0.0;
+    unsigned sched = 0;
+    CK(cudaGetDeviceFlags(&sched));
+    sched &= cudaDeviceScheduleMask;
     bool drain = false;  // only finishes are left: the next iteration waits for all of them
     for (; live > 0 && t < hard_cap; ++t) {
         const int fs = t % FIN_SLOTS;
@@ -1005,7 +1020,7 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
 #endif
         // the lists of this iteration, known as soon as its selection is done: the host launches
         // the finish and queues the next iteration while the rest of this one runs
-        const mpl_status_t vs = wait_view(h, st, (unsigned)t + 1u);
+        const mpl_status_t vs = wait_view(h, st, (unsigned)t + 1u, sched);
         if (vs != MPL_OK) return vs;
         const HostView v = *h->view;
 #ifdef MPL_BOUNDS

@@ -31,7 +31,7 @@ std::vector<std::string> log_;             // the same in order
 std::map<std::string, mpl::Dev> devs;      // the Dev argument of each kernel's last launch
 std::map<void*, size_t> live;              // device allocations
 std::atomic<int> pending{0};
-Graph* capture = nullptr;
+thread_local Graph* capture = nullptr;
 int regs = 96, fail_malloc = 0, iterations = 1, delay_us = 0, view_on = 1;
 unsigned flags = 0;
 const void* train_part = nullptr;
@@ -63,14 +63,17 @@ void drain() {
 }
 
 cudaError_t launch(const void* f, void** args) {
-    const std::string& n = names[f];
+    const std::string& n = names.at(f);
     note(n.c_str());
     const bool fused = n.find("k_select") != std::string::npos && *static_cast<int*>(args[5]) != 0;
     const bool takes_dev = n.find("k_select") != std::string::npos || n.find("k_compact") != std::string::npos ||
                            n.find("k_corr_") != std::string::npos;
     if (takes_dev) {
         const mpl::Dev& d = *static_cast<const mpl::Dev*>(args[0]);
-        devs[n] = d;
+        {
+            std::lock_guard<std::mutex> l(mu);
+            devs[n] = d;
+        }
         if (fused || n.find("k_compact") != std::string::npos) {
             if (capture) {
                 capture->iteration = true;
@@ -211,10 +214,16 @@ cudaError_t CUDARTAPI cudaMalloc(void** p, size_t n) {
     *p = nullptr;
     if (fail_malloc && --fail_malloc == 0) return cudaErrorMemoryAllocation;
     *p = std::calloc(1, n ? n : 1);
+    std::lock_guard<std::mutex> l(mu);
     live[*p] = n;
     return cudaSuccess;
 }
-cudaError_t CUDARTAPI cudaFree(void* p) { live.erase(p); std::free(p); return cudaSuccess; }
+cudaError_t CUDARTAPI cudaFree(void* p) {
+    std::lock_guard<std::mutex> l(mu);
+    live.erase(p);
+    std::free(p);
+    return cudaSuccess;
+}
 cudaError_t CUDARTAPI cudaMallocHost(void** p, size_t n) { *p = std::calloc(1, n); return cudaSuccess; }
 cudaError_t CUDARTAPI cudaHostAlloc(void** p, size_t n, unsigned) { *p = std::calloc(1, n); return cudaSuccess; }
 cudaError_t CUDARTAPI cudaFreeHost(void* p) { std::free(p); return cudaSuccess; }

@@ -169,3 +169,46 @@ def test_autotuner_times_each_setting_once(lib, sync_every):
     v = ctypes.c_double()
     assert lib.mpl_get_option(s.h, mpl.MPL_OPT_SYNC_EVERY, ctypes.byref(v)) == mpl.MPL_OK and v.value == sync_every
     s.close()
+
+
+@pytest.mark.parametrize("flag", [0, 1, 4])
+def test_the_wait_for_the_work_lists_keeps_the_schedule_flag(lib, flag):
+    """A process that asked for blocking synchronisation (cudaDeviceScheduleBlockingSync = 4) does not
+    find a core polled at full rate while a solve runs: 10 iterations of 20 ms cost it a small part of
+    200 ms.  Spinning (1) and no choice (0) only have to finish."""
+    import time
+    s = Handle(lib, 128, 300, RHO=2)
+    fake(lib, iterations=1, flags=flag)
+    assert s.solve(5) == mpl.MPL_OK
+    fake(lib, iterations=10, delay_us=20000, flags=flag)
+    w, c = time.perf_counter(), time.process_time()
+    assert s.solve(5) == mpl.MPL_OK
+    w, c = time.perf_counter() - w, time.process_time() - c
+    s.close()
+    assert w >= 0.2
+    assert flag != 4 or c <= 0.5 * w, (w, c)
+
+
+def test_the_wait_yields_where_asked(lib):
+    """cudaDeviceScheduleYield (2): two solves in two threads still finish, and so does one whose device
+    stops answering."""
+    import threading
+    fake(lib, iterations=20, delay_us=200, flags=2)
+    rc = []
+
+    def one():
+        s = Handle(lib, 128, 300, RHO=2)
+        rc.append(s.solve(5))
+        s.close()
+
+    ts = [threading.Thread(target=one) for _ in range(2)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert rc == [mpl.MPL_OK] * 2
+    for flag in (2, 4):
+        fake(lib, view_on=0, flags=flag)
+        s = Handle(lib, 128, 300, RHO=2)
+        assert s.solve(5) == mpl.MPL_ERR_CUDA
+        s.close()
