@@ -65,7 +65,10 @@ typedef enum {
                                work-list lengths to mapped host memory, and the host reads them
                                while the iteration still runs.  default 2 */
     MPL_OPT_PROFILE = 8,    /* 1: record per-phase device times (mpl_get_phase_times) with
-                               timing events, inside the captured graphs too. default 0 */
+                               timing events, inside the captured graphs too; the host waits for
+                               the stream where a graph is replayed again within a solve (once in
+                               four iterations, past the one whose active-set bound is SMAX), to
+                               read its events first. default 0 */
     MPL_OPT_GRAPH = 9,      /* 1: each outer iteration is replayed from a captured CUDA graph
                                (captured on first use per batch size and iteration), until at
                                most a quarter of the signals is active. default 1 */

@@ -941,6 +941,16 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
     int pend_n[FIN_SLOTS] = {};  // and how many signals it took
     int pend_t[FIN_SLOTS] = {};  // and the iteration it was launched in
     double graph_phase[16] = {0};
+    std::vector<size_t> timed;  // replayed graphs whose timing events have not been read
+    auto read_timed = [&]() {
+        for (size_t gi : timed)
+            for (auto& mk : h->graphs[gi].marks) {
+                float ms = 0.f;
+                cudaEventElapsedTime(&ms, mk.second.first, mk.second.second);
+                graph_phase[mk.first] += ms;
+            }
+        timed.clear();
+    };
     int t = 0;
 #ifdef MPL_TIMELINE
     // diagnostic build: device timestamps of every iteration and finish
@@ -996,16 +1006,17 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
         if (graph && 4 * (long long)act > p) {
             size_t gi = 0;
             CK(iteration_graph(h, d, t, p, tol, st, &gi));
+            if (h->profile) {
+                // a replay overwrites the graph's events: they are read before it
+                const auto again = std::find(timed.begin(), timed.end(), gi);
+                if (again != timed.end()) {
+                    CK(cudaStreamSynchronize(st));
+                    read_timed();
+                }
+                timed.push_back(gi);
+            }
             CK(cudaGraphLaunch(h->graphs[gi].exec, st));
             nl += h->graphs[gi].kernels;
-            if (h->profile) {  // (the next launch of this graph would overwrite its events)
-                CK(cudaStreamSynchronize(st));
-                for (auto& mk : h->graphs[gi].marks) {
-                    float ms = 0.f;
-                    cudaEventElapsedTime(&ms, mk.second.first, mk.second.second);
-                    graph_phase[mk.first] += ms;
-                }
-            }
         } else {
             // Few signals left: grids and kernels for them, launched one by one, instead of the graph's
             // for all p.  A quarter is where the kernels for fewer signals begin to differ (an FP32
@@ -1097,6 +1108,7 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
     in_flight.armed = false;
     if (h->cnt_h->err != 0) return h->cnt_h->err == DERR_TIMEOUT ? MPL_ERR_TIMEOUT : MPL_ERR_CUDA;
     pt.collect();
+    read_timed();
 #ifdef MPL_TIMELINE
     for (auto& mk : marks) {
         float ms = 0.f;

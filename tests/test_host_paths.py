@@ -212,3 +212,22 @@ def test_the_wait_yields_where_asked(lib):
         s = Handle(lib, 128, 300, RHO=2)
         assert s.solve(5) == mpl.MPL_ERR_CUDA
         s.close()
+
+
+@pytest.mark.parametrize("smax,waits", [(128, (1, 1, 1)), (4, (1, 2, 3))])
+def test_profiling_leaves_the_iterations_overlapped(lib, smax, waits):
+    """With MPL_OPT_PROFILE a replayed iteration's timing events are read when its graph is replayed again
+    (iterations beyond the one where the active-set bound saturates share a graph per list slot:
+    with smax 4 and rho 2 those of t = 8..11 repeat 4..7), or at the end: the host does not wait for an
+    iteration before it queues the next.  Every iteration's phases are counted once."""
+    s = Handle(lib, 128, 300, RHO=2, SMAX=smax, PROFILE=1)
+    elapsed, waited = [], []
+    for it in (6, 11, 16):
+        fake(lib, iterations=it)
+        assert s.solve(5) == mpl.MPL_OK
+        assert lib.fake_count(b"cudaGraphLaunch") == it
+        elapsed.append(lib.fake_count(b"cudaEventElapsedTime"))
+        waited.append(lib.fake_count(b"cudaStreamSynchronize"))
+    s.close()
+    assert elapsed[1] - elapsed[0] == elapsed[2] - elapsed[1] > 0
+    assert tuple(waited) == waits
