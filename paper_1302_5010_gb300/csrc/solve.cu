@@ -275,6 +275,10 @@ __global__ void __launch_bounds__((BM / TR) * (BN / TC)) k_gram(Dev d) {
     const int s = d.ssize[i], q = d.snew[i], s0 = s - q;
     const int a0 = blockIdx.y * BM;
     if (a0 >= s || q == 0) return;  // q == 0: a refine pass, the block is complete
+    if (s > (int)gridDim.y * BM) {  // (above the host's bound, which sized the grid)
+        if (threadIdx.x == 0) atomicCAS(&d.cnt->err, 0, (int)DERR_SHAPE);
+        return;
+    }
     const int n = d.n, smax = d.smax;
     if (blockIdx.y == 0 && threadIdx.x == 0)  // s atom columns read, 2 s q of G written
         atomicAdd(&d.cnt->gram_bytes, 4ull * n * s + 8ull * s * q);
@@ -991,10 +995,11 @@ __device__ void apg_reg_signal(const Dev& d, int i, int tid, ApgRegShared& sh) {
     }
 }
 
-// Persistent CTAs (or warps) over the master-problem list; signals with more than NC's rows (or
-// more than the class takes) are left to the other launches of the iteration.
+// Persistent CTAs (or warps) over the master-problem list; signals with more than NC's rows are left
+// to the other launches of the iteration.  There are none up to a bound vcap of APG_REG_S: a
+// set above the bound is an error, as in k_apg.
 template <int NC, bool WARP, int MINB>
-__global__ void __launch_bounds__(WARP ? 32 * APG_WARPS : 4 * NC, MINB) k_apg_reg(Dev d) {
+__global__ void __launch_bounds__(WARP ? 32 * APG_WARPS : 4 * NC, MINB) k_apg_reg(Dev d, int vcap) {
     pdl_enter();
     __shared__ __align__(16) ApgRegShared sha[WARP ? APG_WARPS : 1];
     ApgRegShared& sh = sha[WARP ? threadIdx.x >> 5 : 0];
@@ -1006,7 +1011,9 @@ __global__ void __launch_bounds__(WARP ? 32 * APG_WARPS : 4 * NC, MINB) k_apg_re
         const int it = sh.item;
         if (it >= d.cnt->apg_n) break;
         const int i = d.list_apg[it];
-        if (d.ssize[i] <= ApgReg<NC, WARP>::ROWS) apg_reg_signal<NC, WARP>(d, i, tid, sh);
+        const int s = d.ssize[i];
+        if (s <= ApgReg<NC, WARP>::ROWS) apg_reg_signal<NC, WARP>(d, i, tid, sh);
+        else if (s > vcap && tid == 0) atomicCAS(&d.cnt->err, 0, (int)DERR_SHAPE);
         // every thread has read sh.item (and finished with sh) before the next one is taken
         if (WARP) __syncwarp();
         else __syncthreads();
@@ -1455,14 +1462,14 @@ int apg_classes(const Dev& d, int vcap) {
 // The register variants by the bound on |S|: rows of a warp, then 64, 96 and 128 rows (the more
 // rows, the more registers a thread and the fewer CTAs an SM holds).
 template <int NC, bool WARP, int MINB>
-static cudaError_t launch_apg_reg_t(const Dev& d, int ub, int sms, cudaStream_t s) {
+static cudaError_t launch_apg_reg_t(const Dev& d, int ub, int sms, int vcap, cudaStream_t s) {
     constexpr int nt = WARP ? 32 * APG_WARPS : 4 * NC;
     int per_sm = 0;
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_apg_reg<NC, WARP, MINB>, nt, 0);
     if (e != cudaSuccess) return e;
     const int need = WARP ? (ub + APG_WARPS - 1) / APG_WARPS : ub;
     const int grid = std::min(sms * std::max(per_sm, 1), need);
-    return launch_chain(k_apg_reg<NC, WARP, MINB>, dim3(grid), dim3(nt), 0, s, d);
+    return launch_chain(k_apg_reg<NC, WARP, MINB>, dim3(grid), dim3(nt), 0, s, d, vcap);
 }
 
 cudaError_t launch_apg(const Dev& d, int ub, int sms, int vcap, cudaStream_t s, int64_t* nl, int cls) {
@@ -1470,10 +1477,10 @@ cudaError_t launch_apg(const Dev& d, int ub, int sms, int vcap, cudaStream_t s, 
     vcap = apg_vcap(d, vcap);
     cudaError_t e;
     if (cls == APG_REG) {
-        e = vcap <= 32   ? launch_apg_reg_t<32, true, 4>(d, ub, sms, s)
-            : vcap <= 64 ? launch_apg_reg_t<32, false, 5>(d, ub, sms, s)
-            : vcap <= 96 ? launch_apg_reg_t<48, false, 3>(d, ub, sms, s)
-                         : launch_apg_reg_t<64, false, 2>(d, ub, sms, s);
+        e = vcap <= 32   ? launch_apg_reg_t<32, true, 4>(d, ub, sms, vcap, s)
+            : vcap <= 64 ? launch_apg_reg_t<32, false, 5>(d, ub, sms, vcap, s)
+            : vcap <= 96 ? launch_apg_reg_t<48, false, 3>(d, ub, sms, vcap, s)
+                         : launch_apg_reg_t<64, false, 2>(d, ub, sms, vcap, s);
     } else {
         if ((e = prepare_apg()) != cudaSuccess) return e;
         // APG_SMEM: the blocks past the registers that fit shared memory; APG_GLOBAL: the others,
