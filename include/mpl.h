@@ -239,10 +239,9 @@ mpl_status_t mpl_correlate(mpl_handle_t h, const float* R, int p, float* C, void
  * before any stream capture.  Every call rewrites the scratch it reads, and
  * all calls share it, so calls whose GPU work overlaps (different streams, no
  * ordering between them) race.
- * A failure on the device: for n >= 128, but for p <= 8 with n >= 256, the call
- * runs the tensor-core kernel, whose waits give up after 4 s (nothing but a
- * fault of the device or a debugger that stops it is known to make one last so
- * long).  The call has returned MPL_OK by then; the scores of the tiles that
+ * A failure on the device: for n >= 256 and p > 8 the call runs the tensor-core
+ * kernel, whose waits give up after 4 s (nothing but a fault of the device or a
+ * debugger that stops it is known to make one last so long).  The call has returned MPL_OK by then; the scores of the tiles that
  * were not finished are set to NaN.  Scores of finite vectors and atoms are
  * otherwise NaN only where their FP32 sum overflows in both directions.
  */

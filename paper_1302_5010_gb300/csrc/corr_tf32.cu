@@ -29,8 +29,10 @@
 // (140 TFLOP/s), 4096 x 65536 x 1024: 3.13 ms, 1024 x 8192 x 256: 46 us (three stages); the FP32 chain on the SIMT
 // cores takes 1596 us, 12.2 ms and 162 us.  Loads staged in registers (592 us), six loader warps
 // (507 us) and more, shorter stages with the copies issued ahead (557 to 650 us) were slower.
-// Error against FP64 (2-norm, Gaussian data): 1.3e-7 at n = 128, 2.4e-7 at n = 4096, the chain's
-// 2.0e-7 and 1.15e-6.
+// Error against FP64 (2-norm), relative to the FP32 chain's: Gaussian data 0.65 at n = 128, 0.48 at 256, 0.21
+// at 4096; data of one sign, where the tensor core's truncation does not cancel, 0.85, 0.56, 0.22; the same
+// over 24 binary orders, or one large product in eight, 1.18 at n = 128 and 0.75 at 256, 0.07 at 4096.  So
+// signals of fewer than TF32_MIN_N = 256 entries keep the chain.
 //
 // Inputs at or near overflow (infinities, NaN, |x| >= 2^128 (1 - 2^-12)) have no split: their rows
 // are flagged and the affected scores recomputed with one FP32 FMA chain over n, so that a

@@ -301,8 +301,8 @@ void set_bounds(mpl_ctx* h, Dev& d) {
     // product of their low parts (2^-22), the tensor core's accumulation of 32 x 3 products
     // (assumed to lose at most 2^-22 of the running magnitude per product, as for BF16), and
     // the FP32 sum of the n / 32 groups.  Where a batch can take it, the wider of the two FP32
-    // forms covers it and the chain or the matrix-vector products beside it; short signals and batches of a
-    // few keep the chain's (at n = 64 a quarter of the other)
+    // forms covers it and the chain or the matrix-vector products beside it (that is the chain's for scores,
+    // and up to n = 500 this one for beta); short signals and batches of a few keep the chain's
     const bool split = h->n >= TF32_MIN_N && !gemv_route(d, d.p);
     const double tf = split ? 1.25 * (98.0 * std::ldexp(1.0, -22) + ((double)h->n / 32.0 + 2.0) * u) : 0.0;
     const double cf = std::max(c32, tf);

@@ -203,7 +203,9 @@ struct PropArgs {
 // Each returns the CUDA error of its launch and adds its launches to *nl.
 // FP32 correlation: the matrix-vector route, the split TF32 tensor-core kernel, or the chain.
 cudaError_t launch_corr_f32(const Dev& d, int cur, int act_n_ub, cudaStream_t s, int64_t* nl);
-constexpr int TF32_MIN_N = 128;
+// From this length on: below it, with the chain's error small, the tensor core's truncation shows on data
+// of one sign (see corr_tf32.cu).
+constexpr int TF32_MIN_N = 256;
 cudaError_t launch_corr_tf32(const Dev& d, int cur, int act_n_ub, cudaStream_t s, int64_t* nl);
 // FP32 on the SIMT cores, one FMA chain over n per score (the order of the computed Gram block).
 cudaError_t launch_corr_chain(const Dev& d, int cur, int act_n_ub, cudaStream_t s, int64_t* nl);

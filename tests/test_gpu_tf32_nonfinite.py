@@ -48,7 +48,7 @@ def test_time_with_infinities(n, m, p, few, all_):
     assert every <= all_ * clean, (clean, every)
 
 
-@pytest.mark.parametrize("n,m,p", [(128, 130, 17), (129, 260, 33), (256, 1000, 300), (1021, 700, 129)])
+@pytest.mark.parametrize("n,m,p", [(128, 130, 17), (255, 260, 33), (256, 130, 17), (257, 1000, 300), (1021, 700, 129)])
 def test_chains_are_those_of_the_fp32_chain(n, m, p):
     """Scores that involve a value without a split, bit for bit as one FP32 FMA chain (FP64 products and
     sums rounded to FP32 at each step: the product of two FP32 values is exact in FP64, and 29 spare

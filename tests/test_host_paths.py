@@ -127,12 +127,12 @@ def test_correlation_without_the_registers_it_hands_out(lib, p):
         assert lib.fake_count(b"k_corr_") == lib.fake_count(kernel) == 1
 
 
-@pytest.mark.parametrize("n,p,tf32", [(64, 5, False), (64, 20, False), (127, 20, False), (128, 20, True), (128, 5, True),
-                                      (200, 300, True), (256, 8, False), (256, 9, True), (1024, 5, False),
-                                      (1024, 20, True)])
+@pytest.mark.parametrize("n,p,tf32", [(64, 5, False), (64, 20, False), (128, 5, False), (200, 300, False),
+                                      (255, 20, False), (256, 20, True), (256, 8, False), (256, 9, True),
+                                      (400, 300, True), (1024, 5, False), (1024, 20, True)])
 def test_band_of_the_kernels_that_run(lib, n, p, tf32):
     """The selection's error bound is that of the correlation kernels the batch can take: gamma_n for the
-    chain (n < 128) and the matrix-vector products (at most 8 signals, n >= 256), the wider of
+    chain (n < 256) and the matrix-vector products (at most 8 signals, n >= 256), the wider of
     that and the split TF32 form for the others.  (u = 2^-24; 2 gamma_n + rounding of the residual.)"""
     fake(lib)
     s = Handle(lib, n, 300, RHO=2)
