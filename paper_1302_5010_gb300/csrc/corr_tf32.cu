@@ -36,8 +36,8 @@
 //
 // Inputs at or near overflow (infinities, NaN, |x| >= 2^128 (1 - 2^-12)) have no split: their rows
 // are flagged and the affected scores recomputed with one FP32 FMA chain over n, so that a
-// score is infinite or NaN where the FP32 product is.  2044 x 32771 x 500: 1.64 ms with one infinite
-// atom, 1.40 with one infinite signal, 6.6 with all of them (0.48 without; the SIMT kernel always 1.60;
+// score is infinite or NaN where the FP32 product is.  2044 x 32771 x 500: 1.52 ms with one infinite
+// atom, 1.29 with one infinite signal, 6.3 with all of them (0.48 without; the SIMT kernel always 1.60;
 // one chain at a time 18, 2.3 and 197).
 //
 // Every wait is bounded; on expiry the CTA records DERR_TIMEOUT, the MMA thread waits (bounded) for
@@ -341,6 +341,31 @@ __device__ __noinline__ void chain_block(const float* __restrict__ A, const floa
             C[(size_t)(k0 + e) * m + atom] = s[e];
 }
 
+// The chains of a tile that an accumulating warp has stored, for its 32 atoms and its blocks of signals.
+template <bool VEC>
+__device__ __forceinline__ void chain_tile(const Dev& d, TfShared& sh, int cur, int slot, int tm, int tn, int w,
+                                        int act_n) {
+    const int warp = (threadIdx.x >> 5) - 12, ar = (warp & 3) * 32 + (threadIdx.x & 31);
+#pragma unroll 1
+    for (int c0 = (warp >> 2) * 16; c0 < w && tn * w + c0 < act_n; c0 += 32)
+        chain_block<VEC>(d.A32, d.R32, d.act[cur], d.Cs, d.n, d.m, tm * TF_BM + ar, sh.inf[slot][ar] != 0,
+                         sh.nan[slot][ar] != 0, sh.inf[slot] + TF_BM + c0, sh.nan[slot] + TF_BM + c0, tn * w + c0,
+                         act_n, sh.chain[warp]);
+}
+
+// The scores of an accumulating warp in the tiles from t on, which its block gave up on, are no numbers: a
+// caller who cannot see the error code sees them.
+__device__ __forceinline__ void unfinished(const Dev& d, long long t, long long ntiles, int tiles_n, int w, int act_n) {
+    const int warp = (threadIdx.x >> 5) - 12;
+    for (; t < ntiles; t += gridDim.x) {
+        const int tm = (int)(t / tiles_n), tn = (int)(t - (long long)tm * tiles_n);
+        const int atom = tm * TF_BM + (warp & 3) * 32 + (threadIdx.x & 31);
+        for (int c0 = (warp >> 2) * 16; c0 < w; c0 += 32)
+            for (int k = tn * w + c0; k < min(act_n, tn * w + c0 + 16); ++k)
+                if (atom < d.m) d.Cs[(size_t)k * d.m + atom] = __int_as_float(0x7fffffff);
+    }
+}
+
 template <bool VEC, bool NARROW>
 __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
     pdl_enter();
@@ -475,69 +500,66 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_corr_tf32(Dev d, int cur) {
         unsigned tcount = 0;
         bool ok = true;
         long long t = blockIdx.x;
-        for (; t < ntiles; t += gridDim.x, ++tcount) {
-            const int tm = (int)(t / tiles_n), tn = (int)(t - (long long)tm * tiles_n);
-            float acc[T::BN / 32][16];
+        // a tile with scores to recompute ends the inner loop: their code between its instructions, or a
+        // call among them, costs the accumulation 1 to 3 % (777 x 6001 x 99, 2048 x 32768 x 128)
+        for (;;) {
+            int flag_slot = -1;
+            for (; t < ntiles && flag_slot < 0; t += gridDim.x, ++tcount) {
+                const int tm = (int)(t / tiles_n), tn = (int)(t - (long long)tm * tiles_n);
+                float acc[T::BN / 32][16];
 #pragma unroll
-            for (int i = 0; i < T::BN / 32; ++i)
+                for (int i = 0; i < T::BN / 32; ++i)
 #pragma unroll
-                for (int e = 0; e < 16; ++e) acc[i][e] = 0.f;
-            for (int kb = 0; kb < nk; ++kb) {
-                ok = true;
-                if (lane == 0) ok = mbar_wait(&sh.done[stage], ph, abort_flag);
-                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-                if (!ok) { if (lane == 0) give_up(); break; }
-                fence_after();
-                const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(stage * T::BN);
+                    for (int e = 0; e < 16; ++e) acc[i][e] = 0.f;
+                for (int kb = 0; kb < nk; ++kb) {
+                    ok = true;
+                    if (lane == 0) ok = mbar_wait(&sh.done[stage], ph, abort_flag);
+                    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                    if (!ok) { if (lane == 0) give_up(); break; }
+                    fence_after();
+                    const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(stage * T::BN);
+#pragma unroll
+                    for (int i = 0; i < T::BN / 32; ++i) {
+                        if (2 * i + grp < nblk) {
+                            float v[16];
+                            tmem_ld16(tb + (uint32_t)((2 * i + grp) * 16), v);
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) acc[i][e] += v[e];
+                        }
+                    }
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&sh.tempty[stage]);
+                    if (++stage == nst) { stage = 0; ph ^= 1u; }
+                }
+                if (!ok) break;
+                const int slot = tcount & (TF_SLOTS - 1);
+                const int ar = q * 32 + lane;
+                const int atom = tm * TF_BM + ar;
+                bool flagged = false;
+#pragma unroll
+                for (int l = 0; l < TF_LOADERS; ++l) flagged |= sh.any[slot][l] != 0;
 #pragma unroll
                 for (int i = 0; i < T::BN / 32; ++i) {
                     if (2 * i + grp < nblk) {
-                        float v[16];
-                        tmem_ld16(tb + (uint32_t)((2 * i + grp) * 16), v);
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) acc[i][e] += v[e];
+                        for (int e = 0; e < 16; ++e) {
+                            const int col = (2 * i + grp) * 16 + e;
+                            const int k = tn * w + col;
+                            if (k < act_n && atom < m) d.Cs[(size_t)k * m + atom] = acc[i][e];
+                        }
                     }
                 }
-                fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sh.tempty[stage]);
-                if (++stage == nst) { stage = 0; ph ^= 1u; }
+                if (flagged) flag_slot = slot;
             }
-            if (!ok) break;
-            const int slot = tcount & (TF_SLOTS - 1);
-            const int ar = q * 32 + lane;
-            const int atom = tm * TF_BM + ar;
-            bool flagged = false;
-#pragma unroll
-            for (int l = 0; l < TF_LOADERS; ++l) flagged |= sh.any[slot][l] != 0;
-#pragma unroll
-            for (int i = 0; i < T::BN / 32; ++i) {
-                if (2 * i + grp < nblk) {
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const int col = (2 * i + grp) * 16 + e;
-                        const int k = tn * w + col;
-                        if (k < act_n && atom < m) d.Cs[(size_t)k * m + atom] = acc[i][e];
-                    }
-                }
+            if (flag_slot >= 0) {
+                const long long tp = t - gridDim.x;
+                const int tm = (int)(tp / tiles_n);
+                chain_tile<VEC>(d, sh, cur, flag_slot, tm, (int)(tp - (long long)tm * tiles_n), w, act_n);
+                continue;
             }
-            if (flagged) {
-#pragma unroll 1
-                for (int c0 = grp * 16; c0 < w; c0 += 32)
-                    if (tn * w + c0 < act_n)
-                        chain_block<VEC>(d.A32, d.R32, d.act[cur], d.Cs, n, m, atom, sh.inf[slot][ar] != 0,
-                                         sh.nan[slot][ar] != 0, sh.inf[slot] + TF_BM + c0, sh.nan[slot] + TF_BM + c0,
-                                         tn * w + c0, act_n, &sh.chain[warp - 12][0]);
-            }
-        }
-        // a wait expired: this warp's scores of the tiles it did not finish are no numbers, so that a
-        // caller who cannot see the error code sees them
-        for (; t < ntiles; t += gridDim.x) {
-            const int tm = (int)(t / tiles_n), tn = (int)(t - (long long)tm * tiles_n);
-            const int atom = tm * TF_BM + q * 32 + lane;
-            for (int c0 = grp * 16; c0 < w; c0 += 32)
-                for (int k = tn * w + c0; k < min(act_n, tn * w + c0 + 16); ++k)
-                    if (atom < m) d.Cs[(size_t)k * m + atom] = __int_as_float(0x7fffffff);
+            if (!ok) unfinished(d, t, ntiles, tiles_n, w, act_n);
+            break;
         }
     }
     fence_before();
