@@ -2,7 +2,8 @@
 // every FP32 operand split into two TF32 parts.
 //
 //   x = hi + lo,  hi = x rounded to TF32's 11 significant bits, lo = x - hi rounded to them too:
-//   |x - hi - lo| <= 2^-23 |x|.  a r is taken as a_hi r_lo + a_lo r_hi + a_hi r_hi (the
+//   |x - hi - lo| <= 2^-23 |x| (and 2^-137, TF32's subnormals being multiples of 2^-136: rows all of whose
+//   entries are below 2^-113 lose accuracy).  a r is taken as a_hi r_lo + a_lo r_hi + a_hi r_hi (the
 //   dropped a_lo r_lo is at most 2^-22 |a r|, of either sign).
 //
 // The sums of 32 products along n are accumulated in TMEM (the small products first, then the

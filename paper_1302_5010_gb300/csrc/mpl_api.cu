@@ -307,6 +307,9 @@ void set_bounds(mpl_ctx* h, Dev& d) {
     const double tf = split ? 1.25 * (98.0 * std::ldexp(1.0, -22) + ((double)h->n / 32.0 + 2.0) * u) : 0.0;
     const double cf = std::max(c32, tf);
     d.bound_f32 = (float)(cf * 1.01);
+    // TF32's subnormals are multiples of 2^-136: an entry whose low part falls among them is off by up to
+    // 2^-137, and ||x||_1 <= sqrt(n) ||x||
+    d.bound_sub = split ? (float)(std::sqrt((double)h->n) * std::ldexp(1.0, -136)) : 0.f;
     // identity route: FP32 beta and Q entries (gamma_n each, relative to colmax ||b|| and
     // colmax^2 ||x||_1), the FP32 sum over at most smax terms, and the FP32 residual the
     // re-score reads (gamma_smax each)

@@ -114,6 +114,7 @@ struct Dev {
     float* r16t;                 // p ||bf(r)|| upper bound (mixed)
     float bound_c32;             // same for the fixed-order FP32 re-score
     float bound_f32;             // FP32 correlation GEMM (either precision)
+    float bound_sub;             // and beside it, in split TF32, bound_sub * (colmax + ||r||): entries below 2^-113
     float bound_q;               // identity route: |score - a_j^T r| <= bound_q*colmax*(||b|| + colmax*||x||_1)
     const float* Q;              // m x m Gram matrix A^T A (row k = A^T a_k), identity route only
     float* beta;                 // p x m beta = A^T b (FP32), identity route only

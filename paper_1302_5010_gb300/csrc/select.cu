@@ -875,6 +875,7 @@ __device__ __forceinline__ void select_body(const Dev& d, int cur, int no_grow, 
     // |score - a^T r| for the route that produced this iteration's scores
     float delta = route == ROUTE_Q ? d.bound_q * d.colmax * (d.bnorm[i] + d.colmax * d.xl1[i])
                                    : (route == ROUTE_GEMM_F32 ? d.bound_f32 : d.bound_c) * d.colmax * rn;
+    if (route != ROUTE_GEMM || d.precision == 0) delta += d.bound_sub * (d.colmax + (route == ROUTE_Q ? d.bnorm[i] : rn));
     if (route == ROUTE_GEMM && d.precision == 1 && d.bf_ta > 0.f) {
         // the BF16 GEMM's bound from the measured rounding of this dictionary and this
         // residual (both bounds hold; the measured one is the tighter in practice)

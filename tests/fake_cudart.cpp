@@ -136,7 +136,7 @@ int fake_last(const char* what) {
 }
 int fake_live() { return (int)live.size(); }
 int fake_train_part_null() { return train_part == nullptr; }
-// bound_c, bound_f32, bound_q, bound_c32 of the last launch of a kernel
+// bound_c, bound_f32, bound_q, bound_c32, bound_sub of the last launch of a kernel
 int fake_bounds(const char* kernel, float* out) {
     for (auto& e : devs)
         if (e.first.find(kernel) != std::string::npos) {
@@ -144,6 +144,7 @@ int fake_bounds(const char* kernel, float* out) {
             out[1] = e.second.bound_f32;
             out[2] = e.second.bound_q;
             out[3] = e.second.bound_c32;
+            out[4] = e.second.bound_sub;
             return 1;
         }
     return 0;

@@ -74,3 +74,25 @@ def test_first_sizes_of_the_split(n, m, p):
     err = (C.double() - exact).abs()
     assert bool((err <= tf * (R64.abs() @ A64.abs().T)).all())
     assert err.norm().item() <= 2.0 ** -19 * exact.norm().item()
+
+
+@pytest.mark.parametrize("sa,sr", [(1.0, 1e-34), (1.0, 1e-36), (1.0, 1e-38), (1.0, 1e-40), (1e-35, 1.0), (1e-37, 1e20),
+                                   (1e-19, 1e-18)])
+def test_small_magnitudes(sa, sr):
+    """Entries whose low part is among TF32's subnormals (multiples of 2^-136) are off by up to 2^-137, which the
+    band's bound takes beside the relative term (it fails alone at 1e-40); FP32 sums round to multiples of
+    2^-149, once per 32 columns and product of parts."""
+    import torch
+    n, m, p = 512, 300, 40
+    g = torch.Generator(device="cuda").manual_seed(17)
+    A = torch.randn(m, n, device="cuda", generator=g) * sa
+    R = torch.randn(p, n, device="cuda", generator=g) * sr
+    C = torch.full((p, m), float("nan"), device="cuda")
+    assert mpl.mpl_correlate_noalloc(A, n, m, R, p, C) == mpl.MPL_OK
+    A64, R64 = A.double(), R.double()
+    err = (C.double() - R64 @ A64.T).abs()
+    relative = (98.0 * 2.0 ** -22 + (n / 32.0 + 2.0) * 2.0 ** -24) * (R64.abs() @ A64.abs().T)
+    absolute = 2.0 ** -137 * (R64.abs().sum(1)[:, None] + A64.abs().sum(1)[None, :]) + 4 * n * 2.0 ** -149
+    assert bool((err <= relative + absolute).all()), ((err - relative) / absolute).max().item()
+    if sr == 1e-40:
+        assert bool((err > relative).any())

@@ -137,7 +137,7 @@ def test_band_of_the_kernels_that_run(lib, n, p, tf32):
     fake(lib)
     s = Handle(lib, n, 300, RHO=2)
     assert s.solve(p) == mpl.MPL_OK
-    got = (ctypes.c_float * 4)()
+    got = (ctypes.c_float * 5)()
     assert lib.fake_bounds(b"k_select", got) == 1
     s.close()
     u = 2.0 ** -24
@@ -147,6 +147,7 @@ def test_band_of_the_kernels_that_run(lib, n, p, tf32):
     want = max(chain, split) if tf32 else chain
     np.testing.assert_allclose(got[:2], [want * 1.01] * 2, rtol=1e-6)
     assert got[3] == pytest.approx(chain * 1.01, rel=1e-6)
+    assert got[4] == (np.float32(np.sqrt(n) * 2.0 ** -136) if tf32 else 0.0)
     smax = min(n, 256)
     gs = (smax + 1) * u / (1 - (smax + 1) * u)
     gb = max(gam, split) if tf32 else gam
