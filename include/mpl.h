@@ -241,13 +241,14 @@ mpl_status_t mpl_correlate(mpl_handle_t h, const float* R, int p, float* C, void
  * ordering between them) race.
  * A failure on the device: for n >= 256 and p > 8 the call runs the tensor-core
  * kernel, whose waits give up after 4 s (nothing but a fault of the device or a
- * debugger that stops it is known to make one last so long).  The call has returned MPL_OK by then; the scores of the tiles that
- * were not finished are set to NaN.  Scores of finite vectors and atoms are
- * otherwise NaN only where their FP32 sum overflows in both directions.
+ * debugger that stops it is known to make one last so long).  The call has
+ * returned MPL_OK by then; the scores of the tiles that were not finished are
+ * set to NaN.  Scores of finite vectors and atoms are otherwise NaN only where
+ * their FP32 sum overflows in both directions.
  * Accuracy there: no worse than one FP32 chain over n on the data measured
- * (Gaussian, one sign, wide ranges: 1e-8 to 4e-7 of sum_k |a_jk r_ik|), and an
- * absolute error of up to 2^-137 (||a_j||_1 + ||r_i||_1), which shows where all
- * entries of a vector are below 2^-113 (1e-34).
+ * (Gaussian, one sign, wide ranges; root mean square below 1e-6 of
+ * sum_k |a_jk r_ik|), and an absolute error of up to 2^-137 (||a_j||_1 +
+ * ||r_i||_1), which shows where all entries of a vector are below 2^-113 (1e-34).
  */
 #define MPL_NOALLOC_SCRATCH_BYTES (1u << 20)
 #define MPL_NOALLOC_MAX_SIGNALS ((int)((MPL_NOALLOC_SCRATCH_BYTES - 256u) / 4u))

@@ -169,10 +169,11 @@ __global__ void __launch_bounds__(256) k_gram_gather(Dev d) {
     for (int a = threadIdx.x; a < s; a += blockDim.x) sidx[a] = Si[a];
     __syncthreads();
     // new columns (and, by symmetry, rows) of G_SS in tiles of GT_C new atoms by GT_A positions of
-    // S.  A warp reads the rows of Q of two new atoms, four times 32 entries of each in flight: every entry
-    // is a sector of its own, but a row lies in one page, while the rows of 32 positions of S lie in as many
-    // (4096 x 65536, a Q of 17 GB, batch of 1024: 2.9 -> 2.5 ms a solve; 2048 x 32768 x 512 0.52 -> 0.41, 2048 faces 0.32 -> 0.25).  The new rows G[s0 + c][a] are written along
-    // a, then through a shared-memory tile the new columns G[a][s0 + c] along c.
+    // S.  A warp reads the rows of Q of two new atoms, four times 32 entries of each in flight: every
+    // entry is a sector of its own, but a row lies in one page, while the rows of 32 positions of S
+    // lie in as many (4096 x 65536, a Q of 17 GB, batch of 1024: 2.9 -> 2.5 ms a solve; 2048 x 32768
+    // x 512 0.52 -> 0.41, 2048 faces 0.32 -> 0.25).  The new rows G[s0 + c][a] are written along a,
+    // then through a shared-memory tile the new columns G[a][s0 + c] along c.
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;  // 256 threads: 8 warps
     for (int c0 = 0; c0 < q; c0 += GT_C) {
         for (int a0 = 0; a0 < s; a0 += GT_A) {

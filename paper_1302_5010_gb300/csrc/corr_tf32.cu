@@ -14,8 +14,9 @@
 // A persistent CTA walks output tiles of 128 atoms x w signals.  Roles (five warpgroups):
 //   warps 0-7   loaders: rows of atoms and of the active signals' residuals (gathered through the
 //               active list) are copied asynchronously, as FP32, to where their hi part goes in
-//               one of two stages (three, a stage ahead, up to 128 signals; 128-byte-swizzled tiles); each lane then splits the 16 bytes it
-//               copied, so that no thread waits for another's copies.
+//               one of two stages (three, a stage ahead, up to 128 signals; 128-byte-swizzled
+//               tiles); each lane then splits the 16 bytes it copied, so that no thread waits for
+//               another's copies.
 //   warp 8      allocates TMEM; one thread issues the 12 tcgen05.mma of a stage (kind::tf32,
 //               M = 128, N = w, K = 8) into the stage's accumulator and commits.
 //   warps 12-19 accumulate: tcgen05.ld of the finished stage's accumulator, added to registers
@@ -23,13 +24,14 @@
 // setmaxnreg moves registers from the loaders to the accumulating warps.
 //
 // What bounds it: the loaders' instructions, and with few signals the latency of their copies and
-// splits, which the third stage overlaps (2048 x 32768: 16 signals 181 -> 124 us, 64 193 -> 141, 128 198 -> 155;
-// 777 x 6001 x 99 55 -> 49 us).  A stage of a 128 x 256 tile takes 3500 cycles, of
+// splits, which the third stage overlaps (2048 x 32768: 16 signals 181 -> 124 us, 64 193 -> 141,
+// 128 198 -> 155; 777 x 6001 x 99 55 -> 50 us).  A stage of a 128 x 256 tile takes 3500 cycles, of
 // which the tensor core works 2100 and shared memory (three reads of every operand by
-// the MMAs, the copies and the split: 340 KB) at least 2650.  2044 x 32771 x 500: 480 us
-// (140 TFLOP/s), 4096 x 65536 x 1024: 3.13 ms, 1024 x 8192 x 256: 46 us (three stages); the FP32 chain on the SIMT
-// cores takes 1596 us, 12.2 ms and 162 us.  Loads staged in registers (592 us), six loader warps
-// (507 us) and more, shorter stages with the copies issued ahead (557 to 650 us) were slower.
+// the MMAs, the copies and the split: 340 KB) at least 2650.  2044 x 32771 x 500: 478 us
+// (140 TFLOP/s), 4096 x 65536 x 1024: 3.13 ms, 1024 x 8192 x 256: 48 us (three stages); the FP32
+// chain on the SIMT cores takes 1596 us, 12.2 ms and 162 us.  Loads staged in registers (592 us), six
+// loader warps (507 us) and more, shorter stages with the copies issued ahead (557 to 650 us) were
+// slower.
 // Error against FP64 (2-norm), relative to the FP32 chain's: Gaussian data 0.65 at n = 128, 0.48 at 256, 0.21
 // at 4096; data of one sign, where the tensor core's truncation does not cancel, 0.85, 0.56, 0.22; the same
 // over 24 binary orders, or one large product in eight, 1.18 at n = 128 and 0.75 at 256, 0.07 at 4096.  So
@@ -596,8 +598,9 @@ cudaError_t launch_corr_tf32(const Dev& d, int cur, int act_n_ub, cudaStream_t s
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    // The narrow kernel where its tiles run side by side (1024 x 8192 x 256: 50 -> 46 us, the solve 1.084 -> 1.052 ms); else one wide tile
-    // beats two narrow ones in turn (2048 x 32768 x 256: 245 us against 320).
+    // The narrow kernel where its tiles run side by side (1024 x 8192 x 256: 50 -> 46 us, the solve
+    // 1.084 -> 1.052 ms); else one wide tile beats two narrow ones in turn (2048 x 32768 x 256: 245 us
+    // against 320).
     const long long tiles_m = (d.m + TF_BM - 1) / TF_BM;
     const bool narrow = act_n_ub <= TF_NARROW || tiles_m * ((act_n_ub + TF_NARROW - 1) / TF_NARROW) <= sms;
     if ((d.n & 3) == 0) e = narrow ? launch_t<true, true>(d, cur, act_n_ub, sms, s) : launch_t<true, false>(d, cur, act_n_ub, sms, s);

@@ -1021,11 +1021,12 @@ mpl_status_t bmpl_solve(mpl_handle_t h, const float* B, int p, const float* lamb
             CK(cudaGraphLaunch(h->graphs[gi].exec, st));
             nl += h->graphs[gi].kernels;
         } else {
-            // Few signals left: grids and kernels for them, launched one by one, instead of the graph's
-            // for all p.  A quarter is where the kernels for fewer signals begin to differ (an FP32
-            // correlation of 2048 x 32768: 470 us for 512 signals' tiles, 155 for 128, about 40 by
-            // matrix-vector products up to 8); a launch is 2 us of the host, which is ahead.  512 such signals in
-            // FP32 10.57 -> 10.04 ms, 1024 x 8192 x 256 1.147 -> 1.095; BF16 batches the same.
+            // Few signals left: grids and kernels for them, launched one by one, instead of the
+            // graph's for all p.  A quarter is where the kernels for fewer signals begin to differ (an
+            // FP32 correlation of 2048 x 32768: 470 us for 512 signals' tiles, 155 for 128, about 40
+            // by matrix-vector products up to 8); a launch is 2 us of the host, which is ahead.  512
+            // such signals in FP32 10.57 -> 10.04 ms, 1024 x 8192 x 256 1.147 -> 1.095; BF16 batches
+            // the same.
             // (At least one: the host waits for the lists of every iteration.)
             CK(launch_iteration(h, d, t, std::max(act, 1), st, graph && !h->profile ? nullptr : &pt, &nl));
         }

@@ -114,7 +114,7 @@ struct Dev {
     float* r16t;                 // p ||bf(r)|| upper bound (mixed)
     float bound_c32;             // same for the fixed-order FP32 re-score
     float bound_f32;             // FP32 correlation GEMM (either precision)
-    float bound_sub;             // and beside it, in split TF32, bound_sub * (colmax + ||r||): entries below 2^-113
+    float bound_sub;             // and beside it, in split TF32, bound_sub * (colmax + ||r||)
     float bound_q;               // identity route: |score - a_j^T r| <= bound_q*colmax*(||b|| + colmax*||x||_1)
     const float* Q;              // m x m Gram matrix A^T A (row k = A^T a_k), identity route only
     float* beta;                 // p x m beta = A^T b (FP32), identity route only
@@ -249,8 +249,8 @@ cudaError_t build_gram_q(const float* A32, int n, int m, float* Q, int* act, Cou
 cudaError_t launch_compact(const Dev& d, int cur, int slot, cudaStream_t s, int64_t* nl);
 // The new rows and columns of each growing signal's Gram block (h of the new atoms was
 // written by the selection that appended them).
-// qmax: most atoms a signal can take this iteration (picks the tile width).
-// qmax, scap: bounds on the atoms a signal gained and on its |S|.
+// qmax, scap: bounds on the atoms a signal gains this iteration and on its |S| (they pick the tile and
+// size the grid).
 cudaError_t launch_gram(const Dev& d, int ub, int qmax, int scap, int sms, cudaStream_t s, int64_t* nl);
 // Gram growth gathered from Q (MPL_OPT_QGRAM): same outputs, bit for bit, as launch_gram.
 cudaError_t launch_gram_gather(const Dev& d, int ub, cudaStream_t s, int64_t* nl);

@@ -1375,7 +1375,7 @@ cudaError_t launch_init(const Dev& d, cudaStream_t s, int64_t* nl) {
     return cudaGetLastError();
 }
 
-// The two tiles: GRAM_L for batches that fill the chip, GRAM_S for the others.
+// The two tiles: gram_large for batches that fill the chip, gram_small for the others.
 template <int BM, int BN, int TR, int TC, int BK, int ST>
 static cudaError_t gram_launch(const Dev& d, int ub, int scap, cudaStream_t s, bool prepare) {
     constexpr size_t sm = (size_t)ST * (BM + BN) * (BK + 4) * sizeof(float);
