@@ -23,10 +23,11 @@
 // the next worst-case analysis certifies the atoms outside S (eq. 8).
 //
 // One CTA per signal (256 threads, two CTAs per SM; 512 when the shared-memory
-// layout allows only one, and for signals of FIN_WIDE_MIN_N entries or more).  Shared memory is sized by the host from its bound on
-// |S|; the FP32 factor lives in shared memory when the bound fits there at two
-// CTAs per SM, else in the signal's global workspace (its panels staged through
-// shared memory either way); the FP64 factor always uses the workspace.
+// layout allows only one, and for signals of FIN_WIDE_MIN_N entries or more).
+// Shared memory is sized by the host from the largest |S| of the launch; the FP32
+// factor lives in shared memory when that fits there at two CTAs per SM, else in
+// the signal's global workspace (its panels staged through shared memory either
+// way); the FP64 factor always uses the workspace.
 #include "mpl_internal.cuh"
 
 namespace mpl {
